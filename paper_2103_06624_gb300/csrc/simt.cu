@@ -570,78 +570,145 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
 
 // ----------------------------------------------------------------------------------------
 // FP32 SIMT GEMM  C[M,N] = A[M,K] * B[K,N] (+ bias[N]); row-major, any shape.
-// Each output is a sequential FMA chain over k (error <= gamma_K sum |a b|).
+// Each output is a sequential FMA chain over k (error <= gamma_K sum |a b|), the same chain for
+// every tile shape, so the choice of tile does not change a result.
+//
+// Bound by the FMA pipe.  A thread owns TM x 8 outputs; a K step of 4 costs it TM 16-byte loads of
+// A (its rows, K-contiguous as they lie in memory, so no transposition on the way in) and 8 of B.
+// The FMAs are issued as fma.rn.f32x2 on pairs of neighbouring columns: the pipe does as many
+// FMAs a cycle as with single ones, but the other half of the issue slots is left for the loads
+// and the copies.  Both operands come by cp.async into SG_STAGES stages, zero-filled past the edges.
 // ----------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sgemm(int M, int N, int K, const float* __restrict__ A, int lda,
-                                               const float* __restrict__ B, int ldb, float* __restrict__ C,
-                                               int ldc, const float* __restrict__ bias) {
-  constexpr int BM = 128, BN = 128, BK = 16;
-  constexpr int LPT = BM * BK / 256;   // elements of each operand a thread stages per k step
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  // thread (tx, ty): rows 4ty..4ty+3 and 64+4ty..64+4ty+3, columns 4tx.. and 64+4tx.. of the
-  // tile, so its shared-memory operands are two 16-byte loads per matrix per k
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+constexpr int SG_STAGES = 3;
 
-  float ra[LPT], rb[LPT];
-  auto load_regs = [&](int k0) {
+__device__ __forceinline__ unsigned long long f32x2_dup(float a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ void f32x2_fma(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 f32x2_split(unsigned long long c) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(c));
+  return r;
+}
+
+// Copies `bytes` (0 .. SIZE) of src, the rest of the SIZE-byte piece zero.
+template <int SIZE>
+__device__ __forceinline__ void cp_async_fill(uint32_t dst, const float* src, int bytes) {
+  if (SIZE == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// BM x BN tiles, K steps of BK, TM x 8 outputs per thread; VEC: 16-byte copies (A and B with
+// 16-byte aligned rows).
+template <int BM, int BN, int BK, int TM, bool VEC>
+__global__ void __launch_bounds__((BM / TM) * (BN / 8)) k_sgemm(int M, int N, int K, const float* __restrict__ A,
+                                                               int lda, const float* __restrict__ B, int ldb,
+                                                               float* __restrict__ C, int ldc,
+                                                               const float* __restrict__ bias) {
+  constexpr int TX = BN / 8, TY = BM / TM, NT = TX * TY;
+  constexpr int AP = BK + 4;   // A row pitch: 4 or 8 consecutive rows' 16-byte reads hit distinct banks
+  extern __shared__ __align__(16) float sg_smem[];
+  float* As = sg_smem;                               // [stage][BM][AP]
+  float* Bs = sg_smem + SG_STAGES * BM * AP;         // [stage][BK][BN]
+  const int tid = threadIdx.x;
+  const int tx = tid % TX, ty = tid / TX;
+  // one-dimensional grid (any number of row tiles), a row tile's column tiles next to each other
+  const int ntn = (N + BN - 1) / BN;
+  const int m0 = (int)(blockIdx.x / ntn) * BM, n0 = (int)(blockIdx.x % ntn) * BN;
+  const uint32_t sA = (uint32_t)__cvta_generic_to_shared(As), sB = (uint32_t)__cvta_generic_to_shared(Bs);
+  auto load = [&](int stage, int k0) {
+    constexpr int V = VEC ? 4 : 1;
+    const uint32_t as = sA + (uint32_t)(stage * BM * AP * 4), bs = sB + (uint32_t)(stage * BK * BN * 4);
 #pragma unroll
-    for (int q = 0; q < LPT; ++q) {
-      int e = tid + q * 256;
-      int m = e / BK, kk = e % BK;
-      int gm = m0 + m, gk = k0 + kk;
-      ra[q] = (gm < M && gk < K) ? A[(size_t)gm * lda + gk] : 0.f;
-      int kb = e / BN, n = e % BN;
-      int gk2 = k0 + kb, gn = n0 + n;
-      rb[q] = (gk2 < K && gn < N) ? B[(size_t)gk2 * ldb + gn] : 0.f;
+    for (int e0 = 0; e0 < BM * (BK / V); e0 += NT) {
+      const int e = e0 + tid;
+      if (BM * (BK / V) % NT == 0 || e < BM * (BK / V)) {
+        const int m = e / (BK / V), k = (e % (BK / V)) * V;
+        const int left = m0 + m < M ? K - (k0 + k) : 0;
+        cp_async_fill<4 * V>(as + (uint32_t)(m * AP + k) * 4, left > 0 ? A + (size_t)(m0 + m) * lda + k0 + k : A,
+                             min(max(left, 0), V) * 4);
+      }
+    }
+#pragma unroll
+    for (int e0 = 0; e0 < BK * (BN / V); e0 += NT) {
+      const int e = e0 + tid;
+      if (BK * (BN / V) % NT == 0 || e < BK * (BN / V)) {
+        const int k = e / (BN / V), n = (e % (BN / V)) * V;
+        const int left = k0 + k < K ? N - (n0 + n) : 0;
+        cp_async_fill<4 * V>(bs + (uint32_t)(k * BN + n) * 4, left > 0 ? B + (size_t)(k0 + k) * ldb + n0 + n : B,
+                             min(max(left, 0), V) * 4);
+      }
     }
   };
-  auto store_smem = [&](int buf) {
+  // thread (tx, ty): rows ty + TY i, columns 4 tx .. + 3 of each half of the tile
+  unsigned long long acc[TM][4];
 #pragma unroll
-    for (int q = 0; q < LPT; ++q) {
-      int e = tid + q * 256;
-      As[buf][e % BK][e / BK] = ra[q];
-      Bs[buf][e / BN][e % BN] = rb[q];
-    }
-  };
-  int nk = (K + BK - 1) / BK;
-  load_regs(0);
-  store_smem(0);
-  __syncthreads();
-  for (int t = 0; t < nk; ++t) {
-    int buf = t & 1;
-    if (t + 1 < nk) load_regs((t + 1) * BK);
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][4 * ty]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + 4 * ty]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + 4 * tx]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  const int nk = (K + BK - 1) / BK;
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    if (t + 1 < nk) store_smem(buf ^ 1);
-    __syncthreads();
+  for (int t = 0; t < SG_STAGES - 1; ++t) {
+    if (t < nk) load(t, t * BK);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
+  int st = 0, ld = SG_STAGES - 1;   // the stage read now, the stage the next load fills
+  for (int t = 0; t < nk; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
+    __syncthreads();   // stage t has landed for every thread, and stage t - 1 is no longer read
+    if (t + SG_STAGES - 1 < nk) load(ld, (t + SG_STAGES - 1) * BK);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* as = As + st * BM * AP + ty * AP;
+    const float* bs = Bs + st * BK * BN + 4 * tx;
+    if (++st == SG_STAGES) st = 0;
+    if (++ld == SG_STAGES) ld = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    int gm = m0 + (i < 4 ? 4 * ty + i : 64 + 4 * ty + i - 4);
-    if (gm >= M) continue;
+    for (int k4 = 0; k4 < BK; k4 += 4) {
+      float4 a[TM];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      int gn = n0 + (j < 4 ? 4 * tx + j : 64 + 4 * tx + j - 4);
-      if (gn < N) C[(size_t)gm * ldc + gn] = acc[i][j] + (bias ? bias[gn] : 0.f);
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(as + i * TY * AP + k4);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + (k4 + kk) * BN);
+        const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + (k4 + kk) * BN + BN / 2);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const unsigned long long av = f32x2_dup(kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w);
+          f32x2_fma(acc[i][0], av, b0.x);
+          f32x2_fma(acc[i][1], av, b0.y);
+          f32x2_fma(acc[i][2], av, b1.x);
+          f32x2_fma(acc[i][3], av, b1.y);
+        }
+      }
+    }
+  }
+  const bool out4 = ((ldc & 3) | (int)(reinterpret_cast<uintptr_t>(C) & 15)) == 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int gn = n0 + h * (BN / 2) + 4 * tx;
+    float bv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bv[j] = bias && gn + j < N ? bias[gn + j] : 0.f;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int gm = m0 + ty + TY * i;
+      if (gm >= M) continue;
+      float* c = C + (size_t)gm * ldc + gn;
+      const float2 lo = f32x2_split(acc[i][2 * h]), hi = f32x2_split(acc[i][2 * h + 1]);
+      const float o[4] = {lo.x + bv[0], lo.y + bv[1], hi.x + bv[2], hi.y + bv[3]};
+      if (out4 && gn + 3 < N) {
+        *reinterpret_cast<float4*>(c) = make_float4(o[0], o[1], o[2], o[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (gn + j < N) c[j] = o[j];
+      }
     }
   }
 }
@@ -1506,11 +1573,48 @@ void launch_relax(bool cert, const RowsCtx& c, int layer, int d, long long hoff,
   ++g_launches;
 }
 
+template <int BM, int BN, int BK, int TM>
+struct SgemmTiles {
+  static constexpr int kThreads = (BM / TM) * (BN / 8);
+  static constexpr int kSmem = SG_STAGES * (BM * (BK + 4) + BK * BN) * (int)sizeof(float);
+  static long long count(int M, int N) { return (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
+  static cudaError_t load() {
+    cudaError_t e = cudaFuncSetAttribute(k_sgemm<BM, BN, BK, TM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_sgemm<BM, BN, BK, TM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  }
+  static void launch(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
+                     const float* bias, bool vec, cudaStream_t s) {
+    const unsigned grid = (unsigned)count(M, N);
+    if (vec) k_sgemm<BM, BN, BK, TM, true><<<grid, kThreads, kSmem, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias);
+    else k_sgemm<BM, BN, BK, TM, false><<<grid, kThreads, kSmem, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias);
+    ++g_launches;
+  }
+};
+using SgemmLarge = SgemmTiles<64, 128, 32, 8>;   // 128 threads
+using SgemmSmall = SgemmTiles<32, 64, 32, 4>;    //  64 threads
+
+int sgemm_load() {
+  for (cudaError_t e : {SgemmLarge::load(), SgemmSmall::load()})
+    if (e != cudaSuccess) return fail(BCROWN_ERR_CUDA, std::string("FP32 GEMM: smem attribute: ") + cudaGetErrorString(e));
+  return BCROWN_OK;
+}
+
+// The large tile from about 1.5 tiles an SM (152 SMs) on, the small one below, where the large
+// one would leave SMs idle and a block's own K loop is the time.  Measured (us, large / small):
+// 576 x 256 x 256 17 / 12, 1024 x 512 x 512 31 / 21, 2997 x 512 x 512 53 / 45, 4608 x 256 x 256
+// 18.6 / 18.5 (144 tiles), 4608 x 784 x 256 51 / 51 (504), 9216 x 784 x 256 86 / 90, 2997 x 4096
+// x 512 236 / 271 (53 TFLOP/s, 68 % of the FFMA peak), 576 x 8192 x 512 98 / 113.  One 128 x 128
+// tile shape with operands staged through registers took 42 us at 4608 x 256 x 256, 50 at 9216 x
+// 256 x 256 and 121 at 1024 x 4096 x 512 (now 98).
+constexpr long long SG_LARGE_TILES = 240;
+
 void launch_sgemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                   const float* bias, cudaStream_t s) {
   if (M <= 0 || N <= 0) return;
-  dim3 grid((N + 127) / 128, (M + 127) / 128);
-  { k_sgemm<<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias); ++g_launches; }
+  const bool vec = (((lda | ldb) & 3) | (int)((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15)) == 0;
+  if (SgemmLarge::count(M, N) >= SG_LARGE_TILES) SgemmLarge::launch(M, N, K, A, lda, B, ldb, C, ldc, bias, vec, s);
+  else SgemmSmall::launch(M, N, K, A, lda, B, ldb, C, ldc, bias, vec, s);
 }
 
 void launch_conv_bwd(int R, const LayerGeom& g, const float* Lam, const float* W, float* Ain, cudaStream_t s) {

@@ -16,6 +16,7 @@ void launch_relax(bool cert, const RowsCtx& c, int layer, int d, long long hoff,
                   double* cd, double* E, const float* wm, double gamma, cudaStream_t s);
 void launch_sgemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                   const float* bias, cudaStream_t s);
+int sgemm_load();   // shared-memory sizes of its kernels (at bcrown_load_net)
 void launch_conv_bwd(int R, const LayerGeom& g, const float* Lam, const float* W, float* Ain, cudaStream_t s);
 void launch_conv_fwd(int R, const LayerGeom& g, const float* h, const float* W, const float* bias, float* Z,
                      cudaStream_t s);
