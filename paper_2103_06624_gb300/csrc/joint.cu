@@ -63,6 +63,7 @@ struct View {
   uint8_t* from_pass;      // [B][H] bit 0: l from its target pass, bit 1: u from its target pass
   const int8_t* ssign;     // [B][H] split sign of the neuron in the subdomain (0: not split)
   const int8_t* sslot;     // [B][H] its position in the split list
+  int4* ent;               // [B][H] how a row relaxes the neuron (make_ent), final once its bounds are
   const float* x_lo;       // [P][d0]
   const float* x_hi;
   int* status;
@@ -120,40 +121,27 @@ __device__ __forceinline__ RowRef row_ref(const View& v, const Pass& q, int r) {
   return o;
 }
 
-// Relaxation of neuron n (Lemma 2.1 / Eq. definition_D) in a subdomain: D, lambda, and which
-// case applies (1: alpha slope, 2: upper chord, 0 otherwise).
-struct Rel {
-  float D, lam;
-  int kind;
-  int s, t;
-};
-
-__device__ __forceinline__ Rel relax_of(const View& v, int b, int n, float a, float alpha_val) {
-  Rel o{0.f, 0.f, 0, 0, -1};
-  const size_t bn = (size_t)b * v.H + n;
-  o.s = v.ssign[bn];
-  o.t = v.sslot[bn];
-  if (o.s == -1) {
-    o.D = 1.f;
-    return o;
-  }
-  if (o.s == 1) return o;
-  const float lo = v.lsub[bn], hi = v.usub[bn];
-  if (lo >= 0.f) {
-    o.D = 1.f;
-  } else if (hi <= 0.f) {
-    o.D = 0.f;
-  } else if (a >= 0.f) {
-    o.D = fminf(fmaxf(alpha_val, 0.f), 1.f);
-    o.kind = 1;
-  } else {
+// Relaxation of a neuron (Lemma 2.1 / Eq. definition_D) in a subdomain, worked out once per neuron
+// instead of once per row and neuron, in 16 bytes that a row reads at once: {slope, intercept of the
+// upper chord; the root rank (-1: stable at the root); kind | split sign << 2 | list position << 4},
+// kind 0: D = 0, 1: D = 1, 2: unstable, with sign 0 none, 1: S = +1, 2: S = -1.
+__device__ __forceinline__ int4 make_ent(float lo, float hi, int rk, int s, int t) {
+  int kind = 2;
+  float sl = 0.f, ic = 0.f;
+  if (s != 0) kind = s == -1 ? 1 : 0;
+  else if (lo >= 0.f) kind = 1;
+  else if (hi <= 0.f) kind = 0;
+  else {
     const float den = hi - lo;
-    o.D = hi / den;
-    o.lam = -hi * lo / den;
-    o.kind = 2;
+    sl = hi / den;
+    ic = -hi * lo / den;
   }
-  return o;
+  return make_int4(__float_as_int(sl), __float_as_int(ic), rk,
+                   kind | (s == 1 ? 1 : s == -1 ? 2 : 0) << 2 | (t & 255) << 4);
 }
+__device__ __forceinline__ int ent_kind(const int4& e) { return e.w & 3; }
+__device__ __forceinline__ int ent_sign(const int4& e) { return ((e.w >> 2) & 1) - ((e.w >> 3) & 1); }
+__device__ __forceinline__ int ent_slot(const int4& e) { return e.w >> 4; }
 
 __device__ __forceinline__ float warp_sum(float x) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -246,6 +234,17 @@ __global__ void k_splitmap(View v, const uint8_t* split_layer, const uint32_t* s
   }
 }
 
+// the entries of layer 1, whose bounds are the root's (k_update makes the later layers')
+__global__ void k_ent(View v, int d1) {
+  const int b = blockIdx.y;
+  int p = v.prop_of[b];
+  if (p < 0 || p >= v.P) p = 0;
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= d1) return;
+  const size_t bn = (size_t)b * v.H + n;
+  v.ent[bn] = make_ent(v.lsub[bn], v.usub[bn], v.rank[(size_t)p * v.H + n], v.ssign[bn], v.sslot[bn]);
+}
+
 // alpha' at the root's adaptive rule (1 where u >= -l, else 0) for every (b, T, dir) block
 __global__ void k_init_alpha_p(View v, Hoff hoff, float* alpha_p, int64_t n_alpha_p) {
   const int b = blockIdx.y;
@@ -293,26 +292,35 @@ __global__ void __launch_bounds__(32 * RW) k_relax(View v, Pass q, int R, int d,
   if (r >= R) return;
   const RowRef rr = row_ref(v, q, r);
   float acc = 0.f;
+  const int4* ent = v.ent + (size_t)rr.b * v.H + hoff;
+  const float* Ar = A + (size_t)r * d;
+  float* Lr = Lam + (size_t)r * d;
+#pragma unroll 4
   for (int j = lane; j < d; j += 32) {
-    const int n = (int)(hoff + j);
-    const float a = A[(size_t)r * d + j];
-    const int rk = v.rank[(size_t)rr.p * v.H + n];
-    float al = 0.f;
-    if (rk >= 0 && a >= 0.f) {
-      if (rk < rr.alim && rr.ab + rk < q.na) al = q.va[rr.ab + rk];
-      else jflag(v.status, BCROWN_ERR_ARG);
+    const float a = Ar[j];
+    const int4 e = ent[j];
+    const int kind = ent_kind(e), rk = e.z;
+    float D = kind == 1 ? 1.f : 0.f, lam = 0.f;
+    const bool rin = rk >= 0 && rk < rr.alim && rr.ab + rk < q.na;
+    if (a >= 0.f && !rin && (rk >= 0 || kind == 2)) jflag(v.status, BCROWN_ERR_ARG);
+    if (kind == 2) {
+      if (a >= 0.f) {
+        if (rin) D = fminf(fmaxf(q.va[rr.ab + rk], 0.f), 1.f);
+      } else {
+        D = __int_as_float(e.x);
+        lam = __int_as_float(e.y);
+      }
     }
-    const Rel re = relax_of(v, rr.b, n, a, al);
-    if (re.kind == 1 && rk < 0) jflag(v.status, BCROWN_ERR_ARG);   // unstable in a subdomain only: impossible
     float bs = 0.f;
-    if (re.s != 0) {
-      const long long bi = rr.bb + re.t;
-      if (re.t >= 0 && bi < q.nb) bs = fmaxf(q.vb[bi], 0.f) * (float)re.s;
+    const int sg = ent_sign(e);
+    if (sg != 0) {
+      const long long bi = rr.bb + ent_slot(e);
+      if (ent_slot(e) < BCROWN_MAX_SPLITS && bi < q.nb) bs = fmaxf(q.vb[bi], 0.f) * (float)sg;
       else jflag(v.status, BCROWN_ERR_ARG);
     }
-    const float L = fmaf(a, re.D, bs);
-    Lam[(size_t)r * d + j] = L;
-    acc = fmaf(L, bias[j], fmaf(a, re.lam, acc));
+    const float L = fmaf(a, D, bs);
+    Lr[j] = L;
+    acc = fmaf(L, bias[j], fmaf(a, lam, acc));
   }
   acc = warp_sum(acc);
   if (lane == 0) cf[r] += acc;
@@ -327,6 +335,7 @@ __global__ void __launch_bounds__(32 * RW) k_conc(View v, Pass q, int R, const f
   const float* xl = v.x_lo + (size_t)rr.p * v.d0;
   const float* xh = v.x_hi + (size_t)rr.p * v.d0;
   float s = 0.f;
+#pragma unroll 4
   for (int m = lane; m < v.d0; m += 32) {
     const float a = A0[(size_t)r * v.d0 + m];
     s += fminf(a * xl[m], a * xh[m]);
@@ -368,96 +377,143 @@ __global__ void k_update(View v, Pass q, long long hoffT, const float* __restric
   v.lsub[bn] = lo;
   v.usub[bn] = hi;
   v.from_pass[bn] = f;
+  v.ent[bn] = make_ent(lo, hi, v.rank[(size_t)p * v.H + n], v.ssign[bn], v.sslot[bn]);
 }
 
-// x*: the box corner minimising A^(0) x
-__global__ void k_xstar(View v, Pass q, int R, const float* __restrict__ A0, float* __restrict__ h0) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= (long long)R * v.d0) return;
-  const int r = (int)(id / v.d0), m = (int)(id - (long long)r * v.d0);
-  const RowRef rr = row_ref(v, q, r);
-  h0[id] = A0[id] >= 0.f ? v.x_lo[(size_t)rr.p * v.d0 + m] : v.x_hi[(size_t)rr.p * v.d0 + m];
+// x*: the box corner minimising A^(0) x (one warp per row)
+__global__ void __launch_bounds__(32 * RW) k_xstar(View v, Pass q, int R, const float* __restrict__ A0,
+                                                   float* __restrict__ h0) {
+  const int r = blockIdx.x * RW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= R) return;
+  int p = v.prop_of[q.b0 + r / q.rpb];
+  if (p < 0 || p >= v.P) p = 0;   // flagged by the passes before
+  const float* xl = v.x_lo + (size_t)p * v.d0;
+  const float* xh = v.x_hi + (size_t)p * v.d0;
+#pragma unroll 4
+  for (int m = lane; m < v.d0; m += 32)
+    h0[(size_t)r * v.d0 + m] = A0[(size_t)r * v.d0 + m] >= 0.f ? xl[m] : xh[m];
 }
 
 // Adjoint of layer m along the primal path (zhat = Z, bias added by the GEMM): h = D zhat +
-// lambda for every row, and the gradients.  One thread per (subdomain, neuron), looping over
-// the subdomain's rows in order.  Spec rows write dalpha / dbeta per row; target rows (weighted
-// by dg/dl or -dg/du of their neuron) sum into the subdomain's dalpha' / dbeta'.  Both add
-// their chord terms to dg/dl, dg/du of the neuron.
-__global__ void __launch_bounds__(256) k_adj(View v, Pass q, int d, long long hoff, long long hoffT,
-                                             const float* __restrict__ Z, const float* __restrict__ A,
-                                             float* __restrict__ Hout, float* __restrict__ ga, float* __restrict__ gb,
-                                             float* __restrict__ gl, float* __restrict__ gu) {
-  const int bl = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= d) return;
-  const int b = q.b0 + bl;
+// lambda for every row, and the gradients.  Spec rows write dalpha / dbeta per row; target rows
+// (weighted by dg/dl or -dg/du of their neuron) sum into the subdomain's dalpha' / dbeta'.  Both
+// add their chord terms to dg/dl, dg/du of the neuron.
+//
+// One block per (subdomain, 32 neurons): a lane owns a neuron, so every row's Z, A and h are one
+// contiguous access per warp, and the warps take the subdomain's rows in turn (row w, w + ADJ_W, ..),
+// each summing its own in order; the warps' sums are added in warp order.  Bound by HBM (12 bytes a
+// row and neuron).  One thread per neuron looping over all rows left 16 blocks on the chip at 16
+// subdomains of a 256-wide layer and took 366 us for its 8192 rows.
+constexpr int ADJ_W = 16;
+__global__ void __launch_bounds__(32 * ADJ_W) k_adj(View v, Pass q, int d, long long hoff, long long hoffT,
+                                                    const float* __restrict__ Z, const float* __restrict__ A,
+                                                    float* __restrict__ Hout, float* __restrict__ ga,
+                                                    float* __restrict__ gb, float* __restrict__ gl,
+                                                    float* __restrict__ gu) {
+  __shared__ float sums[6][ADJ_W][32];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int bl = blockIdx.y, b = q.b0 + bl;
+  const int j = blockIdx.x * 32 + lane;
+  const bool jin = j < d;
   int p = v.prop_of[b];
-  if (p < 0 || p >= v.P) p = 0;
-  const int n = (int)(hoff + j);
+  if (p < 0 || p >= v.P) {
+    jflag(v.status, BCROWN_ERR_ARG);
+    p = 0;
+  }
+  const int cnt = v.split_cnt[b];
+  const int n = (int)hoff + (jin ? j : 0);
   const size_t bn = (size_t)b * v.H + n;
-  const int rk = v.rank[(size_t)p * v.H + n];
-  float sa[2] = {0.f, 0.f}, sb[2] = {0.f, 0.f}, sl = 0.f, su = 0.f;
+  const int4 e = v.ent[bn];
+  const int kind = jin ? ent_kind(e) : 0, rk = jin ? e.z : -1, sg = jin ? ent_sign(e) : 0, slot = ent_slot(e);
+  const float sl_ = __int_as_float(e.x), ic_ = __int_as_float(e.y);
   const float lo = v.lsub[bn], hi = v.usub[bn];
-  for (int rr_ = 0; rr_ < q.rpb; ++rr_) {
-    const int r = bl * q.rpb + rr_;
-    const RowRef rr = row_ref(v, q, r);
-    float w = 1.f;
+  // d/dl and d/du of a (zhat s + t), s = u / (u - l), t = -u l / (u - l)
+  float dsdl = 0.f, dsdu = 0.f, dtdl = 0.f, dtdu = 0.f;
+  if (kind == 2) {
+    const float den = hi - lo, i2 = 1.f / (den * den);
+    dsdl = hi * i2, dsdu = -lo * i2, dtdl = -hi * hi * i2, dtdu = lo * lo * i2;
+  }
+  // target passes: alpha' of the two directions; spec rows read their own
+  const int alim = q.target ? v.first[(size_t)p * v.L + q.T] : v.U[p];
+  const long long a0 = q.target ? v.ap_off[b] + v.jblk[(size_t)p * v.L + q.T] : v.alpha_off[b];
+  const long long b0 = q.target ? 2LL * (v.L - 2) * v.split_off[b] + 2LL * (q.T - 2) * cnt
+                                : (long long)v.split_off[b] * v.K;
+  float alt[2] = {0.f, 0.f};
+  if (q.target && rk >= 0 && rk < alim)
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir)
+      if (a0 + (long long)dir * alim + rk < q.na) alt[dir] = q.va[a0 + (long long)dir * alim + rk];
+  float sa[2] = {0.f, 0.f}, sb[2] = {0.f, 0.f}, sl = 0.f, su = 0.f;
+  const size_t base = (size_t)bl * q.rpb * d + (jin ? j : 0);
+#pragma unroll 4
+  for (int rr = wp; rr < q.rpb; rr += ADJ_W) {
+    const float z = Z[base + (size_t)rr * d];
+    const float a = A[base + (size_t)rr * d];
+    float w = 1.f, al;
+    const int dir = q.target && rr >= q.dT ? 1 : 0;
+    const long long ai = a0 + (long long)rr * alim + rk;   // spec rows
     if (q.target) {
-      const size_t bt = (size_t)b * v.H + hoffT + rr.j;
+      const size_t bt = (size_t)b * v.H + hoffT + (rr - dir * q.dT);
       const uint8_t f = v.from_pass[bt];
-      w = rr.dir == 0 ? ((f & 1) ? gl[bt] : 0.f) : ((f & 2) ? -gu[bt] : 0.f);
+      w = dir == 0 ? ((f & 1) ? gl[bt] : 0.f) : ((f & 2) ? -gu[bt] : 0.f);
+      al = dir == 0 ? alt[0] : alt[1];
+    } else {
+      al = (rk >= 0 && a >= 0.f && rk < alim && ai < q.na) ? q.va[ai] : 0.f;
     }
-    const float z = Z[(size_t)r * d + j];
-    const float a = A[(size_t)r * d + j];
-    float al = 0.f;
-    if (rk >= 0 && a >= 0.f && rk < rr.alim && rr.ab + rk < q.na) al = q.va[rr.ab + rk];
-    const Rel re = relax_of(v, b, n, a, al);
-    Hout[(size_t)r * d + j] = fmaf(re.D, z, re.lam);
-    const float gal = re.kind == 1 ? a * z : 0.f;
-    if (!q.target && rk >= 0) {
-      const long long ai = rr.ab + rk;
-      if (rk < rr.alim && ai < q.na) ga[ai] = gal;
-      else jflag(v.status, BCROWN_ERR_ARG);
-    }
-    if (re.s != 0) {
-      if (q.target) {
-        sb[rr.dir] += w * (float)re.s * z;
+    float D = kind == 1 ? 1.f : 0.f, lam = 0.f, gal = 0.f;
+    if (kind == 2) {
+      if (a >= 0.f) {
+        D = fminf(fmaxf(al, 0.f), 1.f);
+        gal = a * z;
       } else {
-        const long long bi = rr.bb + re.t;
-        if (re.t >= 0 && bi < q.nb) gb[bi] = (float)re.s * z;
-        else jflag(v.status, BCROWN_ERR_ARG);
+        D = sl_;
+        lam = ic_;
+        sl += w * a * fmaf(z, dsdl, dtdl);
+        su += w * a * fmaf(z, dsdu, dtdu);
       }
     }
-    if (q.target) sa[rr.dir] += w * gal;
-    if (re.kind == 2) {
-      // d/dl and d/du of a (zhat s + t), s = u / (u - l), t = -u l / (u - l)
-      const float den = hi - lo, i2 = 1.f / (den * den);
-      const float dsdl = hi * i2, dsdu = -lo * i2, dtdl = -hi * hi * i2, dtdu = lo * lo * i2;
-      sl += w * a * fmaf(z, dsdl, dtdl);
-      su += w * a * fmaf(z, dsdu, dtdu);
+    if (jin) Hout[base + (size_t)rr * d] = fmaf(D, z, lam);
+    if (q.target) {
+      if (dir == 0) {
+        sa[0] += w * gal;
+        if (sg != 0) sb[0] += w * (float)sg * z;
+      } else {
+        sa[1] += w * gal;
+        if (sg != 0) sb[1] += w * (float)sg * z;
+      }
+    } else {
+      if (rk >= 0) {
+        if (rk < alim && ai < q.na) ga[ai] = gal;
+        else jflag(v.status, BCROWN_ERR_ARG);
+      }
+      if (sg != 0) {
+        const long long bi = b0 + (long long)rr * cnt + slot;
+        if (slot < BCROWN_MAX_SPLITS && bi < q.nb) gb[bi] = (float)sg * z;
+        else jflag(v.status, BCROWN_ERR_ARG);
+      }
     }
   }
-  gl[bn] += sl;
-  gu[bn] += su;
-  if (q.target) {
+  const float mine[6] = {sl, su, sa[0], sa[1], sb[0], sb[1]};
+#pragma unroll
+  for (int i = 0; i < 6; ++i) sums[i][wp][lane] = mine[i];
+  __syncthreads();
+  // warp i adds up sum i
+  if (wp >= 6 || !jin) return;
+  float t = sums[wp][0][lane];
+#pragma unroll
+  for (int i = 1; i < ADJ_W; ++i) t += sums[wp][i][lane];
+  if (wp == 0) gl[bn] += t;
+  else if (wp == 1) gu[bn] += t;
+  else if (q.target && wp < 4) {
     if (rk >= 0) {
-      const int f = v.first[(size_t)p * v.L + q.T];
-      for (int dir = 0; dir < 2; ++dir) {
-        const long long ai = v.ap_off[b] + v.jblk[(size_t)p * v.L + q.T] + (long long)dir * f + rk;
-        if (rk < f && ai < q.na) ga[ai] = sa[dir];
-        else jflag(v.status, BCROWN_ERR_ARG);
-      }
+      const long long ai = a0 + (long long)(wp - 2) * alim + rk;
+      if (rk < alim && ai < q.na) ga[ai] = t;
+      else jflag(v.status, BCROWN_ERR_ARG);
     }
-    const int s = v.ssign[bn], t = v.sslot[bn];
-    if (s != 0) {
-      const int cnt = v.split_cnt[b];
-      for (int dir = 0; dir < 2; ++dir) {
-        const long long bi = 2LL * (v.L - 2) * v.split_off[b] + (long long)(2 * (q.T - 2) + dir) * cnt + t;
-        if (t >= 0 && bi < q.nb) gb[bi] = sb[dir];
-        else jflag(v.status, BCROWN_ERR_ARG);
-      }
-    }
+  } else if (q.target && sg != 0) {
+    const long long bi = b0 + (long long)(wp - 4) * cnt + slot;
+    if (slot < BCROWN_MAX_SPLITS && bi < q.nb) gb[bi] = t;
+    else jflag(v.status, BCROWN_ERR_ARG);
   }
 }
 
@@ -521,6 +577,9 @@ struct Work {
   // chunk buffers
   int Bc, rows_max;
   std::vector<float*> A;     // [L]: A^(m) [rows][d_m]
+  // with a gradient, where the memory allows it: A^(m) of every target pass, kept for its adjoint
+  // (empty: the pass is recomputed there)
+  std::vector<std::vector<float*>> At;   // [T][m]
   float *Lam, *Z, *Hb, *cf, *tlb;
   float *gl, *gu;
 };
@@ -546,19 +605,32 @@ static int setup(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* 
   for (int m = 0; m < L; ++m) per_row += (size_t)net->d[m];
   per_row += (size_t)net->max_hidden + 2 * (size_t)net->max_width + 2;
   const size_t budget = size_t(4) << 30;
-  w.Bc = (int)std::max<long long>(1, std::min<long long>(B, (long long)(budget / ((size_t)rpb * per_row * 4))));
+  const long long Bc0 = std::max<long long>(1, std::min<long long>(B, (long long)(budget / ((size_t)rpb * per_row * 4))));
+  w.Bc = (int)Bc0;
+  // Keeping the target passes' A^(m) saves a third of the gradient's contractions and takes more
+  // memory a subdomain, so fewer subdomains fit a chunk: kept while a chunk still holds 4 subdomains
+  // (or the batch), whose rows fill the chip.  784-256x6-10, 16 subdomains: 15.9 MB a subdomain.
+  size_t kept = 0;
+  for (int T = 2; T <= L - 1; ++T)
+    for (int m = 0; m < T; ++m) kept += (size_t)2 * net->d[T] * net->d[m] * 4;
+  const long long Bk = (long long)(budget / ((size_t)rpb * per_row * 4 + kept));
+  const bool keep = grad && L >= 3 && Bk >= std::min<long long>(B, 4);
+  if (keep) w.Bc = (int)std::min<long long>(Bc0, Bk);
   w.rows_max = w.Bc * rpb;
   const size_t PH = (size_t)P * H, BH = (size_t)B * H;
   size_t bytes = 0;
   auto add = [&](size_t n) { bytes += align_up(n); };
   add(PH), add(PH * 4), add(PH * 4), add(PH * 4), add((size_t)P * 4);           // tables
   add((size_t)P * L * 4), add((size_t)P * L * 8), add((size_t)(B + 1) * 8);      // layout
-  add(BH * 4), add(BH * 4), add(BH), add(BH), add(BH);                             // state
+  add(BH * 4), add(BH * 4), add(BH), add(BH), add(BH), add(BH * 16);               // state
   if (grad) add(BH * 4), add(BH * 4);
   for (int m = 0; m < L; ++m) add((size_t)w.rows_max * net->d[m] * 4);
   add((size_t)w.rows_max * net->max_hidden * 4);
   add((size_t)w.rows_max * net->max_width * 4), add((size_t)w.rows_max * net->max_width * 4);
   add((size_t)w.rows_max * 4), add((size_t)w.rows_max * 4);
+  if (keep)
+    for (int T = 2; T <= L - 1; ++T)
+      for (int m = 0; m < T; ++m) add((size_t)w.Bc * 2 * net->d[T] * net->d[m] * 4);
   int st = 0;
   void* base = ws_get(net, bytes, &st);
   if (!base) return st;
@@ -585,6 +657,7 @@ static int setup(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* 
   int8_t* ssign = ar.take<int8_t>(BH);
   int8_t* sslot = ar.take<int8_t>(BH);
   v.ssign = ssign, v.sslot = sslot;
+  v.ent = ar.take<int4>(BH);
   v.x_lo = dom->x_lo, v.x_hi = dom->x_hi;
   v.status = net->status;
   for (int i = 0; i < MAXL; ++i) w.hoff.v[i] = i < L ? net->hoff[i] : 0;
@@ -601,12 +674,20 @@ static int setup(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* 
   w.Hb = ar.take<float>((size_t)w.rows_max * net->max_width);
   w.cf = ar.take<float>(w.rows_max);
   w.tlb = ar.take<float>(w.rows_max);
+  w.At.assign(L, std::vector<float*>());
+  if (keep)
+    for (int T = 2; T <= L - 1; ++T)
+      for (int m = 0; m < T; ++m) w.At[T].push_back(ar.take<float>((size_t)w.Bc * 2 * net->d[T] * net->d[m]));
   if (ar.off > net->ws.size) return fail(BCROWN_ERR_OOM, "joint: workspace plan overflow");
   k_layout<<<(P + 127) / 128, 128, 0, s>>>(P, H, L, w.hoff, rank, first, jblk);
   k_ap_off<<<1, 1, 0, s>>>(B, L, bt->prop_of, first, jblk, P, ap_off, net->status);
   k_init<<<dim3((H + 255) / 256, B), 256, 0, s>>>(v);
   k_splitmap<<<(B + 127) / 128, 128, 0, s>>>(v, bt->split_layer, bt->split_idx, bt->split_sign, w.hoff);
   g_launches += 4;
+  if (L >= 2) {
+    k_ent<<<dim3((net->d[1] + 127) / 128, B), 128, 0, s>>>(v, net->d[1]);
+    ++g_launches;
+  }
   if (grad) {
     BC_CUDA(cudaMemsetAsync(w.gl, 0, BH * 4, s));
     BC_CUDA(cudaMemsetAsync(w.gu, 0, BH * 4, s));
@@ -616,43 +697,44 @@ static int setup(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* 
 }
 
 // The backward recursion of one pass over the chunk (top, relaxation and contraction down to
-// the input, concretisation into out): A^(m) of every layer stays in w.A for the adjoint.
-static int backward(bcrown_net* net, Work& w, const Pass& q, float* out, cudaStream_t s) {
+// the input, concretisation into out): A^(m) of every layer stays in A for the adjoint.
+static int backward(bcrown_net* net, Work& w, const Pass& q, const std::vector<float*>& A, float* out,
+                    cudaStream_t s) {
   const int R = q.Bc * q.rpb;
   const int T = q.T;
   const LayerDev& top = net->ly[T - 1];
   if (q.target)
-    k_top<<<R, 128, 0, s>>>(w.v, q, net->d[T - 1], top.W, top.b, w.A[T - 1], w.cf);
+    k_top<<<R, 128, 0, s>>>(w.v, q, net->d[T - 1], top.W, top.b, A[T - 1], w.cf);
   else
-    k_top<<<R, 128, 0, s>>>(w.v, q, net->d[T - 1], net->Wbar, net->bbar, w.A[T - 1], w.cf);
+    k_top<<<R, 128, 0, s>>>(w.v, q, net->d[T - 1], net->Wbar, net->bbar, A[T - 1], w.cf);
   ++g_launches;
   for (int m = T - 1; m >= 1; --m) {
     const LayerDev& l = net->ly[m - 1];
-    k_relax<<<(R + RW - 1) / RW, 32 * RW, 0, s>>>(w.v, q, R, net->d[m], net->hoff[m - 1], l.b, w.A[m], w.Lam,
+    k_relax<<<(R + RW - 1) / RW, 32 * RW, 0, s>>>(w.v, q, R, net->d[m], net->hoff[m - 1], l.b, A[m], w.Lam,
                                                   w.cf);
     ++g_launches;
     // A^(m-1) = Lambda^(m) W^(m)
-    launch_sgemm(R, l.d_in, l.d_out, w.Lam, l.d_out, l.W, l.d_in, w.A[m - 1], l.d_in, nullptr, s);
+    launch_sgemm(R, l.d_in, l.d_out, w.Lam, l.d_out, l.W, l.d_in, A[m - 1], l.d_in, nullptr, s);
   }
-  k_conc<<<(R + RW - 1) / RW, 32 * RW, 0, s>>>(w.v, q, R, w.A[0], w.cf, out);
+  k_conc<<<(R + RW - 1) / RW, 32 * RW, 0, s>>>(w.v, q, R, A[0], w.cf, out);
   ++g_launches;
   BC_CUDA(cudaGetLastError());
   return BCROWN_OK;
 }
 
-// The adjoint of the pass just run by backward(): h^(0) = x*, then for m = 1..T-1
+// The adjoint of a pass of backward() from the A^(m) it left: h^(0) = x*, then for m = 1..T-1
 // zhat = W^(m) h + b^(m) and the layer's gradients.
-static int adjoint(bcrown_net* net, Work& w, const Pass& q, float* ga, float* gb, cudaStream_t s) {
+static int adjoint(bcrown_net* net, Work& w, const Pass& q, const std::vector<float*>& A, float* ga, float* gb,
+                   cudaStream_t s) {
   const int R = q.Bc * q.rpb;
-  const int d0 = net->d[0];
-  k_xstar<<<grid1d((long long)R * d0, 256), 256, 0, s>>>(w.v, q, R, w.A[0], w.Hb);
+  k_xstar<<<(R + RW - 1) / RW, 32 * RW, 0, s>>>(w.v, q, R, A[0], w.Hb);
   ++g_launches;
   const long long hoffT = q.target ? net->hoff[q.T - 1] : 0;
   for (int m = 1; m <= q.T - 1; ++m) {
     const LayerDev& l = net->ly[m - 1];
     launch_sgemm(R, l.d_out, l.d_in, w.Hb, l.d_in, l.Wt, l.d_out, w.Z, l.d_out, l.b, s);
-    k_adj<<<dim3((l.d_out + 255) / 256, q.Bc), 256, 0, s>>>(w.v, q, l.d_out, net->hoff[m - 1], hoffT, w.Z,
-                                                            w.A[m], w.Hb, ga, gb, w.gl, w.gu);
+    k_adj<<<dim3((l.d_out + 31) / 32, q.Bc), 32 * ADJ_W, 0, s>>>(w.v, q, l.d_out, net->hoff[m - 1], hoffT, w.Z,
+                                                            A[m], w.Hb, ga, gb, w.gl, w.gu);
     ++g_launches;
   }
   BC_CUDA(cudaGetLastError());
@@ -690,18 +772,19 @@ static int run(bcrown_net* net, Work& w, const bcrown_batch* bt, const float* al
     const int Bc = std::min(w.Bc, B - b0);
     for (int T = 2; T <= L - 1; ++T) {
       Pass q = make_pass(net, true, T, b0, Bc, alpha_p, n_alpha_p, beta_p, n_beta_p);
-      BC_CHECK(backward(net, w, q, w.tlb, s));
+      BC_CHECK(backward(net, w, q, w.At[T].empty() ? w.A : w.At[T], w.tlb, s));
       k_update<<<dim3((net->d[T] + 127) / 128, Bc), 128, 0, s>>>(w.v, q, net->hoff[T - 1], w.tlb);
       ++g_launches;
     }
     Pass f = make_pass(net, false, L, b0, Bc, alpha, bt->n_alpha, beta, bt->n_beta);
-    BC_CHECK(backward(net, w, f, lb + (size_t)b0 * K, s));
+    BC_CHECK(backward(net, w, f, w.A, lb + (size_t)b0 * K, s));
     if (!grad) continue;
-    BC_CHECK(adjoint(net, w, f, dalpha, dbeta, s));
+    BC_CHECK(adjoint(net, w, f, w.A, dalpha, dbeta, s));
     for (int T = L - 1; T >= 2; --T) {
       Pass q = make_pass(net, true, T, b0, Bc, alpha_p, n_alpha_p, beta_p, n_beta_p);
-      BC_CHECK(backward(net, w, q, w.tlb, s));   // recomputed: A^(m) of this pass for its adjoint
-      BC_CHECK(adjoint(net, w, q, dalpha_p, dbeta_p, s));
+      const std::vector<float*>& A = w.At[T].empty() ? w.A : w.At[T];
+      if (w.At[T].empty()) BC_CHECK(backward(net, w, q, A, w.tlb, s));   // A^(m) of this pass again
+      BC_CHECK(adjoint(net, w, q, A, dalpha_p, dbeta_p, s));
     }
   }
   BC_CUDA(cudaGetLastError());
