@@ -504,43 +504,66 @@ extern "C" int bcrown_root_bounds(bcrown_net* net, int n_props, const float* x_l
   cudaStream_t s = (cudaStream_t)stream;
   const bool cert = precision == BCROWN_CERTIFY;
   const int L = net->L;
-  int maxrows = 2 * std::max(net->max_hidden, 1);
+  // rows of the largest target layer beyond the first, all properties
+  long long maxrows = 1;
+  for (int T = 2; T <= L - 1; ++T) maxrows = std::max(maxrows, 2LL * net->d[T] * n_props);
   Plan pl;
-  BC_CHECK(make_plan(net, n_props, maxrows, cert, false, 0, 0, 0, pl));
-  bcrown_domain dom{n_props, x_lo, x_hi, l, u};
-  for (int top = 1; top <= L - 1; ++top) {
-    // tables and |W| M terms of layers < top are complete once l, u of those layers are.
-    build_tables(net, &dom, pl, s);
-    if (cert) {
-      long long hprev = top >= 2 ? net->hoff[top - 2] : -1;
-      // wm of layers 1..top-1 (recomputed: cheap)
-      for (int m = 1; m < top; ++m) {
-        long long hp = m >= 2 ? net->hoff[m - 2] : -1;
-        launch_absw_m(geom_of(net->ly[m - 1]), net->ly[m - 1].W, n_props, net->H, net->hoff[m - 1], hp, u, x_lo,
-                      x_hi, net->d[0], pl.wm, s);
-      }
-      (void)hprev;
+  BC_CHECK(make_plan(net, n_props, (int)std::min<long long>(maxrows, 1 << 30), cert, false, 0, 0, 0, pl));
+  RootCtx c;
+  c.H = net->H;
+  c.d0 = net->d[0];
+  c.l = l;
+  c.u = u;
+  c.x_lo = x_lo;
+  c.x_hi = x_hi;
+  for (int T = 1; T <= L - 1; ++T) {
+    const LayerDev& top = net->ly[T - 1];
+    c.d_top = net->d[T];
+    c.top_h = std::max(top.out_h, 1);
+    c.top_w = std::max(top.out_w, 1);
+    c.hoff_top = net->hoff[T - 1];
+    if (T == 1) {
+      c.g0 = 0, c.R = 0;
+      launch_root_first(cert, c, n_props, geom_of(top), top.W, top.b, s);
+      continue;
     }
-    const int d_top = net->d[top];
-    const int rows = 2 * d_top;
-    for (int p = 0; p < n_props; ++p) {
-      for (int q0 = 0; q0 < rows; q0 += pl.Rc) {
-        int Rc = std::min(pl.Rc, rows - q0);
-        launch_root_top(q0, Rc, d_top, net->ly[top - 1].b, pl.Lam, pl.cf, pl.cd, pl.E, s);
-        contract_bwd(net, top, Rc, pl.Lam, pl.Abuf[top - 1], s);
-        for (int m = top - 1; m >= 1; --m) {
-          const LayerDev& ly = net->ly[m - 1];
-          launch_relax_root(cert, Rc, p, net->H, net->d[m], net->hoff[m - 1], l, u, pl.tb, alpha_rule, alpha_value,
-                            pl.Abuf[m], pl.Lam, ly.b, pl.cf, pl.cd, pl.E, pl.wm, gamma_n(ly.terms_bwd), s);
-          contract_bwd(net, m, Rc, pl.Lam, pl.Abuf[m - 1], s);
+    // the error terms |W| M of layer T - 1, whose bounds are complete now
+    if (cert)
+      launch_absw_m(geom_of(net->ly[T - 2]), net->ly[T - 2].W, n_props, net->H, net->hoff[T - 2],
+                    T >= 3 ? net->hoff[T - 3] : -1, u, x_lo, x_hi, net->d[0], pl.wm, s);
+    std::vector<int> n;
+    const bool patch = root_patch(net, T, n);
+    std::vector<RootMap> map(T, RootMap{0, 0, 0, 0, 0});
+    std::vector<int> d(T);
+    for (int m = T - 1, os = 1, oo = 0; m >= 0; --m) {
+      d[m] = net->d[m];
+      if (!patch) continue;
+      const LayerDev& ly = net->ly[m];   // layer m + 1: from map m to map m + 1
+      os *= ly.stride;
+      oo = oo * ly.stride + ly.pad;
+      map[m] = RootMap{n[m], ly.in_h, ly.in_w, os, oo};
+      d[m] = ly.in_c * n[m] * n[m];
+    }
+    const long long rows = 2LL * c.d_top * n_props;
+    for (long long g0 = 0; g0 < rows; g0 += pl.Rc) {
+      c.g0 = g0;
+      c.R = (int)std::min<long long>(pl.Rc, rows - g0);
+      launch_root_top(c, geom_of(top), patch, top.W, top.b, pl.Abuf[T - 1], pl.cf, pl.cd, pl.E, s);
+      for (int m = T - 1; m >= 1; --m) {
+        const LayerDev& ly = net->ly[m - 1];
+        launch_root_relax(cert, c, map[m], d[m], net->hoff[m - 1], alpha_rule, alpha_value, pl.Abuf[m], pl.Lam, ly.b,
+                          pl.cf, pl.cd, pl.E, pl.wm, gamma_n(ly.terms_bwd), s);
+        if (patch) {
+          ProfScope ps(net, BCROWN_PROF_CONTRACT, s);
+          BC_CHECK(sconv_patch(net, T, m, c.R, pl.Lam, pl.Abuf[m - 1], s));
+        } else {
+          BC_CHECK(contract_bwd(net, m, c.R, pl.Lam, pl.Abuf[m - 1], s));
         }
-        launch_concretize_root(cert, q0, Rc, p, net->d[0], d_top, net->H, net->hoff[top - 1], x_lo, x_hi, pl.Abuf[0],
-                               pl.cf, pl.cd, pl.E, l, u, s);
       }
+      launch_root_concretize(cert, c, map[0], d[0], pl.Abuf[0], pl.cf, pl.cd, pl.E, s);
     }
   }
-  build_tables(net, &dom, pl, s);
-  launch_copy_count(n_props, net->H, pl.U, unstable_count, s);
+  launch_count_unstable(n_props, net->H, l, u, unstable_count, s);
   BC_CUDA(cudaGetLastError());
   return BCROWN_OK;
 }

@@ -20,8 +20,6 @@ namespace bcrown {
 
 extern std::atomic<long long> g_launches;
 
-bool sconv_supported(const bcrown_net* net, int i);
-
 namespace {
 
 struct SconvPass {
@@ -35,6 +33,7 @@ struct SconvPass {
   long long HWo;   // output position (oa + os i) Wo + ob + os j, channel stride HWo
   const int4* tab; // [K]: {source offset c HWs + dy Ws + dx, dy, dx, 0}
   const float* B;  // [K][N] weights
+  int ky0, kx0;    // the phase's first tap (B depends on nothing else)
 };
 
 constexpr int SC_BM = 128, SC_BK = 16, SC_THREADS = 256;
@@ -215,6 +214,8 @@ int sconv_smem(int BN, int K) { return 2 * SC_BK * (SC_BM + 4) * 4 + 2 * SC_BK *
 struct LayerF32 {
   std::vector<SconvPass> bwd;   // one per stride phase with positions
   SconvPass fwd;
+  // [T]: the backward passes over the patches of layer T's root rows (root.cu)
+  std::vector<std::vector<SconvPass>> patch;
 };
 struct SconvNet {
   bool ready = false;
@@ -263,46 +264,63 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
       return fail(BCROWN_ERR_CUDA, "FP32 conv: copy of weights");
     LayerF32& P = t->ly[i];
     // backward phases: source Lambda^(i) (out_c x out_h x out_w), output the input map
+    auto backward = [&](int in_h, int in_w, int out_h, int out_w, int pad, std::vector<SconvPass>& made) -> int {
     for (int a = 0; a < s; ++a)
       for (int b = 0; b < s; ++b) {
         int ky0, nky, offy, ny, kx0, nkx, offx, nx;
-        sc_phase(a, k, s, l.pad, l.in_h, &ky0, &nky, &offy, &ny);
-        sc_phase(b, k, s, l.pad, l.in_w, &kx0, &nkx, &offx, &nx);
+        sc_phase(a, k, s, pad, in_h, &ky0, &nky, &offy, &ny);
+        sc_phase(b, k, s, pad, in_w, &kx0, &nkx, &offx, &nx);
         if (ny * nx == 0) continue;
         SconvPass q{};
         q.Pm = ny * nx;
         q.nJ = nx;
         q.N = l.in_c;
         q.K = std::max(1, l.out_c * nky * nkx);
-        q.Hs = l.out_h;
-        q.Ws = l.out_w;
-        q.HWs = (long long)l.out_h * l.out_w;
+        q.Hs = out_h;
+        q.Ws = out_w;
+        q.HWs = (long long)out_h * out_w;
         q.ms = 1;
         q.cy = offy;
         q.cx = offx;
         q.oa = a;
         q.ob = b;
         q.os = s;
-        q.Wo = l.in_w;
-        q.HWo = (long long)l.in_h * l.in_w;
+        q.Wo = in_w;
+        q.HWo = (long long)in_h * in_w;
+        q.ky0 = ky0;
+        q.kx0 = kx0;
         std::vector<int4> tab((size_t)q.K, make_int4(0, -32768, 0, 0));
-        std::vector<float> B((size_t)q.K * q.N, 0.f);
         for (int co = 0; co < l.out_c; ++co)
           for (int dy = 0; dy < nky; ++dy)
-            for (int dx = 0; dx < nkx; ++dx) {
-              const int kq = (co * nky + dy) * nkx + dx;
-              tab[kq] = make_int4((int)(co * q.HWs - dy * l.out_w - dx), -dy, -dx, 0);
-              const int ky = ky0 + s * dy, kx = kx0 + s * dx;
-              for (int ci = 0; ci < l.in_c; ++ci)
-                B[(size_t)kq * q.N + ci] = w[(((size_t)co * l.in_c + ci) * k + ky) * k + kx];
-            }
+            for (int dx = 0; dx < nkx; ++dx)
+              tab[(co * nky + dy) * nkx + dx] = make_int4((int)(co * q.HWs - dy * out_w - dx), -dy, -dx, 0);
         void *dt = nullptr, *dB = nullptr;
         BC_CHECK(sc_upload(t, tab.data(), tab.size() * sizeof(int4), &dt));
-        BC_CHECK(sc_upload(t, B.data(), B.size() * 4, &dB));
         q.tab = reinterpret_cast<const int4*>(dt);
-        q.B = reinterpret_cast<const float*>(dB);
-        P.bwd.push_back(q);
+        for (const SconvPass& o : P.bwd)   // the phase's weights, if another pass of the layer has them
+          if (o.ky0 == ky0 && o.kx0 == kx0) q.B = o.B;
+        if (!q.B) {
+          std::vector<float> B((size_t)q.K * q.N, 0.f);
+          for (int co = 0; co < l.out_c; ++co)
+            for (int dy = 0; dy < nky; ++dy)
+              for (int dx = 0; dx < nkx; ++dx) {
+                const int kq = (co * nky + dy) * nkx + dx, ky = ky0 + s * dy, kx = kx0 + s * dx;
+                for (int ci = 0; ci < l.in_c; ++ci)
+                  B[(size_t)kq * q.N + ci] = w[(((size_t)co * l.in_c + ci) * k + ky) * k + kx];
+              }
+          BC_CHECK(sc_upload(t, B.data(), B.size() * 4, &dB));
+          q.B = reinterpret_cast<const float*>(dB);
+        }
+        made.push_back(q);
       }
+      return BCROWN_OK;
+    };
+    BC_CHECK(backward(l.in_h, l.in_w, l.out_h, l.out_w, l.pad, P.bwd));
+    P.patch.assign(net->L, std::vector<SconvPass>());
+    for (int T = i + 1; T <= net->L - 1; ++T) {
+      std::vector<int> n;
+      if (root_patch(net, T, n)) BC_CHECK(backward(n[i - 1], n[i - 1], n[i], n[i], 0, P.patch[T]));
+    }
     // forward: source h^(i-1) (in_c x in_h x in_w), output the layer's map
     SconvPass f{};
     f.Pm = l.out_h * l.out_w;
@@ -400,6 +418,29 @@ int sconv_bwd(bcrown_net* net, int i, int R, const float* Lam, float* Ain, cudaS
   if (!t->ready) return fail(BCROWN_ERR_ARG, "FP32 conv: tables not built");
   const LayerDev& l = net->ly[i - 1];
   for (const SconvPass& q : t->ly[i].bwd) BC_CHECK(sc_launch(q, R, Lam, l.d_out, Ain, l.d_in, nullptr, s));
+  return BCROWN_OK;
+}
+
+bool root_patch(const bcrown_net* net, int T, std::vector<int>& n) {
+  n.assign(T + 1, 1);
+  for (int m = T; m >= 1; --m) {
+    const LayerDev& l = net->ly[m - 1];
+    if (l.kind != BCROWN_LAYER_CONV || (m < T && !sconv_supported(net, m))) return false;
+    const long long nm = (long long)(n[m] - 1) * l.stride + l.k;
+    if (nm > 32768 || nm * nm * l.in_c > (long long)l.d_in) return false;
+    n[m - 1] = (int)nm;
+  }
+  return true;
+}
+
+int sconv_patch(bcrown_net* net, int T, int i, int R, const float* Lam, float* Ain, cudaStream_t s) {
+  SconvNet* t = sc_of(net);
+  std::vector<int> n;
+  if (!t->ready || !root_patch(net, T, n)) return fail(BCROWN_ERR_ARG, "FP32 conv: no patch tables");
+  const LayerDev& l = net->ly[i - 1];
+  for (const SconvPass& q : t->ly[i].patch[T])
+    BC_CHECK(sc_launch(q, R, Lam, (long long)l.out_c * n[i] * n[i], Ain, (long long)l.in_c * n[i - 1] * n[i - 1],
+                       nullptr, s));
   return BCROWN_OK;
 }
 

@@ -1397,123 +1397,6 @@ __global__ void __launch_bounds__(128) k_split_copy(BatchView bt, int K, const i
 }
 
 // ----------------------------------------------------------------------------------------
-// Root bounds: rows (j, sign) for hidden layer `top`; the top of the recursion is
-// Lambda = +-e_j at layer `top`, c = +-b_j.
-// ----------------------------------------------------------------------------------------
-__global__ void k_root_top(int q0, int Rc, int d_top, const float* __restrict__ b_top, float* __restrict__ Lam,
-                           float* __restrict__ cf, double* __restrict__ cd, double* __restrict__ E) {
-  long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= (long long)Rc * d_top) return;
-  int rl = (int)(id / d_top);
-  int j = (int)(id - (long long)rl * d_top);
-  int q = q0 + rl;
-  int jj = q < d_top ? q : q - d_top;
-  float sg = q < d_top ? 1.f : -1.f;
-  Lam[id] = (j == jj) ? sg : 0.f;
-  if (j == 0) {
-    float bv = sg * b_top[jj];
-    if (cf) cf[rl] = bv;
-    if (cd) cd[rl] = (double)bv;
-    if (E) E[rl] = 0.0;
-  }
-}
-
-// Relaxation for root rows: no splits, alpha' from the rule.
-template <bool CERT>
-__global__ void __launch_bounds__(256) k_relax_root(int Rc, int p, int H, int d, long long hoff,
-                                                    const float* __restrict__ l, const float* __restrict__ u,
-                                                    Tables tb, int rule, float rule_value,
-                                                    const float* __restrict__ Ain, float* __restrict__ Lam,
-                                                    const float* __restrict__ bias, float* __restrict__ cf,
-                                                    double* __restrict__ cd, double* __restrict__ E,
-                                                    const float* __restrict__ wm, double gamma) {
-  __shared__ float shf[32];
-  int rl = blockIdx.x;
-  const float* a_row = Ain + (size_t)rl * d;
-  float* lam_row = Lam + (size_t)rl * d;
-  // CERT: acc rounded down, e1 and e2 rounded up (as in k_relax)
-  float acc = 0.f, e1 = 0.f, e2 = 0.f;
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
-    float a = a_row[j];
-    size_t n = (size_t)p * H + hoff + j;
-    uint8_t code = tb.code[n];
-    float lv = l[n], uv = u[n];
-    float D = 0.f, lm = 0.f;
-    if (code == CODE_ACTIVE) D = 1.f;
-    else if (code == CODE_INACTIVE) D = 0.f;
-    else if (a >= 0.f) D = rule == BCROWN_ALPHA_ADAPTIVE ? (uv >= -lv ? 1.f : 0.f) : rule_value;
-    else {
-      D = tb.slope[n];
-      lm = tb.icpt[n];
-    }
-    float L = a * D;
-    lam_row[j] = L;
-    float bj = bias[j];
-    if (CERT) {
-      acc = __fadd_rd(acc, __fadd_rd(__fmul_rd(L, bj), __fmul_rd(a, lm)));
-      if (!(D == 0.f || D == 1.f)) {
-        float zmax = fmaxf(fabsf(lv), fabsf(uv));
-        float er = __fmaf_ru(fabsf(L), 0x1p-23f, 0x1p-140f);
-        e1 = __fadd_ru(e1, __fmul_ru(er, zmax));
-      }
-      e2 = __fadd_ru(e2, __fmul_ru(fabsf(L), wm[n]));
-    } else {
-      acc = fmaf(L, bj, fmaf(a, lm, acc));
-    }
-  }
-  if (CERT) {
-    acc = block_fsum<1>(acc, shf);
-    e1 = block_fsum<2>(e1, shf);
-    e2 = block_fsum<2>(e2, shf);
-    if (threadIdx.x == 0) {
-      cd[rl] = __dadd_rd(cd[rl], (double)acc);
-      E[rl] = __dadd_ru(E[rl], __dadd_ru((double)e1, __dmul_ru(gamma, (double)e2)));
-    }
-  } else {
-    acc = block_sum(acc, shf);
-    if (threadIdx.x == 0) cf[rl] += acc;
-  }
-}
-
-template <bool CERT>
-__global__ void __launch_bounds__(256) k_concretize_root(int q0, int Rc, int p, int d0, int d_top, int H,
-                                                         long long hoff_top, const float* __restrict__ x_lo,
-                                                         const float* __restrict__ x_hi,
-                                                         const float* __restrict__ A0, const float* __restrict__ cf,
-                                                         const double* __restrict__ cd, const double* __restrict__ E,
-                                                         float* __restrict__ l, float* __restrict__ u) {
-  __shared__ float shf[32];
-  int rl = blockIdx.x;
-  const float* a = A0 + (size_t)rl * d0;
-  const float* xl = x_lo + (size_t)p * d0;
-  const float* xh = x_hi + (size_t)p * d0;
-  float s = 0.f;
-  for (int m = threadIdx.x; m < d0; m += blockDim.x) {
-    float am = a[m];
-    if (CERT) s = __fadd_rd(s, fminf(__fmul_rd(am, xl[m]), __fmul_rd(am, xh[m])));
-    else s += fminf(am * xl[m], am * xh[m]);
-  }
-  float out;
-  if (CERT) {
-    s = block_fsum<1>(s, shf);
-    out = __double2float_rd(__dsub_rd(__dadd_rd(cd[rl], (double)s), E[rl]));
-  } else {
-    s = block_sum(s, shf);
-    out = cf[rl] + s;
-  }
-  if (threadIdx.x == 0) {
-    int q = q0 + rl;
-    if (q < d_top) l[(size_t)p * H + hoff_top + q] = isfinite(out) ? out : -INFINITY;
-    else u[(size_t)p * H + hoff_top + (q - d_top)] = isfinite(out) ? -out : INFINITY;
-  }
-}
-
-__global__ void k_count_unstable(int P, int H, const int32_t* __restrict__ U, int32_t* __restrict__ out) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < P) out[p] = U[p];
-}
-
-// ----------------------------------------------------------------------------------------
 // Host launchers
 // ----------------------------------------------------------------------------------------
 void launch_tables(int P, int H, const float* l, const float* u, Tables& t, uint8_t* code, int32_t* rank,
@@ -1703,34 +1586,6 @@ void launch_split(const BatchView& bt, int K, const int32_t* U, int P, const uin
                                         c_sign, c_alpha, c_beta); ++g_launches; }
 }
 
-void launch_root_top(int q0, int Rc, int d_top, const float* b_top, float* Lam, float* cf, double* cd, double* E,
-                     cudaStream_t s) {
-  long long n = (long long)Rc * d_top;
-  if (n > 0) { k_root_top<<<grid1d(n, 256), 256, 0, s>>>(q0, Rc, d_top, b_top, Lam, cf, cd, E); ++g_launches; }
-}
-
-void launch_relax_root(bool cert, int Rc, int p, int H, int d, long long hoff, const float* l, const float* u,
-                       const Tables& tb, int rule, float rule_value, const float* Ain, float* Lam, const float* bias,
-                       float* cf, double* cd, double* E, const float* wm, double gamma, cudaStream_t s) {
-  if (Rc <= 0) return;
-  if (cert)
-    { k_relax_root<true><<<Rc, 256, 0, s>>>(Rc, p, H, d, hoff, l, u, tb, rule, rule_value, Ain, Lam, bias, cf, cd, E,
-                                          wm, gamma); ++g_launches; }
-  else
-    { k_relax_root<false><<<Rc, 256, 0, s>>>(Rc, p, H, d, hoff, l, u, tb, rule, rule_value, Ain, Lam, bias, cf, cd, E,
-                                           wm, gamma); ++g_launches; }
-}
-
-void launch_concretize_root(bool cert, int q0, int Rc, int p, int d0, int d_top, int H, long long hoff_top,
-                            const float* x_lo, const float* x_hi, const float* A0, const float* cf, const double* cd,
-                            const double* E, float* l, float* u, cudaStream_t s) {
-  if (Rc <= 0) return;
-  if (cert)
-    { k_concretize_root<true><<<Rc, 256, 0, s>>>(q0, Rc, p, d0, d_top, H, hoff_top, x_lo, x_hi, A0, cf, cd, E, l, u); ++g_launches; }
-  else
-    { k_concretize_root<false><<<Rc, 256, 0, s>>>(q0, Rc, p, d0, d_top, H, hoff_top, x_lo, x_hi, A0, cf, cd, E, l, u); ++g_launches; }
-}
-
 __global__ void k_fill(float* p, long long n, float v) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
@@ -1782,10 +1637,6 @@ void launch_f32_to_bf16(const float* src, __nv_bfloat16* dst, long long n, cudaS
 }
 void launch_bf16_to_f32(const __nv_bfloat16* src, float* dst, long long n, cudaStream_t s) {
   if (n > 0) { k_bf16_to_f32<<<grid1d(n, 256), 256, 0, s>>>(src, dst, n); ++g_launches; }
-}
-
-void launch_copy_count(int P, int H, const int32_t* U, int32_t* out, cudaStream_t s) {
-  if (P > 0 && out) { k_count_unstable<<<grid1d(P, 128), 128, 0, s>>>(P, H, U, out); ++g_launches; }
 }
 
 }  // namespace bcrown

@@ -41,14 +41,6 @@ void launch_split(const BatchView& bt, int K, const int32_t* U, int P, const uin
                   const uint32_t* pick_idx, const float* alpha, const float* beta, int32_t* c_prop, int32_t* c_off,
                   int32_t* c_cnt, int64_t* c_aoff, uint8_t* c_layer, uint32_t* c_idx, int8_t* c_sign,
                   float* c_alpha, float* c_beta, int* status, cudaStream_t s);
-void launch_root_top(int q0, int Rc, int d_top, const float* b_top, float* Lam, float* cf, double* cd, double* E,
-                     cudaStream_t s);
-void launch_relax_root(bool cert, int Rc, int p, int H, int d, long long hoff, const float* l, const float* u,
-                       const Tables& tb, int rule, float rule_value, const float* Ain, float* Lam, const float* bias,
-                       float* cf, double* cd, double* E, const float* wm, double gamma, cudaStream_t s);
-void launch_concretize_root(bool cert, int q0, int Rc, int p, int d0, int d_top, int H, long long hoff_top,
-                            const float* x_lo, const float* x_hi, const float* A0, const float* cf, const double* cd,
-                            const double* E, float* l, float* u, cudaStream_t s);
 void launch_fill(float* p, long long n, float v, cudaStream_t s);
 // FP32 implicit-GEMM convolutions (conv_f32.cu): the transposed convolution of conv layer i split
 // into stride phases (backward), and the convolution plus bias (forward), for R rows.
@@ -63,6 +55,39 @@ void launch_spec_out(int R, int K, int d, const float* h, const float* Wbar, con
                      cudaStream_t s);
 void launch_f32_to_bf16(const float* src, __nv_bfloat16* dst, long long n, cudaStream_t s);
 void launch_bf16_to_f32(const __nv_bfloat16* src, float* dst, long long n, cudaStream_t s);
-void launch_copy_count(int P, int H, const int32_t* U, int32_t* out, cudaStream_t s);
+
+// Root bounds (root.cu): a chunk of the rows (property, +-, neuron of layer T) of one target layer.
+struct RootCtx {
+  long long g0;            // first row of the chunk
+  int R;                   // rows in the chunk
+  int d_top;               // neurons of layer T (rows per property: 2 d_top)
+  int top_h, top_w;        // its map (convolutions)
+  int H, d0;
+  long long hoff_top;      // its first global hidden index
+  float* l;                // [P][H], the layers below T complete
+  float* u;
+  const float* x_lo;       // [P][d0]
+  const float* x_hi;
+};
+// How a row's A^(m) lies over map m: n = 0 dense, else the n x n patch of every channel whose
+// origin is (position in layer T) * os - oo, over an Hm x Wm map.
+struct RootMap {
+  int n, Hm, Wm, os, oo;
+};
+void launch_root_first(bool cert, const RootCtx& c, int P, const LayerGeom& g, const float* W, const float* b,
+                       cudaStream_t s);
+void launch_root_top(const RootCtx& c, const LayerGeom& g, bool patch, const float* W, const float* b, float* A,
+                     float* cf, double* cd, double* E, cudaStream_t s);
+void launch_root_relax(bool cert, const RootCtx& c, const RootMap& m, int d, long long hoff, int rule,
+                       float rule_value, const float* Ain, float* Lam, const float* bias, float* cf, double* cd,
+                       double* E, const float* wm, double gamma, cudaStream_t s);
+void launch_root_concretize(bool cert, const RootCtx& c, const RootMap& m, int d, const float* A0, const float* cf,
+                            const double* cd, const double* E, cudaStream_t s);
+void launch_count_unstable(int P, int H, const float* l, const float* u, int32_t* out, cudaStream_t s);
+// Whether layer T's root rows run over patches: layers 1 .. T convolutions, and no patch larger
+// than its map; n[m] = the patch's side in map m, m = 0 .. T.
+bool root_patch(const bcrown_net* net, int T, std::vector<int>& n);
+// Backward pass of conv layer i over the patches of layer T's root rows.
+int sconv_patch(bcrown_net* net, int T, int i, int R, const float* Lam, float* Ain, cudaStream_t s);
 
 }  // namespace bcrown
