@@ -42,11 +42,13 @@ namespace tc {
 
 constexpr int TR = 64;            // rows per tile = MMA N
 constexpr int MCH = 128;          // neurons per M chunk = MMA M
-constexpr int NSLOT = 8;          // activation (B operand) ring
-constexpr int NSTAGE = 4;         // weight (A operand) ring
+constexpr int NKP_RES = 2;        // K pairs (2 blocks of 64) an operand may keep resident: 256 neurons
+constexpr int NSLOT = 3;          // activation (B operand) ring, of K pairs: a resident operand's 2
+                                  // stay until the last M chunk; the first chunk's epilogue writes a third
+constexpr int NSTAGE = 3;         // weight (A operand) ring, of K pairs
 constexpr int NACC = 4;           // accumulator ring (TR columns each)
-constexpr int SLOT_BYTES = TR * 128;     // 8 KB
-constexpr int STAGE_BYTES = MCH * 128;   // 16 KB
+constexpr int SLOT_BYTES = TR * 128;     // 8 KB: one K block of a slot
+constexpr int STAGE_BYTES = MCH * 128;   // 16 KB: one K block of a stage
 constexpr int NEPI = 16;                 // epilogue warps
 constexpr int TMA_WARP = 16, MMA_WARP = 17;
 constexpr int NTHREADS = 18 * 32;
@@ -59,11 +61,10 @@ constexpr int MAX_H = MAX_MASK_WORDS * 32;  // hidden neurons whose tables a til
 constexpr int MAX_HIDDEN = 256;
 
 struct Smem {
-  uint8_t act[NSLOT][SLOT_BYTES];        // 64 KB, 1024-aligned slots
-  uint8_t w[NSTAGE][STAGE_BYTES];        // 64 KB
+  uint8_t act[NSLOT][2 * SLOT_BYTES];    // 48 KB, 1024-aligned blocks
+  uint8_t w[NSTAGE][2 * STAGE_BYTES];    // 96 KB
   uint32_t sign[TR][SIGN_WORDS];         // 8 KB: A^(0) >= 0 per (row, input)
   uint32_t smask[MAX_MASK_WORDS][TR];    // split present, [word][row]: a warp reads its 16 rows at once
-  uint32_t sneg[MAX_MASK_WORDS][TR];     // split sign +1 (z < 0)
   unsigned long long wrows[MAX_MASK_WORDS];  // rows with any split in mask word w
   float part[4][TR];                     // lb partial sums per lane quadrant
   long long abase[TR];                   // first alpha of the row
@@ -74,7 +75,7 @@ struct Smem {
   int scnt[TR];                          // the row's split count and first split entry
   int soff[TR];
   uint8_t sorig[TR][BCROWN_MAX_SPLITS];  // the row's splits in (mask word, bit) order: list position
-  float sbeta[TR][BCROWN_MAX_SPLITS];    //   and beta (clamped at 0)
+  float sbeta[TR][BCROWN_MAX_SPLITS];    //   and beta S (beta clamped at 0; the sign bit tells S)
   uint8_t wfirst[MAX_MASK_WORDS][TR];    // splits of the row in mask words before w
   uint32_t tcode[MAX_H];                 // the tile's property: code << 16 | unstable rank, per hidden neuron
   float tslope[MAX_H];                   //   upper chord slope
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSLOT; ++i) {
-      mbar_init(&sm->act_full[i], NEPI / 2);   // the 8 warps that write a K block
+      mbar_init(&sm->act_full[i], NEPI);
       mbar_init(&sm->act_empty[i], 1);
     }
     for (int i = 0; i < NSTAGE; ++i) {
@@ -353,137 +354,133 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
   tc_fence_after();
   const uint32_t tmem = sm->tmem_base;
 
+  // The TMA and the MMA warp run their loops as whole warps (every lane takes the same waits and
+  // branches) and one lane issues: the loop state then stays in uniform registers, which the
+  // tcgen05 and TMA instructions take their operands from.  What bounds these loops is their own
+  // instructions: with one K block per wait, commit and turn, issued from a one-lane branch, a
+  // 256-deep chunk of 16 MMAs took 1.7 us, whatever the ring's depth.
   if (warp == TMA_WARP) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t wseq = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
-        for (int ci = 0; ci < n_contr && ok; ++ci) {
-          int layer, N, K;
-          bool fwd;
-          contraction(a, ci, layer, N, K, fwd);
-          const CUtensorMap* map = fwd ? &maps.fwd[layer] : &maps.bwd[layer];
-          const uint32_t bytes = (uint32_t)(fwd ? a.box_fwd[layer] : a.box_bwd[layer]) * 128u;
-          const int nmc = nmc_of(N), nkb = nkb_of(K);
-          const bool stream = nkb > NSLOT / 2;   // same order as the MMA issuer
-          const int n_outer = stream ? nkb : nmc, n_inner = stream ? nmc : nkb;
-          for (int o = 0; o < n_outer && ok; ++o)
-            for (int in = 0; in < n_inner && ok; ++in) {
-              const int mc = stream ? in : o, kb = stream ? o : in;
-              int st = wseq % NSTAGE;
-              if (!mbar_wait(&sm->w_empty[st], ((wseq / NSTAGE) & 1) ^ 1, sm, a.status)) {
-                ok = false;
-                break;
-              }
-              mbar_expect_tx(&sm->w_full[st], bytes);
-              tma_load_2d(sm->w[st], map, kb * KBLK, mc * MCH, &sm->w_full[st]);
-              ++wseq;
+    uint32_t wseq = 0, st = 0, ph = 1;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
+      for (int ci = 0; ci < n_contr && ok; ++ci) {
+        int layer, N, K;
+        bool fwd;
+        contraction(a, ci, layer, N, K, fwd);
+        const CUtensorMap* map = fwd ? &maps.fwd[layer] : &maps.bwd[layer];
+        const uint32_t bytes = (uint32_t)(fwd ? a.box_fwd[layer] : a.box_bwd[layer]) * 128u;
+        const int nmc = nmc_of(N), nkb = nkb_of(K), nkp = (nkb + 1) / 2;
+        const bool stream = nkp > NKP_RES;   // same order as the MMA issuer
+        const int n_outer = stream ? nkp : nmc, n_inner = stream ? nmc : nkp;
+        for (int o = 0; o < n_outer && ok; ++o)
+          for (int in = 0; in < n_inner; ++in) {
+            const int mc = stream ? in : o, kp = stream ? o : in;
+            if (!mbar_wait(&sm->w_empty[st], ph, sm, a.status)) {
+              ok = false;
+              break;
             }
-        }
-      if (!ok) {
-        // wait (bounded) for the copies still in flight before the CTA may exit
-        for (uint32_t s = (wseq > NSTAGE ? wseq - NSTAGE : 0); s < wseq; ++s) {
-          long long t0 = clock64();
-          while (!mbar_try(&sm->w_full[s % NSTAGE], (s / NSTAGE) & 1) && clock64() - t0 < 200000000LL) {
+            if (lane == 0) {
+              const bool two = 2 * kp + 1 < nkb;
+              mbar_expect_tx(&sm->w_full[st], two ? 2 * bytes : bytes);
+              tma_load_2d(sm->w[st], map, 2 * kp * KBLK, mc * MCH, &sm->w_full[st]);
+              if (two) tma_load_2d(sm->w[st] + STAGE_BYTES, map, (2 * kp + 1) * KBLK, mc * MCH, &sm->w_full[st]);
+            }
+            ++wseq;
+            if (++st == NSTAGE) st = 0, ph ^= 1;
           }
+      }
+    if (!ok && lane == 0) {
+      // wait (bounded) for the copies still in flight before the CTA may exit
+      for (uint32_t s = (wseq > NSTAGE ? wseq - NSTAGE : 0); s < wseq; ++s) {
+        long long t0 = clock64();
+        while (!mbar_try(&sm->w_full[s % NSTAGE], (s / NSTAGE) & 1) && clock64() - t0 < 200000000LL) {
         }
       }
     }
   } else if (warp == MMA_WARP) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      uint32_t wseq = 0, accseq = 0, aseq = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
-        for (int ci = 0; ci < n_contr && ok; ++ci) {
-          int layer, N, K;
-          bool fwd;
-          contraction(a, ci, layer, N, K, fwd);
-          const int nmc = nmc_of(N), nkb = nkb_of(K);
-          const uint32_t idesc = idesc_bf16(TR);
-          if (nkb > NSLOT / 2) {
-            // Streamed operand (more K blocks than stay resident): K blocks outer, all M
-            // chunks accumulate at once (nmc <= NACC), each K block released after use.
-            for (int mc = 0; mc < nmc && ok; ++mc) {
-              const uint32_t sq = accseq + mc;
-              if (!mbar_wait(&sm->acc_empty[sq % NACC], ((sq / NACC) & 1) ^ 1, sm, a.status)) ok = false;
-            }
-            tc_fence_after();
-            for (int kb = 0; kb < nkb && ok; ++kb) {
-              const uint32_t as = aseq + kb;
-              const int slot = as % NSLOT;
-              if (!mbar_wait(&sm->act_full[slot], (as / NSLOT) & 1, sm, a.status)) {
-                ok = false;
-                break;
-              }
-              for (int mc = 0; mc < nmc; ++mc) {
-                const int st = wseq % NSTAGE;
-                if (!mbar_wait(&sm->w_full[st], (wseq / NSTAGE) & 1, sm, a.status)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-                const uint32_t dt = tmem + (uint32_t)(((accseq + mc) % NACC) * TR);
-                const uint32_t wa = su32(sm->w[st]);
-                const uint32_t ba = su32(sm->act[slot]);
-                umma_kblock(dt, sdesc(wa), sdesc(ba), idesc, kb != 0 ? 1u : 0u);
-                umma_commit(&sm->w_empty[st]);
-                ++wseq;
-              }
-              if (!ok) break;
-              umma_commit(&sm->act_empty[slot]);
-            }
-            if (!ok) break;
-            for (int mc = 0; mc < nmc; ++mc) umma_commit(&sm->acc_full[(accseq + mc) % NACC]);
-            accseq += nmc;
-            aseq += nkb;
-            continue;
-          }
+    // (st, wph), (slot, aph): the weight stage and the activation slot read next, with the parity
+    // of their full barriers; (buf, cph): the accumulator filled next, parity of its empty barrier
+    uint32_t st = 0, wph = 0, slot = 0, aph = 0, buf = 0, cph = 1;
+    const uint32_t w0 = sdesc_lo(su32(sm->w[0])), a0 = sdesc_lo(su32(sm->act[0]));
+    const uint32_t b_wempty = su32(&sm->w_empty[0]), b_aempty = su32(&sm->act_empty[0]), b_acc = su32(&sm->acc_full[0]);
+    const uint32_t leader = lane == 0;
+    constexpr uint32_t WSTEP = 2 * STAGE_BYTES >> 4, ASTEP = 2 * SLOT_BYTES >> 4;
+    constexpr uint32_t idesc = idesc_bf16(TR);
+    bool ok = true;
+    // one K pair (or its first block) of a chunk: weights of stage st, activations of slot s
+    auto pair = [&](uint32_t dt, uint32_t s, bool first, bool two) -> bool {
+      if (!mbar_wait(&sm->w_full[st], wph, sm, a.status)) return false;
+      tc_fence_after();
+      umma_kpair<(STAGE_BYTES >> 4), (SLOT_BYTES >> 4)>(leader, dt, w0 + st * WSTEP, a0 + s * ASTEP, idesc,
+                                                        first ? 0u : 1u, two ? 1u : 0u);
+      umma_commit_if(leader, b_wempty + 8 * st);
+      if (++st == NSTAGE) st = 0, wph ^= 1;
+      return true;
+    };
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
+      for (int ci = 0; ci < n_contr && ok; ++ci) {
+        int layer, N, K;
+        bool fwd;
+        contraction(a, ci, layer, N, K, fwd);
+        const int nmc = nmc_of(N), nkb = nkb_of(K), nkp = (nkb + 1) / 2;
+        if (nkp > NKP_RES) {
+          // Streamed operand (more K pairs than stay resident): K pairs outer, all M chunks
+          // accumulate at once (nmc <= NACC), each K pair released after use.
+          uint32_t b2 = buf, c2 = cph;
           for (int mc = 0; mc < nmc && ok; ++mc) {
-            const int buf = accseq % NACC;
-            if (!mbar_wait(&sm->acc_empty[buf], ((accseq / NACC) & 1) ^ 1, sm, a.status)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t dt = tmem + (uint32_t)(buf * TR);
-            for (int kb = 0; kb < nkb; ++kb) {
-              const uint32_t as = aseq + kb;
-              const int slot = as % NSLOT;
-              if (mc == 0 && !mbar_wait(&sm->act_full[slot], (as / NSLOT) & 1, sm, a.status)) {
-                ok = false;
-                break;
-              }
-              const int st = wseq % NSTAGE;
-              if (!mbar_wait(&sm->w_full[st], (wseq / NSTAGE) & 1, sm, a.status)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              const uint32_t wa = su32(sm->w[st]);
-              const uint32_t ba = su32(sm->act[slot]);
-              umma_kblock(dt, sdesc(wa), sdesc(ba), idesc, kb != 0 ? 1u : 0u);
-              umma_commit(&sm->w_empty[st]);
-              ++wseq;
-              if (mc == nmc - 1) umma_commit(&sm->act_empty[slot]);
-            }
-            if (!ok) break;
-            umma_commit(&sm->acc_full[buf]);
-            ++accseq;
+            ok = mbar_wait(&sm->acc_empty[b2], c2, sm, a.status);
+            if (++b2 == NACC) b2 = 0, c2 ^= 1;
           }
-          aseq += nkb;
+          if (!ok) break;
+          tc_fence_after();
+          for (int kp = 0; kp < nkp && ok; ++kp) {
+            if (!(ok = mbar_wait(&sm->act_full[slot], aph, sm, a.status))) break;
+            for (int mc = 0; mc < nmc && ok; ++mc)
+              ok = pair(tmem + ((buf + mc) % NACC) * TR, slot, kp == 0, 2 * kp + 1 < nkb);
+            if (!ok) break;
+            umma_commit_if(leader, b_aempty + 8 * slot);
+            if (++slot == NSLOT) slot = 0, aph ^= 1;
+          }
+          if (!ok) break;
+          for (int mc = 0; mc < nmc; ++mc) {
+            umma_commit_if(leader, b_acc + 8 * buf);
+            if (++buf == NACC) buf = 0, cph ^= 1;
+          }
+          continue;
         }
-      umma_commit(&sm->done);
-      mbar_wait(&sm->done, 0, sm, a.status);
-    }
+        // Resident operand (one or two K pairs in slots s0, s1 for every chunk)
+        const uint32_t s0 = slot, p0 = aph;
+        const uint32_t s1 = s0 + 1 == NSLOT ? 0 : s0 + 1, p1 = s1 ? p0 : p0 ^ 1;
+        for (int mc = 0; mc < nmc; ++mc) {
+          const bool last = mc == nmc - 1;
+          if (!(ok = mbar_wait(&sm->acc_empty[buf], cph, sm, a.status))) break;
+          tc_fence_after();
+          const uint32_t dt = tmem + buf * TR;
+          if (mc == 0 && !(ok = mbar_wait(&sm->act_full[s0], p0, sm, a.status))) break;
+          if (!(ok = pair(dt, s0, true, nkb > 1))) break;
+          umma_commit_if(leader & (uint32_t)last, b_aempty + 8 * s0);
+          if (nkp > 1) {
+            if (mc == 0 && !(ok = mbar_wait(&sm->act_full[s1], p1, sm, a.status))) break;
+            if (!(ok = pair(dt, s1, false, nkb > 3))) break;
+            umma_commit_if(leader & (uint32_t)last, b_aempty + 8 * s1);
+          }
+          umma_commit_if(leader, b_acc + 8 * buf);
+          if (++buf == NACC) buf = 0, cph ^= 1;
+        }
+        for (int kp = 0; kp < nkp; ++kp)
+          if (++slot == NSLOT) slot = 0, aph ^= 1;
+      }
+    umma_commit_if(leader, su32(&sm->done));
+    mbar_wait(&sm->done, 0, sm, a.status);
   } else {
     // ---------------------------------------------------------------- epilogue (warps 0..15)
     const int q = warp & 3;          // TMEM lane quadrant: neurons 32q..32q+31 of an M chunk
     const int cg = warp >> 2;        // column group: tile rows 16cg..16cg+15
     const int r0 = 16 * cg;          // first tile row of this thread
     const int etid = threadIdx.x;    // 0..511
-    const int pg = warp & 1;         // producer group: writes the K blocks kb with kb % 2 == pg
+    const int pg = warp & 1;         // producer group: writes block pg of every K pair
     const int gt = (warp >> 1) * 32 + lane;   // thread index within the producer group, 0..255
     const int prow = gt >> 2, pc16 = gt & 3;  // producer thread: tile row, 16 consecutive k
     uint32_t aseq = 0, accseq = 0, eseq = 0;
@@ -572,10 +569,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           }
         }
       }
-      for (int x = etid; x < a.mask_words * TR; x += NEPI * 32) {
-        (&sm->smask[0][0])[x] = 0u;
-        (&sm->sneg[0][0])[x] = 0u;
-      }
+      for (int x = etid; x < a.mask_words * TR; x += NEPI * 32) (&sm->smask[0][0])[x] = 0u;
       if (etid < a.mask_words) sm->wrows[etid] = 0ull;
       if (!epi_sync(sm, eseq, a.status)) {
         ok = false;
@@ -605,8 +599,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
             } else {
               const int wd = a.woff[ly] + (j >> 5);
               atomicOr(&sm->smask[wd][row], 1u << (j & 31));
-              if (s == 1) atomicOr(&sm->sneg[wd][row], 1u << (j & 31));
               ent[m] = (wd << 5) | (j & 31);
+              bv[m] = fmaxf(bv[m], 0.f) * (float)s;
             }
           }
         }
@@ -656,7 +650,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           if (ent[m] >= 0) {
             const int ks = split_slot(sm, row, ent[m] >> 5, ent[m] & 31);
             sm->sorig[row][ks] = (uint8_t)(e0 + 8 * m);
-            sm->sbeta[row][ks] = fmaxf(bv[m], 0.f);
+            sm->sbeta[row][ks] = bv[m];
           }
         }
       }
@@ -681,7 +675,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
         const int nmc = nmc_of(N);
         const bool concretise = (i == 1);
         const int li = i - 1;
-        const int nkb_next = concretise ? 0 : nkb_of(N);
+        const int nkb_next = concretise ? 0 : nkb_of(N), nkp_next = (nkb_next + 1) / 2;
         for (int mc = 0; mc < nmc && ok; ++mc) {
           const int buf = accseq % NACC;
           const int j = mc * MCH + 32 * q + lane;   // output neuron of this lane
@@ -735,8 +729,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           const bool unst = code == CODE_UNSTABLE;
           const float apos = code == CODE_ACTIVE ? 1.f : 0.f;
           const int kb = (mc * MCH + 32 * q) / KBLK;   // this warp's K block of the next operand
-          const bool writer = kb < nkb_next;
-          const uint32_t as = aseq + kb;
+          const bool writer = kb < nkb_next;          // (the pair's second block may lie past the end)
+          const bool pwriter = mc < nkp_next;         // chunk mc is K pair mc of the next operand
+          const uint32_t as = aseq + mc;
           const int slot = as % NSLOT;
           // split bits of the warp's 32 neurons (none when they all lie past the layer's end)
           const int wd = a.woff[li] + ((mc * MCH + 32 * q) >> 5);
@@ -748,7 +743,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           for (int c = 0; c < 16; ++c) al[c] = ldg_f32(a.alpha + sm->abase[r0 + c] + rank, unst && ((vbits >> c) & 1u));
           // byte offset of (row r0 + 8h + c8, k = j % 64) in the slot: row & 7 == c8
           const int kk = j & (KBLK - 1);
-          uint8_t* aslot = sm->act[slot] + r0 * 128 + ((kk & 7) << 1);
+          uint8_t* aslot = sm->act[slot] + (kb & 1) * SLOT_BYTES + r0 * 128 + ((kk & 7) << 1);
           const uint32_t kx = (uint32_t)(kk >> 3) << 4;
           // rows r0 + 8h .. r0 + 8h + 7 of A^(i-1)_j: relaxation, lb terms, operand and stash
           auto relax8 = [&](const int h, const float (&v)[8]) {
@@ -763,10 +758,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
               float bs = 0.f;
               if ((rbits >> c) & 1u) {
                 if (sm->smask[wd][row] & bit) {
-                  const int sg = (sm->sneg[wd][row] & bit) ? 1 : -1;
-                  D = sg == -1 ? 1.f : 0.f;
+                  bs = sm->sbeta[row][split_slot(sm, row, wd, lane)];
+                  D = signbit(bs) ? 1.f : 0.f;
                   lm = 0.f;
-                  bs = sm->sbeta[row][split_slot(sm, row, wd, lane)] * (float)sg;
                 }
               }
               const float L = fmaf(av, D, bs);
@@ -795,7 +789,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
             }
             tc_fence_after();
           }
-          if (writer && !mbar_wait_warp(&sm->act_empty[slot], ((as / NSLOT) & 1) ^ 1, sm, a.status)) {
+          if (pwriter && !mbar_wait_warp(&sm->act_empty[slot], ((as / NSLOT) & 1) ^ 1, sm, a.status)) {
             ok = false;
             break;
           }
@@ -831,14 +825,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
             for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(u1[e]);
             relax8(1, v);
           }
-          // each K block is complete once its 8 writer warps arrived
-          if (writer) {
+          // each K pair is complete once all warps arrived
+          if (pwriter) {
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm->act_full[slot]);
           }
         }
-        aseq += nkb_next;
+        aseq += nkp_next;
       }
       if (!ok) break;
 
@@ -865,10 +859,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
       // ---------------- adjoint: x* operand (K blocks of d0), then forward contractions
       {
         const int d0 = a.d[0];
-        const int nkb = nkb_of(d0);
+        const int nkb = nkb_of(d0), nkp = (nkb + 1) / 2;
         const bool rv = sm->valid[prow] != 0;
-        for (int kb = pg; kb < nkb && ok; kb += 2) {
-          const uint32_t as = aseq + kb;
+        for (int kp = 0; kp < nkp && ok; ++kp) {
+          const int kb = 2 * kp + pg;   // past the end in an odd operand's last pair: zeros, unread
+          const uint32_t as = aseq + kp;
           const int slot = as % NSLOT;
           if (!mbar_wait_warp(&sm->act_empty[slot], ((as / NSLOT) & 1) ^ 1, sm, a.status)) {
             ok = false;
@@ -892,20 +887,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
             __nv_bfloat162 v2 = __floats2bfloat162_rn(xv[0], xv[1]);
             pk[e >> 1] = *reinterpret_cast<uint32_t*>(&v2);
           }
-          *reinterpret_cast<uint4*>(sm->act[slot] + act_off(prow, pc16 * 16)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          *reinterpret_cast<uint4*>(sm->act[slot] + act_off(prow, pc16 * 16 + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          *reinterpret_cast<uint4*>(sm->act[slot] + pg * SLOT_BYTES + act_off(prow, pc16 * 16)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          *reinterpret_cast<uint4*>(sm->act[slot] + pg * SLOT_BYTES + act_off(prow, pc16 * 16 + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
           fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(&sm->act_full[slot]);
         }
-        aseq += nkb;
+        aseq += nkp;
       }
       // zhat^(i) = W^(i) h^(i-1) + b^(i); dalpha = A zhat (unstable, unsplit, A >= 0), dbeta = S zhat;
       // h^(i) = D zhat + lambda is the next forward operand
       for (int i = 1; i <= a.L - 1 && ok; ++i) {
         const int N = a.d[i];
         const int nmc = nmc_of(N);
-        const int nkb_next = (i + 1 <= a.L - 1) ? nkb_of(N) : 0;
+        const int nkb_next = (i + 1 <= a.L - 1) ? nkb_of(N) : 0, nkp_next = (nkb_next + 1) / 2;
         for (int mc = 0; mc < nmc && ok; ++mc) {
           const int buf = accseq % NACC;
           const int j = mc * MCH + 32 * q + lane;
@@ -924,8 +919,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           const bool unst = code == CODE_UNSTABLE;
           const float apos = code == CODE_ACTIVE ? 1.f : 0.f;
           const int kb = (mc * MCH + 32 * q) / KBLK;
-          const bool writer = kb < nkb_next;
-          const uint32_t as = aseq + kb;
+          const bool writer = kb < nkb_next;          // (the pair's second block may lie past the end)
+          const bool pwriter = mc < nkp_next;         // chunk mc is K pair mc of the next operand
+          const uint32_t as = aseq + mc;
           const int slot = as % NSLOT;
           const int wd = a.woff[i] + ((mc * MCH + 32 * q) >> 5);
           const uint32_t bit = 1u << lane;
@@ -941,12 +937,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
             break;
           }
           tc_fence_after();
-          if (writer && !mbar_wait_warp(&sm->act_empty[slot], ((as / NSLOT) & 1) ^ 1, sm, a.status)) {
+          if (pwriter && !mbar_wait_warp(&sm->act_empty[slot], ((as / NSLOT) & 1) ^ 1, sm, a.status)) {
             ok = false;
             break;
           }
           const int kk = j & (KBLK - 1);
-          uint8_t* aslot = sm->act[slot] + r0 * 128 + ((kk & 7) << 1);
+          uint8_t* aslot = sm->act[slot] + (kb & 1) * SLOT_BYTES + r0 * 128 + ((kk & 7) << 1);
           const uint32_t kx = (uint32_t)(kk >> 3) << 4;
           const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * TR + r0);
           // rows r0 + 8h .. r0 + 8h + 7: zhat, gradients, next operand
@@ -966,12 +962,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
               float g = pos ? A * z : 0.f;
               if ((rbits >> c) & 1u) {
                 if (sm->smask[wd][row] & bit) {
-                  const int sg = (sm->sneg[wd][row] & bit) ? 1 : -1;
-                  D = sg == -1 ? 1.f : 0.f;
+                  const int ks = split_slot(sm, row, wd, lane);
+                  const bool neg = signbit(sm->sbeta[row][ks]);   // S = -1: z >= 0
+                  D = neg ? 1.f : 0.f;
                   lm = 0.f;
                   g = 0.f;
-                  const long long bi = sm->bbase[row] + sm->sorig[row][split_slot(sm, row, wd, lane)];
-                  if (bi < a.n_beta) a.dbeta[bi] = (float)sg * z;
+                  const long long bi = sm->bbase[row] + sm->sorig[row][ks];
+                  if (bi < a.n_beta) a.dbeta[bi] = neg ? -z : z;
                 }
               }
               if (unst && rin) {
@@ -995,13 +992,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
           if (lane == 0) mbar_arrive(&sm->acc_empty[buf]);
           ++accseq;
           fwd8(1, u1);
-          if (writer) {
+          if (pwriter) {
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm->act_full[slot]);
           }
         }
-        aseq += nkb_next;
+        aseq += nkp_next;
       }
       if (ok && !epi_sync(sm, eseq, a.status)) ok = false;
     }

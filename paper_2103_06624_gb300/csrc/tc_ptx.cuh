@@ -96,6 +96,37 @@ __device__ __forceinline__ void umma_kblock(uint32_t dtmem, uint64_t ad, uint64_
       "l"(bd + 6)
       : "memory");
 }
+// Low word of sdesc (the high word is a constant).
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
+// A K pair -- the K block at (alo, blo) and, with `two`, the one astep / bstep 16-byte units on --
+// issued by a whole warp's code with `leader` set in one lane: predicated instructions instead of a
+// one-lane branch, and descriptors built from 32-bit words, for a warp whose own instructions are
+// what an MMA waits for.
+template <uint32_t ASTEP, uint32_t BSTEP>
+__device__ __forceinline__ void umma_kpair(uint32_t leader, uint32_t dtmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                           uint32_t acc, uint32_t two) {
+  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+#define BC_UMMA(P, OFF_A, OFF_B, ACC)                                                                  \
+  "add.u32 x, %1, " OFF_A ";\n\tadd.u32 y, %2, " OFF_B ";\n\tmov.b64 a, {x, %6};\n\tmov.b64 b, {y, %6};\n\t" \
+  "@" P " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, " ACC ";\n\t"
+  asm volatile(
+      "{\n\t.reg .pred l, m, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
+      "setp.ne.b32 l, %7, 0;\n\tsetp.ne.and.b32 m, %5, 0, l;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      BC_UMMA("l", "0", "0", "p") BC_UMMA("l", "2", "2", "q") BC_UMMA("l", "4", "4", "q") BC_UMMA("l", "6", "6", "q")
+      BC_UMMA("m", "%8", "%9", "q") BC_UMMA("m", "%10", "%11", "q") BC_UMMA("m", "%12", "%13", "q")
+      BC_UMMA("m", "%14", "%15", "q") "}" ::"r"(dtmem),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(two), "n"(hi), "r"(leader), "n"(ASTEP), "n"(BSTEP),
+      "n"(ASTEP + 2), "n"(BSTEP + 2), "n"(ASTEP + 4), "n"(BSTEP + 4), "n"(ASTEP + 6), "n"(BSTEP + 6)
+      : "memory");
+#undef BC_UMMA
+}
+__device__ __forceinline__ void umma_commit_if(uint32_t pred, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+      "@p tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+      "r"(pred)
+      : "memory");
+}
 // Shared-memory descriptor, K-major, no swizzle: 8-row x 16-byte core matrices stored as 128
 // contiguous bytes, `sbo` bytes apart along M and `lbo` bytes apart along K.
 __device__ __forceinline__ uint64_t sdesc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
@@ -158,6 +189,28 @@ __device__ __forceinline__ void tmem_wait8(uint32_t (&r)[8]) {
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
                :
                : "memory");
+}
+
+// The same for 4 columns.
+__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait4(uint32_t (&r)[4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[N]) {
+  static_assert(N == 4 || N == 8, "columns per load");
+  if constexpr (N == 8) tmem_ld8_issue(taddr, r);
+  else tmem_ld4_issue(taddr, r);
+}
+template <int N>
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[N]) {
+  if constexpr (N == 8) tmem_wait8(r);
+  else tmem_wait4(r);
 }
 
 // Tensor map of a BF16 [rows][kp] matrix (kp a multiple of 64): boxes of 64 x box_rows, 128-byte
