@@ -98,33 +98,57 @@ __device__ __forceinline__ void umma_kblock(uint32_t dtmem, uint64_t ad, uint64_
 }
 // Low word of sdesc (the high word is a constant).
 __device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
-// A K pair -- the K block at (alo, blo) and, with `two`, the one astep / bstep 16-byte units on --
-// issued by a whole warp's code with `leader` set in one lane: predicated instructions instead of a
-// one-lane branch, and descriptors built from 32-bit words, for a warp whose own instructions are
-// what an MMA waits for.
+// A K pair -- the K block at (alo, blo) and, with `two`, the one ASTEP / BSTEP 16-byte units on -- and
+// the commit to `bar`, for a whole converged warp: elect.sync picks the lane, the instructions are
+// predicated (no one-lane branch), and the descriptors are built from 32-bit words.  This matters
+// to a warp whose own instructions are what an MMA waits for: measured per MMA of 128 x N x 16,
+// issued back to back, 39 cycles (48 at N = 64, the tensor core's own time) against 47 from a
+// one-lane branch and 67 under a predicate computed from the lane index.
 template <uint32_t ASTEP, uint32_t BSTEP>
-__device__ __forceinline__ void umma_kpair(uint32_t leader, uint32_t dtmem, uint32_t alo, uint32_t blo, uint32_t idesc,
-                                           uint32_t acc, uint32_t two) {
+__device__ __forceinline__ void umma_kpair(uint32_t dtmem, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc,
+                                           uint32_t two, uint32_t bar) {
   constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
 #define BC_UMMA(P, OFF_A, OFF_B, ACC)                                                                  \
   "add.u32 x, %1, " OFF_A ";\n\tadd.u32 y, %2, " OFF_B ";\n\tmov.b64 a, {x, %6};\n\tmov.b64 b, {y, %6};\n\t" \
   "@" P " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, " ACC ";\n\t"
   asm volatile(
-      "{\n\t.reg .pred l, m, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
-      "setp.ne.b32 l, %7, 0;\n\tsetp.ne.and.b32 m, %5, 0, l;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "{\n\t.reg .pred l, m, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y, d;\n\telect.sync d|l, 0xffffffff;\n\t"
+      "setp.ne.and.b32 m, %5, 0, l;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
       BC_UMMA("l", "0", "0", "p") BC_UMMA("l", "2", "2", "q") BC_UMMA("l", "4", "4", "q") BC_UMMA("l", "6", "6", "q")
       BC_UMMA("m", "%8", "%9", "q") BC_UMMA("m", "%10", "%11", "q") BC_UMMA("m", "%12", "%13", "q")
-      BC_UMMA("m", "%14", "%15", "q") "}" ::"r"(dtmem),
-      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(two), "n"(hi), "r"(leader), "n"(ASTEP), "n"(BSTEP),
+      BC_UMMA("m", "%14", "%15", "q")
+      "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t}" ::"r"(dtmem),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(two), "n"(hi), "r"(bar), "n"(ASTEP), "n"(BSTEP),
       "n"(ASTEP + 2), "n"(BSTEP + 2), "n"(ASTEP + 4), "n"(BSTEP + 4), "n"(ASTEP + 6), "n"(BSTEP + 6)
       : "memory");
 #undef BC_UMMA
 }
-__device__ __forceinline__ void umma_commit_if(uint32_t pred, uint32_t bar) {
+// One K block and the commit to `bar` for a converged warp, as above.  HI_A: high word of the A
+// descriptor, STEP_A: its advance per K step of 16 (16-byte units).
+template <uint32_t HI_A, uint32_t STEP_A>
+__device__ __forceinline__ void umma_kblock_warp(uint32_t dtmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                                 uint32_t acc, uint32_t bar) {
+  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+#define BC_UMMA1(OFF_A, OFF_B, ACC)                                                                    \
+  "add.u32 x, %1, " OFF_A ";\n\tadd.u32 y, %2, " OFF_B ";\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %6};\n\t" \
+  "@l tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, " ACC ";\n\t"
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t"
-      "@p tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
-      "r"(pred)
+      "{\n\t.reg .pred l, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y, d;\n\telect.sync d|l, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      BC_UMMA1("0", "0", "p") BC_UMMA1("%8", "2", "q") BC_UMMA1("%9", "4", "q") BC_UMMA1("%10", "6", "q")
+      "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t}" ::"r"(dtmem),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(HI_A), "n"(hi), "r"(bar), "n"(STEP_A), "n"(2 * STEP_A),
+      "n"(3 * STEP_A)
+      : "memory");
+#undef BC_UMMA1
+}
+constexpr uint32_t SDESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);         // sdesc's high word
+__host__ __device__ constexpr uint32_t SDESC_PLAIN_HI(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }   // sdesc_plain's
+// A commit by one lane of a converged warp.
+__device__ __forceinline__ void umma_commit_warp(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred l;\n\t.reg .b32 d;\n\telect.sync d|l, 0xffffffff;\n\t"
+      "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
       : "memory");
 }
 // Shared-memory descriptor, K-major, no swizzle: 8-row x 16-byte core matrices stored as 128
