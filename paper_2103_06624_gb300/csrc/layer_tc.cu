@@ -16,13 +16,12 @@
 //                       epilogue: dalpha = A zhat (unstable, unsplit, A >= 0), dbeta = S zhat,
 //                       h^(i) = D zhat + lambda stored in BF16 as the next operand.
 //
-// Activations are BF16 in NHWC order (channels innermost, padded to a multiple of 8), so that the
-// GEMM operand -- rows = (subdomain row, output position), K = (tap, channel) -- is gathered into
-// shared memory in 16-byte pieces of 8 channels, one load each; gather warps write it in the
-// 128-byte-swizzled K-major layout the MMA reads, TMA streams the weights, one thread issues the
-// MMAs into one of three TMEM accumulators (two for 256-column tiles), and three groups of 4
-// epilogue warps read them with tcgen05.ld, each group every third tile, so that up to three
-// tiles' epilogues run at once (576 threads: 12 epilogue, 1 TMA, 1 MMA and 4 gather warps).
+// Activations are BF16 in NHWC order (channels innermost, padded to a multiple of 8).  The GEMM
+// operand -- rows = (subdomain row, output position), K = (tap, channel) -- comes by TMA where an M
+// tile is one box of the map, else it is gathered into shared memory in 16-byte pieces of 8 channels
+// by 4 gather warps.  TMA streams the weights, one warp issues the MMAs into up to four TMEM
+// accumulators (two for 256-column tiles), and as many groups of 4 epilogue warps read them, each
+// group its own, so that their tiles' epilogues run at once.
 // The bias sums of each row are written as partial sums (one slot per position block and column
 // group) and added in a fixed order at the end, so the result does not depend on scheduling.
 // A at the unstable neurons is stashed in BF16, laid out like alpha, for the adjoint pass; its
@@ -46,29 +45,47 @@ namespace lt {
 
 using namespace tc;
 
-constexpr int NS = 4;                       // pipeline stages (A: 128 x 64, B: Np x 64)
+// Pipeline stages of one K block (A: 128 x 64, B: Np x 64); the gathering form has one per gather warp.
+constexpr int NS_MAX = 5, NS_GATHER = 4;
+__host__ __device__ constexpr int lt_stages(bool ta, int Np) {
+  return Np > 128 ? 3 : !ta ? NS_GATHER : Np <= 64 ? 5 : 4;
+}
+// An epilogue warp's list of special elements (32 lanes x at most 16 columns, or 64 columns that hold
+// fewer) and its lanes' rows.
+constexpr int CAP = 512;
+struct LtList {
+  int4 row[32][2];           // {alpha base lo, hi, neuron table offset lo, hi}, {output offset lo, hi, chord base, -}
+  float val[CAP];
+  uint16_t ent[CAP];         // column | lane << 8 | split << 15
+  // the splits of the warp's row in this layer, where its positions lie in one row of a convolution
+  // (at most 256 channels, 2^22 positions): packed entry, channel | position << 9
+  int2 split[BCROWN_MAX_SPLITS];
+};
+
+// n / d for n < 2^31 by multiplication.
+struct FastDiv {
+  uint32_t d, mul, sh;
+  __host__ void set(uint32_t v) {
+    d = v;
+    sh = 0;
+    while ((1ull << sh) < v) ++sh;
+    mul = (uint32_t)((((1ull << sh) - v) << 32) / v + 1);
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t n) const { return (__umulhi(n, mul) + n) >> sh; }
+};
 // Warp roles.  Gathered A operand: 12 epilogue warps (three groups of 4, every third tile) and 4
-// gather warps (one per ring slot).  A operand by TMA: 16 epilogue warps (four groups).  Both with
+// gather warps.  A operand by TMA: 16 epilogue warps (four groups).  Both with
 // the TMA and the MMA warp: 18 warps, which leaves 96 registers a thread.
-// LT_TA_GROUPS: epilogue groups of the TMA form (4: 18 warps, 96 registers a thread -- 5 warps on
-// two of the SM's four schedulers; 3: 14 warps, 128 registers).
-#ifndef LT_TA_GROUPS
-#define LT_TA_GROUPS 4
-#endif
-#ifndef LT_FWD_PREFETCH
-#define LT_FWD_PREFETCH 0
-#endif
 template <bool TA>
 struct LtRoles {
-  static constexpr int EPI = TA ? 4 * LT_TA_GROUPS : 12;   // epilogue warps
+  static constexpr int EPI = TA ? 16 : 12;   // epilogue warps
   static constexpr int NGRP = EPI / 4;       // epilogue groups, one TMEM accumulator each
-  static constexpr int GW = TA ? 0 : NS;     // gather warps, one per ring slot
+  static constexpr int GW = TA ? 0 : NS_GATHER;   // gather warps
   static constexpr int TMA_W = EPI, MMA_W = EPI + 1, GATHER0 = EPI + 2;
   static constexpr int THREADS = (EPI + 2 + GW) * 32;
 };
 constexpr int MAX_NP = 256;
 constexpr int MAX_KP = 2048;
-constexpr int MAX_KEEP = 6;                 // splits of a row kept in registers per tile
 
 enum { EPI_RELAX = 0, EPI_CONCRETIZE = 1, EPI_FWD = 2 };
 
@@ -88,6 +105,7 @@ struct Pass {
   // output position of (row, pp): (oa + os * i) * Wo + ob + os * j; npos: position from n
   int oa, ob, os, Wo, npos;
   int Co, HWo, Cpo;          // output map: channels, positions, padded channels
+  FastDiv dPm, dnJ, dntn, dHWo, dCpo;   // (set at the launch)
   __nv_bfloat16* dst;        // NHWC BF16 output (null: none)
   long long dst_stride;
   int layer;                 // hidden layer of the epilogue (0: the input)
@@ -96,6 +114,7 @@ struct Pass {
   const float* bnhwc;        // its bias in NHWC order (padded channels 0)
   const uint32_t* ntab;      // its neurons in NHWC order, property 0 (stride Ctx::NH per property):
                              // code (0 inactive, 1 active, 2 unstable) | rank among the unstable << 2
+  const uint16_t* mtab;      // the same per 8 neurons (stride NH / 8): active bits | unstable bits << 8
   int slot0;                 // first partial-sum slot of this pass
   // A operand by TMA instead of the gather warps: 0 gathered; 4: one box [64 channels][bw][bh][br]
   // of the NHWC source per (tap, 64-channel block) -- an M tile is br rows x bh x bw positions;
@@ -109,6 +128,7 @@ struct Pass {
 // Per-call context of the epilogues.
 struct Ctx {
   int r0, R, K, P, H, d0, S;
+  FastDiv dK;
   BatchView bt;
   Tables tb;
   const float* x_lo;
@@ -140,8 +160,7 @@ __device__ __forceinline__ bool lt_wait(uint64_t* b, uint32_t parity, volatile i
   if (mbar_try(b, parity)) return true;
   long long t0 = clock64();
   while (true) {
-    // try_wait without a suspend-time hint: the hardware's own short wait window, then a re-poll
-    if (mbar_try(b, parity)) return true;
+    if (mbar_try_sleep(b, parity, 20000u)) return true;
     if (*abort) return false;
     if (clock64() - t0 > 4000000000LL) {
       atomicCAS(status, 0, BCROWN_ERR_TIMEOUT);
@@ -192,17 +211,19 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
   const uint32_t pad = (1024u - (su32(lsm_raw) & 1023u)) & 1023u;
   uint8_t* base = lsm_raw + pad;
   const int bbytes = Np * 128;
+  const int NS = lt_stages(TA, Np);
   uint8_t* sA = base;                                  // NS x 16 KB
   uint8_t* sB = base + NS * 16384;                     // NS x Np * 128
   uint64_t* bars = reinterpret_cast<uint64_t*>(sB + NS * bbytes);
   uint64_t* full = bars;
-  uint64_t* empty = bars + NS;
-  uint64_t* acc_full = bars + 2 * NS;        // up to 4 accumulators
-  uint64_t* acc_empty = bars + 2 * NS + 4;
-  uint32_t* tbase_sm = reinterpret_cast<uint32_t*>(bars + 2 * NS + 8);
+  uint64_t* empty = bars + NS_MAX;
+  uint64_t* acc_full = bars + 2 * NS_MAX;    // up to 4 accumulators
+  uint64_t* acc_empty = bars + 2 * NS_MAX + 4;
+  uint32_t* tbase_sm = reinterpret_cast<uint32_t*>(bars + 2 * NS_MAX + 8);
   volatile int* abort = reinterpret_cast<volatile int*>(tbase_sm + 1);
   int2* stab = reinterpret_cast<int2*>(bars + 32);     // 256 bytes past the barriers
   float* sbias = reinterpret_cast<float*>(stab + MAX_KP / 8);   // conv passes: the layer's channel biases
+  LtList* slist = reinterpret_cast<LtList*>(sbias + MAX_NP);    // one per epilogue warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long ntiles = (M + 127) / 128 * ps.ntn;   // tile = m tile * ntn + n tile
   // accumulators in use: one per epilogue group, as many groups as their Np columns each fit in
@@ -234,41 +255,42 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
 
   if (warp == RL::TMA_W) {
     // ------------------------------------------------------------ weights (B) by TMA, and A with TA
-    // One thread issues every copy, so its loop holds no division and no global load per K
-    // block: the tile's coordinates are worked out once per tile, the tap table is in shared
-    // memory (the gathering kernel's table space).
+    // The whole warp runs the loop and one elected lane issues: no division and no global load per
+    // K block (the tile's coordinates are worked out once per tile, the tap table is in shared
+    // memory, the gathering kernel's table space).
     int4* sktab = reinterpret_cast<int4*>(stab);
     if (TA && (ps.ta == 4 || ps.ta == 8)) {
       for (int k = lane; k < (ps.ta == 8 ? 8 * nkb : nkb); k += 32) sktab[k] = ps.ktab[k];
       __syncwarp();
     }
-    if (lane == 0) {
-      uint32_t seq = 0;
-      int st = 0;
-      uint32_t ph = 0;   // parity of the current pass over the ring
-      bool ok = true;
-      for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const long long mt = tile / ps.ntn;
-        const int brow = ps.brow + (int)(tile - mt * ps.ntn) * Np;
-        int ax = 0, ay = 0, ar = 0;   // TA: the box origin of the tile's first position, tap 0
-        if constexpr (TA) {
-          const long long m0 = mt * 128;
-          if (ps.ta == 2) {
-            ar = (int)m0;
-          } else {
-            const long long r0 = m0 / ps.Pm;
-            const int pp0 = (int)(m0 - r0 * ps.Pm);
-            const int i0 = pp0 / ps.nJ;
-            ax = (pp0 - i0 * ps.nJ) * ps.ms + ps.cx;
-            ay = i0 * ps.ms + ps.cy;
-            ar = (int)r0;
-          }
+    uint32_t seq = 0;
+    int st = 0;
+    uint32_t ph = 0;   // parity of the current pass over the ring
+    bool ok = true;
+    for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      const long long mt = tile / ps.ntn;
+      const int brow = ps.brow + (int)(tile - mt * ps.ntn) * Np;
+      int ax = 0, ay = 0, ar = 0;   // TA: the box origin of the tile's first position, tap 0
+      if constexpr (TA) {
+        const long long m0 = mt * 128;
+        if (ps.ta == 2) {
+          ar = (int)m0;
+        } else {
+          const long long r0 = m0 / ps.Pm;
+          const int pp0 = (int)(m0 - r0 * ps.Pm);
+          const int i0 = pp0 / ps.nJ;
+          ax = (pp0 - i0 * ps.nJ) * ps.ms + ps.cx;
+          ay = i0 * ps.ms + ps.cy;
+          ar = (int)r0;
         }
-        for (int kb = 0; kb < nkb; ++kb, ++seq) {
-          if (!lt_wait(&empty[st], ph ^ 1, abort, cx.status)) {
-            ok = false;
-            break;
-          }
+      }
+      for (int kb = 0; kb < nkb; ++kb, ++seq) {
+        if (!lt_wait(&empty[st], ph ^ 1, abort, cx.status)) {
+          ok = false;
+          break;
+        }
+        __syncwarp();
+        if (lane == 0) {
           mbar_expect_tx(&full[st], (TA ? 16384u : 0u) + (uint32_t)bbytes);
           if constexpr (TA) {
             if (ps.ta == 2) {
@@ -289,51 +311,55 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
             }
           }
           tma_load_2d(sB + st * bbytes, &mapB, kb * 64, brow, &full[st]);
-          if (++st == NS) st = 0, ph ^= 1;
         }
+        if (++st == NS) st = 0, ph ^= 1;
       }
-      if (!ok) {
-        for (uint32_t q = (seq > NS ? seq - NS : 0); q < seq; ++q) {
-          long long t0 = clock64();
-          while (!mbar_try(&full[q % NS], (q / NS) & 1) && clock64() - t0 < 200000000LL) {
-          }
+    }
+    if (!ok && lane == 0) {
+      for (uint32_t q = (seq > (uint32_t)NS ? seq - NS : 0); q < seq; ++q) {
+        long long t0 = clock64();
+        while (!mbar_try(&full[q % NS], (q / NS) & 1) && clock64() - t0 < 200000000LL) {
         }
       }
     }
   } else if (warp == RL::MMA_W) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t seq = 0, accseq = 0;
-      bool ok = true;
-      const uint32_t idesc = idesc_bf16(Np);
-      for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++accseq) {
-        const int buf = (int)(accseq % (uint32_t)ngrp);
-        if (!lt_wait(&acc_empty[buf], ((accseq / (uint32_t)ngrp) & 1) ^ 1, abort, cx.status)) break;
-        tc_fence_after();
-        const uint32_t dt = tmem + (uint32_t)(buf * Np);
-        for (int kb = 0; kb < nkb; ++kb, ++seq) {
-          const int st = seq % NS;
-          if (!lt_wait(&full[st], (seq / NS) & 1, abort, cx.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          if (TA && ps.ta == 8)   // A without swizzle: core matrices 128 B apart along M, 2 KB along K
-            umma_kblock_astep(dt, sdesc_plain(su32(sA + st * 16384), 2048, 128), sdesc(su32(sB + st * bbytes)),
-                              idesc, kb != 0 ? 1u : 0u, 4096 >> 4);
-          else
-            umma_kblock(dt, sdesc(su32(sA + st * 16384)), sdesc(su32(sB + st * bbytes)), idesc, kb != 0 ? 1u : 0u);
-          umma_commit(&empty[st]);
+    // (whole warp, one elected lane issues: see umma_kpair)
+    uint32_t buf = 0, cph = 1, wph = 0;
+    int st = 0;
+    bool ok = true;
+    const uint32_t idesc = idesc_bf16(Np);
+    const uint32_t b0 = sdesc_lo(su32(sB)), bstep = (uint32_t)bbytes >> 4;
+    const bool plain = TA && ps.ta == 8;   // A without swizzle: core matrices 128 B apart along M, 2 KB along K
+    const uint32_t a0 = plain ? ((su32(sA) >> 4) & 0x3FFFu) | ((2048u >> 4) << 16) : sdesc_lo(su32(sA));
+    const uint32_t b_empty = su32(empty), b_acc = su32(acc_full);
+    for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      if (!lt_wait(&acc_empty[buf], cph, abort, cx.status)) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + buf * (uint32_t)Np;
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!lt_wait(&full[st], wph, abort, cx.status)) {
+          ok = false;
+          break;
         }
-        if (!ok) break;
-        umma_commit(&acc_full[buf]);
+        __syncwarp();
+        tc_fence_after();
+        const uint32_t al = a0 + (uint32_t)st * (16384 >> 4), bl = b0 + (uint32_t)st * bstep;
+        if (plain)
+          umma_kblock_warp<SDESC_PLAIN_HI(128), (4096 >> 4)>(dt, al, bl, idesc, kb != 0 ? 1u : 0u, b_empty + 8 * st);
+        else
+          umma_kblock_warp<SDESC_HI, 2>(dt, al, bl, idesc, kb != 0 ? 1u : 0u, b_empty + 8 * st);
+        if (++st == NS) st = 0, wph ^= 1;
       }
+      if (!ok) break;
+      umma_commit_warp(b_acc + 8 * buf);
+      if (++buf == (uint32_t)ngrp) buf = 0, cph ^= 1;
     }
   } else if (!TA && warp >= RL::GATHER0) {
     // ------------------------------------------------------------ operand (A) gather
-    // ring slot g takes sequence numbers g, g + NS, ... of the (tile, K block) order; this warp
-    // writes chunks CPW part .. CPW part + CPW - 1 (of 8 per row) of its slot's stages
-    const int g = (warp - RL::GATHER0) % NS, part = 0;
+    // warp g takes the K blocks g, g + 4, ... of the (tile, K block) order, each into the ring slot
+    // its number falls on; it writes chunks CPW part .. CPW part + CPW - 1 (of 8 per row)
+    const int g = (warp - RL::GATHER0) % NS_GATHER, part = 0;
     constexpr int CPW = 8;
     constexpr int GW = RL::GW > 0 ? RL::GW : 1;
     const bool linear = ps.tab == nullptr;
@@ -357,15 +383,16 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         srow[q] = ps.src + r * ps.src_stride + (mv ? ((long long)y0[q] * ps.Ws + x0[q]) * ps.Cps : 0);
       }
       for (int kb = 0; kb < nkb; ++kb, ++seq) {
-        if ((int)(seq % NS) != g) continue;
+        if ((int)(seq % NS_GATHER) != g) continue;
+        const uint32_t slot = seq % (uint32_t)NS;
         int okw = 1;
-        if (lane == 0) okw = lt_wait(&empty[g], ((seq / NS) & 1) ^ 1, abort, cx.status) ? 1 : 0;
+        if (lane == 0) okw = lt_wait(&empty[slot], ((seq / (uint32_t)NS) & 1) ^ 1, abort, cx.status) ? 1 : 0;
         okw = __shfl_sync(0xffffffffu, okw, 0);
         if (!okw) {
           ok = false;
           break;
         }
-        uint8_t* stage = sA + g * 16384;
+        uint8_t* stage = sA + slot * 16384;
         // 4 chunks (of 4 rows each) in flight at a time: 16 loads of 16 bytes per lane
 #pragma unroll
         for (int c0 = 0; c0 < CPW; c0 += 4) {
@@ -393,7 +420,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         }
         fence_proxy_async();   // generic-proxy stores of the stage, before the MMA reads it
         __syncwarp();
-        if (lane == 0) mbar_arrive(&full[g]);
+        if (lane == 0) mbar_arrive(&full[slot]);
       }
     }
   } else {
@@ -413,238 +440,361 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
     for (long long tile = blockIdx.x + (long long)eg * gridDim.x; eg < ngrp && tile < ntiles;
          tile += (long long)ngrp * gridDim.x, accseq += ngrp) {
       const int buf = eg;
-      const int nt = (int)(tile % ps.ntn);
-      const long long m = tile / ps.ntn * 128 + 32 * q4 + lane;
-      const bool mv = m < M;
-      const int rl = mv ? (int)(m / ps.Pm) : 0;              // row within the chunk
-      const int pp = mv ? (int)(m - (long long)rl * ps.Pm) : 0;
-      const int pi = pp / ps.nJ, pj = pp - (pp / ps.nJ) * ps.nJ;
+      // (fewer than 2^31 positions a launch: the rows of a chunk are bounded by its 16 GB)
+      const uint32_t mt = ps.dntn((uint32_t)tile);
+      const int nt = (int)((uint32_t)tile - mt * ps.dntn.d);
+      const uint32_t m = mt * 128 + 32 * q4 + lane;
+      const bool mv = m < (uint32_t)M;
+      const int rl = mv ? (int)ps.dPm(m) : 0;                 // row within the chunk
+      const int pp = mv ? (int)(m - (uint32_t)rl * ps.dPm.d) : 0;
+      const int pi = (int)ps.dnJ((uint32_t)pp), pj = pp - pi * ps.nJ;
       const int pm = ps.npos ? 0 : (ps.oa + ps.os * pi) * ps.Wo + ps.ob + ps.os * pj;
       // the row: subdomain b, spec k, property p (one 16-byte load of the row table)
       const int r = cx.r0 + rl;
-      const int b = r / cx.K;
+      const int b = (int)cx.dK((uint32_t)r);
       const int4 ri = mv ? cx.rowinfo[r] : make_int4(0, 0, 0, 0);
+      int s0 = 0, s1 = 0;
+      if (mv && MODE != EPI_CONCRETIZE) {
+        const int* sl = cx.slayer + (size_t)b * (cx.L + 1) + ps.layer;
+        s0 = b * BCROWN_MAX_SPLITS + sl[0];
+        s1 = b * BCROWN_MAX_SPLITS + sl[1];
+      }
       const long long abase = ((long long)(uint32_t)ri.y << 32) | (uint32_t)ri.x;
       const long long bbase = ri.z;
       const int prop = ri.w & 0x7FFFFFFF;
       const bool rv = mv && (ri.w < 0);
-      // the row's splits in this layer that fall on this thread's elements of the tile
-      // kept splits, packed: n | t << 20 | (S == +1) << 27 (n < 2^20, t < 64); -1: none
-      int kp_[MAX_KEEP];
-#pragma unroll
-      for (int q = 0; q < MAX_KEEP; ++q) kp_[q] = -1;
-      int nkeep = 0;
-      bool many = false;
-      int s0 = 0, s1 = 0;
-      const int nlo = nt * Np, nhi = min(nt * Np + Np, ps.N);
-      if (rv && MODE != EPI_CONCRETIZE) {
-        const int* sl = cx.slayer + (size_t)b * (cx.L + 1) + ps.layer;
-        s0 = b * BCROWN_MAX_SPLITS + sl[0];
-        s1 = b * BCROWN_MAX_SPLITS + sl[1];
-        for (int q = s0; q < s1; ++q) {
-          const uint32_t e = cx.ssplit[q];
-          const int jn = sp_j(e);
-          const int c_s = jn / ps.HWo, p_s = jn - c_s * ps.HWo;
-          const int nn = ps.npos ? p_s * ps.Cpo + c_s : c_s;   // the element's n
-          const bool mine = nn >= nlo && nn < nhi && (ps.npos || p_s == pm);
-          if (!mine) continue;
-          // register slot nkeep (constant indices keep the arrays in registers)
-#pragma unroll
-          for (int u = 0; u < MAX_KEEP; ++u)
-            if (u == nkeep) {
-              kp_[u] = nn | (sp_t(e) << 20) | ((sp_s(e) == 1 ? 1 : 0) << 27);
-            }
-          if (nkeep < MAX_KEEP) ++nkeep;
-          else many = true;
+      const int nlo = nt * Np;
+      // the row's splits in this layer: element n and position of an entry (n: the NHWC index of a
+      // fully connected pass over a map, whose one position stands for all)
+      auto place = [&](uint32_t e, int& n, int& p) {
+        const int jn = sp_j(e);
+        const int c = (int)ps.dHWo((uint32_t)jn);
+        p = jn - c * ps.HWo;
+        n = c;
+        if (ps.npos) n += p * ps.Cpo, p = 0;
+      };
+      const int pos_here = ps.npos ? 0 : pm;
+      int nsplit = 0;
+      if constexpr (MODE != EPI_CONCRETIZE) {
+        nsplit = rv ? s1 - s0 : 0;
+        __syncwarp();
+        if (warp_sum_ok) {   // one row per warp: the lanes place its entries once, for all
+          nsplit = __shfl_sync(0xffffffffu, nsplit, 0);
+          const int f = __shfl_sync(0xffffffffu, s0, 0);
+          for (int q = lane; q < nsplit; q += 32) {
+            const uint32_t e = cx.ssplit[f + q];
+            int n, p;
+            place(e, n, p);
+            slist[warp].split[q] = make_int2((int)e, n | p << 9);
+          }
         }
       }
+      // entry q of this thread's row
+      auto split_at = [&](int q, int& n, int& p) -> uint32_t {
+        if (warp_sum_ok) {
+          const int2 x = slist[warp].split[q];
+          n = x.y & 511;
+          p = (int)((uint32_t)x.y >> 9);
+          return (uint32_t)x.x;
+        }
+        const uint32_t e = cx.ssplit[s0 + q];
+        place(e, n, p);
+        return e;
+      };
       int okw = 1;
-      if (lane == 0) okw = lt_wait(&acc_full[buf], (accseq / (uint32_t)ngrp) & 1, abort, cx.status) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw) break;
-      tc_fence_after();
+      if constexpr (MODE == EPI_CONCRETIZE) {
+        if (lane == 0) okw = lt_wait(&acc_full[buf], (accseq / (uint32_t)ngrp) & 1, abort, cx.status) ? 1 : 0;
+        okw = __shfl_sync(0xffffffffu, okw, 0);
+        if (!okw) break;
+        tc_fence_after();
+      }
       float acc = 0.f;
-      // per-tile bases: the row's alpha block (and stash, gradient), the property's tables
-      const float* alpha_r = cx.alpha + abase;
-      __nv_bfloat16* stash_r = cx.stash ? cx.stash + abase : nullptr;
-      float* dalpha_r = cx.dalpha ? cx.dalpha + abase : nullptr;
-      const float2* chord_p = cx.chord + (size_t)prop * cx.H;
-      const uint32_t* tab_p = MODE == EPI_CONCRETIZE ? nullptr : ps.ntab + (size_t)prop * cx.NH;
-      // the chunk's NHWC index: conv, (pm, channels nb ..); fully connected over a map, nb itself
-      auto nhwc = [&](int nb) -> long long { return ps.npos ? (long long)nb : (long long)pm * ps.Cpo + nb; };
-      // the neuron entries of a chunk are loaded one chunk ahead, so that the dependent loads of
-      // the unstable elements' operands do not wait for them as well
-      // (not in the adjoint epilogue unless LT_FWD_PREFETCH: its registers are at the limit, and
-      // the spills it then needs cost more than the prefetch gains: 3.03k against 3.12k subdomains/s)
-      constexpr bool PF = MODE == EPI_RELAX || (MODE == EPI_FWD && LT_FWD_PREFETCH);
-      uint4 tn0 = make_uint4(0, 0, 0, 0), tn1 = tn0;
-      if (PF && mv && nlo < ps.N) {
-        const uint4* tp = reinterpret_cast<const uint4*>(tab_p + nhwc(nlo));
-        tn0 = tp[0], tn1 = tp[1];
-      }
-      for (int n0 = 0; n0 < Np; n0 += 8) {
-        // 8 columns per step (one 16-byte chunk of the BF16 NHWC output): the element loop's
-        // registers fit the 96 a thread has at 18 warps per SM
-        uint4 t0 = tn0, t1 = tn1;
-        if (PF && mv && n0 + 8 < Np && nlo + n0 + 8 < ps.N) {
-          const uint4* tp = reinterpret_cast<const uint4*>(tab_p + nhwc(nlo + n0 + 8));
-          tn0 = tp[0], tn1 = tp[1];
-        }
-        if (!PF && MODE != EPI_CONCRETIZE && mv && nlo + n0 < ps.N) {
-          const uint4* tp = reinterpret_cast<const uint4*>(tab_p + nhwc(nlo + n0));
-          t0 = tp[0], t1 = tp[1];
-        }
-        float v[8];
-        tmem_ld8(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(buf * Np + n0), v);
-        const int nb = nlo + n0;   // first n of the chunk
-        if (mv && nb < ps.N) {
-        uint32_t o2[4];            // the chunk's results, packed in BF16 pairs
-        const long long nn0 = nhwc(nb);
-        const int lim = ps.npos ? ps.N : ps.Cpo;   // elements of the chunk that exist in the map
-        if (MODE == EPI_CONCRETIZE) {
-          float o[8];
+      const uint32_t tacc = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(buf * Np);
+      __nv_bfloat16* dst_r = ps.dst ? ps.dst + (long long)rl * ps.dst_stride : nullptr;
+      // the NHWC index of element n of this thread's position (fully connected over a map: n itself)
+      const long long nhwc0 = ps.npos ? 0 : (long long)pm * ps.Cpo;
+      if constexpr (MODE == EPI_CONCRETIZE) {
+        for (int n0 = 0; n0 < Np; n0 += 8) {
+          float v[8];
+          tmem_ld8(tacc + n0, v);
+          const int nb = nlo + n0;   // first n of the chunk
+          if (mv && nb < ps.N) {
+            float o[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int n = nb + e;
-            o[e] = 0.f;
-            if (!rv || n >= ps.Co) continue;
-            const int jl = n * ps.HWo + pm;   // input coordinate (channel-major)
-            const float a = v[e];
-            const float xl = cx.x_lo[(size_t)prop * cx.d0 + jl], xh = cx.x_hi[(size_t)prop * cx.d0 + jl];
-            acc += fminf(a * xl, a * xh);
-            o[e] = a >= 0.f ? xl : xh;   // x* minimises A^(0) x over the box
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) o2[e] = pack2(o[2 * e], o[2 * e + 1]);
-        } else {
-          // the 8 elements' neuron entries (loaded with the previous chunk)
-          uint32_t ent[8];
-          ent[0] = t0.x, ent[1] = t0.y, ent[2] = t0.z, ent[3] = t0.w;
-          ent[4] = t1.x, ent[5] = t1.y, ent[6] = t1.z, ent[7] = t1.w;
-          // elements of the chunk with a split of the row (all of them when the row's list overflowed)
-          uint32_t smask = many ? 0xFFu : 0u;
-          if (nkeep > 0) {   // most threads hold no split in the tile: skip the scan
-#pragma unroll
-            for (int q = 0; q < MAX_KEEP; ++q)
-              if (q < nkeep && (unsigned)((kp_[q] & 0xFFFFF) - nb) < 8u) smask |= 1u << ((kp_[q] & 0xFFFFF) - nb);
-          }
-          float o[8];
-#pragma unroll
-          for (int hb = 0; hb < 8; hb += 4) {
-            // the unstable elements' operands of 4 elements, issued together before any is used:
-            // alpha, the chord and, in the adjoint, the stash
-            float al[4], st[4], bv[4];
-            float2 ch[4];
-#pragma unroll
-            for (int uu = 0; uu < 4; ++uu) {
-              const int u = hb + uu;
-              const bool un = rv && nb + u < lim && (ent[u] & 3u) == CODE_UNSTABLE;
-              const int rk = (int)(ent[u] >> 2);
-              al[uu] = un ? alpha_r[rk] : 0.f;
-              ch[uu] = un ? chord_p[rk] : make_float2(0.f, 0.f);
-              st[uu] = (MODE == EPI_FWD && un) ? __bfloat162float(stash_r[rk]) : 0.f;
-              // biases: a conv layer's are per channel (shared memory, up to MAX_NP channels); a
-              // fully connected pass's per n, and a wider layer's channels from global memory
-              if (MODE != EPI_FWD || !sb_smem)
-                bv[uu] = ps.npos ? ps.bnhwc[nn0 + u]
-                                 : (sb_smem ? sbias[min(nb + u, MAX_NP - 1)] : (nb + u < lim ? ps.bnhwc[nb + u] : 0.f));
+            for (int e = 0; e < 8; ++e) {
+              const int n = nb + e;
+              o[e] = 0.f;
+              if (!rv || n >= ps.Co) continue;
+              const int jl = n * ps.HWo + pm;   // input coordinate (channel-major)
+              const float a = v[e];
+              const float xl = cx.x_lo[(size_t)prop * cx.d0 + jl], xh = cx.x_hi[(size_t)prop * cx.d0 + jl];
+              acc += fminf(a * xl, a * xh);
+              o[e] = a >= 0.f ? xl : xh;   // x* minimises A^(0) x over the box
             }
-            if (MODE == EPI_FWD && sb_smem) {
-              // the adjoint: 4 channel biases in one shared-memory load (nb + hb + 3 < MAX_NP); in the
-              // relaxation the 4 registers this holds at once would spill
-              const float4 b4 = *reinterpret_cast<const float4*>(sbias + nb + hb);
-              bv[0] = b4.x, bv[1] = b4.y, bv[2] = b4.z, bv[3] = b4.w;
-            }
+            if (dst_r && nb + 8 <= (ps.npos ? ps.N : ps.Cpo))
+              *reinterpret_cast<uint4*>(dst_r + nhwc0 + nb) =
+                  make_uint4(pack2(o[0], o[1]), pack2(o[2], o[3]), pack2(o[4], o[5]), pack2(o[6], o[7]));
+          }
+        }
+      } else {
+        // Most neurons are stable and unsplit and need no load of their own: 8 columns at a time
+        // they take D = 1 or 0 from bit masks.  The special ones (unstable or split; 5 to 35 % on the
+        // convolutional maps) leave their value in the warp's list, whose entries the 32 lanes then
+        // share out evenly, 4 each at a time, whichever position they lie at; each overwrites its
+        // element of the output.  The list's order is known from the masks before the accumulator is
+        // complete, so the first 4 entries' ranks are loaded during that wait and their alpha, chord
+        // and stash during the pass over the columns: what bounds this kernel is the latency of
+        // those dependent loads.  A split element is worked off by its own lane.  Measured on the
+        // CIFAR-shaped 4-conv network at 9,216 rows, bound and gradient: 14.2 ms with one pass over
+        // all elements, the special ones' loads predicated (71 instructions an element); 14.8 with a
+        // list per lane, which waits for the longest one's loads; 8.7 with this.
+        LtList& wl = slist[warp];
+        const long long tofs = (long long)prop * cx.NH + nhwc0;   // the position's neurons in the tables
+        const int lim = ps.npos ? ps.N : ps.Cpo;                  // elements that exist in the map
+        __syncwarp();
+        {
+          const long long dofs = (long long)rl * ps.dst_stride + nhwc0;
+          wl.row[lane][0] = make_int4(ri.x, ri.y, (int)(uint32_t)tofs, (int)(tofs >> 32));
+          wl.row[lane][1] = make_int4((int)(uint32_t)dofs, (int)(dofs >> 32), prop * cx.H, 0);
+        }
+        const bool mvec = ((ps.Cpo | ps.N) & 63) == 0 && !(nlo & 63);   // 64 columns' masks in one 16-byte load
+        bool waited = false;
+        for (int cb = 0; cb < Np && okw; cb += 64) {
+          const int nb0 = nlo + cb, wid = min(64, Np - cb);
+          // the block's active and unstable bits
+          uint32_t w[4] = {0u, 0u, 0u, 0u};
+          if (rv && mvec && nb0 < lim) {
+            const uint4 x = *reinterpret_cast<const uint4*>(ps.mtab + (tofs + nb0) / 8);
+            w[0] = x.x, w[1] = x.y, w[2] = x.z, w[3] = x.w;
+          } else if (rv) {
 #pragma unroll
-            for (int uu = 0; uu < 4; ++uu) {
-              const int u = hb + uu;
-              const int n = nb + u;
-              const bool valid = rv && n < lim;
-              const int code = (int)(ent[u] & 3u);
-              const int rk = (int)(ent[u] >> 2);
-              // split of this element (sign s, list position t): rare
-              int s = 0, ts = 0;
-              if (valid && ((smask >> u) & 1u)) {
-                int c = n, p = pm;
-                if (ps.npos) {
-                  p = n / ps.Cpo;
-                  c = n - p * ps.Cpo;
+            for (int c = 0; c < 8; ++c)
+              if (8 * c < wid && nb0 + 8 * c < lim)
+                w[c >> 1] |= (uint32_t)ps.mtab[(tofs + nb0) / 8 + c] << (16 * (c & 1));
+          }
+          const unsigned long long act64 =
+              (unsigned long long)__byte_perm(w[2], w[3], 0x6420) << 32 | __byte_perm(w[0], w[1], 0x6420);
+          unsigned long long spec64 =
+              (unsigned long long)__byte_perm(w[2], w[3], 0x7531) << 32 | __byte_perm(w[0], w[1], 0x7531);
+          unsigned long long split64 = 0;
+          for (int q = 0; q < nsplit; ++q) {
+            int n, p;
+            split_at(q, n, p);
+            if (rv && p == pos_here && (unsigned)(n - nb0) < (unsigned)wid) split64 |= 1ull << (n - nb0);
+          }
+          spec64 |= split64;
+          // 64 columns at once where the list holds their special elements, else 16 at a time
+          const int all = __reduce_add_sync(0xffffffffu, __popcll(spec64));
+          const int sub = all <= CAP ? wid : 16;
+          for (int c0 = 0; c0 < wid && okw; c0 += sub) {
+            const unsigned long long range = (sub == 64 ? ~0ull : ((1ull << sub) - 1ull)) << c0;
+            unsigned long long spec = spec64 & range;
+            const int mine = __popcll(spec);
+            int off = mine;   // exclusive prefix over the lanes
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int y = __shfl_up_sync(0xffffffffu, off, o);
+              if (lane >= o) off += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, off, 31);
+            off -= mine;
+            __syncwarp();   // the list's last use
+            for (int i = off; spec; ++i) {
+              const int bit = __ffsll((long long)spec) - 1;
+              wl.ent[i] = (uint16_t)((cb + bit) | lane << 8 | ((split64 >> bit) & 1ull ? 0x8000 : 0));
+              spec &= spec - 1;
+            }
+            __syncwarp();
+            // entries first + lane + 32 q: their ranks (-1: none, or a split one), then alpha and stash.
+            // (The rows' bases are read from the list again where they are needed: values that live
+            // through the pass over the columns are spilled, and a spilled value's reload misses the
+            // little L1 that the stages leave.)
+            int rk[4];
+            auto ranks = [&](int first) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int i = first + lane + 32 * q;
+                const int en = i < total ? (int)wl.ent[i] : 0x8000;
+                rk[q] = -1;
+                if (!(en & 0x8000)) {
+                  const int4 x = wl.row[en >> 8][0];
+                  const long long t = ((long long)x.w << 32) | (uint32_t)x.z;
+                  rk[q] = (int)(ps.ntab[t + nlo + (en & 255)] >> 2);
                 }
-                const int jl = c * ps.HWo + p;   // neuron of the layer (channel-major)
-#pragma unroll
-                for (int q = 0; q < MAX_KEEP; ++q)
-                  if (q < nkeep && (kp_[q] & 0xFFFFF) == n) {
-                    s = (kp_[q] >> 27) & 1 ? 1 : -1;
-                    ts = (kp_[q] >> 20) & 127;
-                  }
-                if (many && s == 0)
-                  for (int q = s0; q < s1; ++q) {
-                    const uint32_t e2 = cx.ssplit[q];
-                    if (sp_j(e2) == jl) {
-                      s = sp_s(e2);
-                      ts = sp_t(e2);
-                    }
-                  }
               }
-              const bool unst = valid && s == 0 && code == CODE_UNSTABLE;
+            };
+            float al[4];
+            uint32_t st[4];
+            auto operands = [&](int first) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                al[q] = 0.f;
+                st[q] = 0u;
+                if (rk[q] < 0) continue;
+                const int4 x = wl.row[wl.ent[first + lane + 32 * q] >> 8][0];
+                const long long ab = (((long long)x.y << 32) | (uint32_t)x.x) + rk[q];
+                al[q] = cx.alpha[ab];
+                if (MODE == EPI_FWD) st[q] = reinterpret_cast<const uint16_t*>(cx.stash)[ab];
+              }
+            };
+            ranks(0);
+            if (!waited) {
+              if (lane == 0) okw = lt_wait(&acc_full[buf], (accseq / (uint32_t)ngrp) & 1, abort, cx.status) ? 1 : 0;
+              okw = __shfl_sync(0xffffffffu, okw, 0);
+              if (!okw) break;
+              tc_fence_after();
+              waited = true;
+            }
+            uint32_t u[8];
+            __syncwarp();
+            tmem_ld8_issue(tacc + cb + c0, u);
+            operands(0);
+            // the columns
+            int put = off;
+            unsigned long long actr = act64 >> c0, specr = spec64 >> c0;
+#pragma unroll 1
+            for (int n0 = cb + c0; n0 < cb + c0 + sub; n0 += 8) {
+              const int nb = nlo + n0;   // first n of the chunk
+              float v[8];
+              __syncwarp();
+              tmem_wait8(u);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(u[e]);
+              if (n0 + 8 < cb + c0 + sub) tmem_ld8_issue(tacc + n0 + 8, u);
+              // biases: a conv layer's are per channel (shared memory, up to MAX_NP channels); a fully
+              // connected pass's per n, and a wider layer's channels from global memory
+              float4 bx = make_float4(0.f, 0.f, 0.f, 0.f), by = bx;
+              if (sb_smem) {
+                bx = *reinterpret_cast<const float4*>(sbias + nb);
+                by = *reinterpret_cast<const float4*>(sbias + nb + 4);
+              } else if (nb < lim) {
+                bx = *reinterpret_cast<const float4*>(ps.bnhwc + nb);
+                by = *reinterpret_cast<const float4*>(ps.bnhwc + nb + 4);
+              }
+              const float bv[8] = {bx.x, bx.y, bx.z, bx.w, by.x, by.y, by.z, by.w};
+              const uint32_t sp8 = (uint32_t)specr & 255u, ac8 = (uint32_t)actr & ~sp8;
+              actr >>= 8;
+              specr >>= 8;
+              float o[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                if (MODE == EPI_RELAX) {
+                  o[e] = (ac8 >> e) & 1u ? v[e] : v[e] * 0.f;   // (0, or NaN where A is not finite)
+                  acc = fmaf(o[e], bv[e], acc);
+                } else {
+                  v[e] += bv[e];
+                  o[e] = (ac8 >> e) & 1u ? v[e] : 0.f;
+                }
+                if ((sp8 >> e) & 1u) wl.val[put++] = v[e];
+              }
+              if (dst_r && mv && nb + 8 <= lim)
+                // the chunk's elements are contiguous in the NHWC output
+                *reinterpret_cast<uint4*>(dst_r + nhwc0 + nb) = make_uint4(
+                    rv ? pack2(o[0], o[1]) : 0u, rv ? pack2(o[2], o[3]) : 0u, rv ? pack2(o[4], o[5]) : 0u,
+                    rv ? pack2(o[6], o[7]) : 0u);
+            }
+            if (cb + c0 + sub == Np) {   // the accumulator has been read: the next tile may take it
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            }
+            __syncwarp();
+            // the special elements, shared out over the lanes
+#pragma unroll 1
+            for (int first = 0; first < total; first += 128) {
+              if (first > 0) {
+                ranks(first);
+                operands(first);
+              }
+              float2 ch[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                ch[q] = make_float2(0.f, 0.f);
+                if (rk[q] >= 0) ch[q] = cx.chord[wl.row[wl.ent[first + lane + 32 * q] >> 8][1].z + rk[q]];
+              }
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (rk[q] < 0) continue;
+                const int i = first + lane + 32 * q, en = wl.ent[i], n = nlo + (en & 255);
+                const float a = wl.val[i];
+                const int4 rw = wl.row[en >> 8][0];
+                const long long ab = (((long long)rw.y << 32) | (uint32_t)rw.x) + rk[q];
+                float out;
+                if (MODE == EPI_RELAX) {
+                  const float bn = sb_smem ? sbias[n] : ps.bnhwc[n];
+                  const bool pos = a >= 0.f;
+                  const float D = pos ? __saturatef(al[q]) : ch[q].x, lm = pos ? 0.f : ch[q].y;
+                  if (cx.stash) cx.stash[ab] = bf16_signed(a);
+                  out = a * D;
+                  const float c = fmaf(out, bn, a * lm);
+                  if (warp_sum_ok) acc += c;   // every lane's position lies in the same row
+                  else wl.val[i] = c;
+                } else {   // a holds zhat
+                  const float A = __uint_as_float(st[q] << 16);
+                  const bool pos = A >= 0.f;
+                  out = pos ? __saturatef(al[q]) * a : fmaf(ch[q].x, a, ch[q].y);
+                  cx.dalpha[ab] = pos ? A * a : 0.f;
+                }
+                if (ps.dst) {
+                  const int4 x = wl.row[en >> 8][1];
+                  const long long t = ((long long)x.y << 32) | (uint32_t)x.x;
+                  ps.dst[t + n] = __float2bfloat16_rn(out);
+                }
+              }
+            }
+            if (MODE == EPI_RELAX && !warp_sum_ok) {
+              // each lane adds up its own row's terms, in order
+              __syncwarp();
+              unsigned long long mask = spec64 & range;
+              for (int i = off; mask; ++i) {
+                const int bit = __ffsll((long long)mask) - 1;
+                if (!((split64 >> bit) & 1ull)) acc += wl.val[i];
+                mask &= mask - 1;
+              }
+            }
+            // split elements: rare, by their own lane
+            unsigned long long todo = split64 & range;
+            while (todo) {
+              const int bit = __ffsll((long long)todo) - 1;
+              todo &= todo - 1;
+              const int n = nb0 + bit;
+              const float a = wl.val[off + __popcll(spec64 & range & ((1ull << bit) - 1ull))];
+              const uint32_t ent = ps.ntab[tofs + n];
+              const int code = (int)(ent & 3u), rank = (int)(ent >> 2);
+              int s = 0, ts = 0;   // its sign and list position (the last entry, as everywhere)
+              for (int q = 0; q < nsplit; ++q) {
+                int n2, p2;
+                const uint32_t e = split_at(q, n2, p2);
+                if (p2 == pos_here && n2 == n) {
+                  s = sp_s(e);
+                  ts = sp_t(e);
+                }
+              }
+              const long long bi = bbase + ts;
+              if (bi >= cx.n_beta) atomicCAS(cx.status, 0, BCROWN_ERR_ARG);
+              float out;
               if (MODE == EPI_RELAX) {
-                const float a = v[u];
-                float D = code == CODE_ACTIVE ? 1.f : 0.f, lm = 0.f, bs = 0.f;
-                if (unst) {
-                  if (a >= 0.f) {
-                    D = __saturatef(al[uu]);
-                  } else {
-                    D = ch[uu].x;
-                    lm = ch[uu].y;
-                  }
-                  if (stash_r) stash_r[rk] = bf16_signed(a);
-                }
-                if (s != 0) {
-                  D = s == -1 ? 1.f : 0.f;
-                  const long long bi = bbase + ts;
-                  if (bi < cx.n_beta) bs = fmaxf(cx.beta[bi], 0.f) * (float)s;
-                  else atomicCAS(cx.status, 0, BCROWN_ERR_ARG);
-                }
-                const float L = valid ? fmaf(a, D, bs) : 0.f;
-                acc = fmaf(L, bv[uu], fmaf(valid ? a : 0.f, lm, acc));
-                o[u] = L;
-              } else {   // EPI_FWD
-                const float z = v[u] + bv[uu];
-                float hv = code == CODE_ACTIVE ? z : 0.f;
-                if (unst) {
-                  if (st[uu] >= 0.f) {
-                    hv = __saturatef(al[uu]) * z;
-                    dalpha_r[rk] = st[uu] * z;
-                  } else {
-                    hv = fmaf(ch[uu].x, z, ch[uu].y);
-                    dalpha_r[rk] = 0.f;
-                  }
-                }
-                if (s != 0) {
-                  const long long bi = bbase + ts;
-                  if (bi < cx.n_beta) cx.dbeta[bi] = (float)s * z;
-                  else atomicCAS(cx.status, 0, BCROWN_ERR_ARG);
-                  hv = s == -1 ? z : 0.f;
-                  // a split unstable neuron keeps its alpha slot, which the bound does not use
-                  if (code == CODE_UNSTABLE) dalpha_r[rk] = 0.f;
-                }
-                o[u] = valid ? hv : 0.f;
+                const float bn = sb_smem ? sbias[n] : ps.bnhwc[n];
+                const float bs = bi < cx.n_beta ? fmaxf(cx.beta[bi], 0.f) * (float)s : 0.f;
+                out = fmaf(a, s == -1 ? 1.f : 0.f, bs);
+                acc = fmaf(out, bn, acc);
+              } else {
+                if (bi < cx.n_beta) cx.dbeta[bi] = (float)s * a;
+                out = s == -1 ? a : 0.f;
+                // a split unstable neuron keeps its alpha slot, which the bound does not use
+                if (code == CODE_UNSTABLE) cx.dalpha[abase + rank] = 0.f;
               }
+              if (dst_r) dst_r[nhwc0 + n] = __float2bfloat16_rn(out);
             }
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) o2[u] = pack2(o[2 * u], o[2 * u + 1]);
         }
-        if (ps.dst && nb + 8 <= lim) {
-          // the chunk's elements are contiguous in the NHWC output
-          *reinterpret_cast<uint4*>(ps.dst + (long long)rl * ps.dst_stride + nn0) =
-              make_uint4(o2[0], o2[1], o2[2], o2[3]);
-        }
-        }
+        if (!okw) break;
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[buf]);
+      if (MODE == EPI_CONCRETIZE) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+      }
       if (MODE != EPI_FWD) {
         // partial sum of c for (row, this thread's positions and columns); a fixed slot each
         if (warp_sum_ok) {
@@ -813,26 +963,42 @@ __global__ void __launch_bounds__(256) k_lt_lb(Ctx cx, const float* __restrict__
   }
 }
 
-// The neurons of one hidden layer in NHWC order per property, so that an epilogue reads 16
-// channels' entries with four 16-byte loads: code (0 inactive, 1 active, 2 unstable) | rank << 2;
-// and the upper chord of each unstable neuron by rank.
+// The neurons of one hidden layer in NHWC order per property: code (0 inactive, 1 active, 2 unstable)
+// | rank << 2 per neuron, the active and the unstable bits of each 8 of them, and the upper chord of
+// each unstable neuron by rank.  One thread per (property, 8 channels, position); neighbouring threads
+// take neighbouring positions, so the channel-major tables are read in order.
 __global__ void k_lt_ntab(int P, long long H, long long hoff, int C, int HW, int Cp, long long NH, long long off,
-                          Tables tb, uint32_t* __restrict__ ntab, float2* __restrict__ chord) {
+                          Tables tb, uint32_t* __restrict__ ntab, uint16_t* __restrict__ mtab,
+                          float2* __restrict__ chord) {
   const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long d = (long long)C * HW;
-  if (id >= (long long)P * d) return;
-  const int p = (int)(id / d);
-  const int j = (int)(id - (long long)p * d);
-  const int c = j / HW, pos = j - c * HW;
-  const size_t n = (size_t)p * H + hoff + j;
-  const uint32_t code = tb.code[n];
-  const int rk = tb.rank[n];
-  ntab[(size_t)p * NH + off + (size_t)pos * Cp + c] = code | ((uint32_t)max(rk, 0) << 2);
-  if (code == CODE_UNSTABLE && rk >= 0) chord[(size_t)p * H + rk] = make_float2(tb.slope[n], tb.icpt[n]);
+  const long long per = (long long)(Cp / 8) * HW;
+  if (id >= (long long)P * per) return;
+  const int p = (int)(id / per);
+  const int rem = (int)(id - (long long)p * per);
+  const int c8 = rem / HW, pos = rem - c8 * HW;
+  uint32_t ent[8], act = 0, uns = 0;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int c = 8 * c8 + e;
+    ent[e] = 0;
+    if (c >= C) continue;
+    const size_t n = (size_t)p * H + hoff + (size_t)c * HW + pos;
+    const uint32_t code = tb.code[n];
+    const int rk = tb.rank[n];
+    ent[e] = code | ((uint32_t)max(rk, 0) << 2);
+    act |= (code == CODE_ACTIVE ? 1u : 0u) << e;
+    uns |= (code == CODE_UNSTABLE ? 1u : 0u) << e;
+    if (code == CODE_UNSTABLE && rk >= 0) chord[(size_t)p * H + rk] = make_float2(tb.slope[n], tb.icpt[n]);
+  }
+  const size_t o = (size_t)p * NH + off + (size_t)pos * Cp + 8 * c8;
+  *reinterpret_cast<uint4*>(ntab + o) = make_uint4(ent[0], ent[1], ent[2], ent[3]);
+  *reinterpret_cast<uint4*>(ntab + o + 4) = make_uint4(ent[4], ent[5], ent[6], ent[7]);
+  mtab[o / 8] = (uint16_t)(act | uns << 8);
 }
 
-inline int lt_smem(int Np) {
-  return 1024 + NS * (16384 + Np * 128) + 256 + (MAX_KP / 8) * (int)sizeof(int2) + MAX_NP * (int)sizeof(float);
+inline int lt_smem(bool ta, int Np) {
+  return 1024 + lt_stages(ta, Np) * (16384 + Np * 128) + 256 + (MAX_KP / 8) * (int)sizeof(int2) +
+         MAX_NP * (int)sizeof(float) + (ta ? LtRoles<true>::EPI : LtRoles<false>::EPI) * (int)sizeof(LtList);
 }
 
 }  // namespace lt
@@ -862,6 +1028,10 @@ MapDims map_of(const bcrown_net* net, int l) {
   m.Cp = pad_to(m.C, 8);
   return m;
 }
+
+// Entries of a map in the NHWC neuron tables: a multiple of 64, so that 64 neurons' masks are 16-byte
+// aligned, and at least 8 beyond the map.
+long long nhwc_elems(const MapDims& m) { return ((long long)m.HW() * m.Cp + 8 + 63) / 64 * 64; }
 
 // One prepared GEMM of a layer: B matrix rows [brow, brow + ntn * Np) of the layer's weight map,
 // the gather table, and the pass geometry except the per-call pointers.
@@ -959,9 +1129,9 @@ int prepare(bcrown_net* net, LtNet* t) {
     BC_CHECK(upload(t, bn.data(), bn.size() * 4, &d));
     t->bnhwc[l] = reinterpret_cast<float*>(d);
     t->nhwc_off[l] = nh;
-    nh += (long long)m.HW() * m.Cp;
+    nh += nhwc_elems(m);
   }
-  t->NH = nh + 16;
+  t->NH = nh;
   const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
   int slot = 1;   // slot 0: the top relaxation
   for (int i = L - 1; i >= 1; --i) {
@@ -1042,7 +1212,9 @@ int prepare(bcrown_net* net, LtNet* t) {
           q.N = mo.C;
           q.Np = Np;
           q.ntn = ntn;
-          q.nkb = kp / 64;
+          // the phase's own taps (a stride-2 3x3 layer's phases have 1, 2, 2 and 4)
+          const int kph = std::max(64, pad_to(py.nk * px.nk * mi.Cp, 64));
+          q.nkb = kph / 64;
           q.brow = ph * Np;
           q.Hs = mi.H;
           q.Ws = mi.W;
@@ -1050,7 +1222,7 @@ int prepare(bcrown_net* net, LtNet* t) {
           q.ms = 1;
           q.cy = py.off;
           q.cx = px.off;
-          q.kchunks = kp / 8;
+          q.kchunks = kph / 8;
           q.oa = a;
           q.ob = bb;
           q.os = s;
@@ -1063,7 +1235,7 @@ int prepare(bcrown_net* net, LtNet* t) {
           q.hoff = i >= 2 ? net->hoff[i - 2] : 0;
           q.bias = i >= 2 ? net->ly[i - 2].b : nullptr;
           q.bnhwc = i >= 2 ? t->bnhwc[i - 1] : nullptr;
-          std::vector<int2> tab((size_t)kp / 8, kNoChunk);
+          std::vector<int2> tab((size_t)kph / 8, kNoChunk);
           for (int dy = 0; dy < py.nk; ++dy)
             for (int dx = 0; dx < px.nk; ++dx) {
               const int tap = dy * px.nk + dx;
@@ -1222,14 +1394,17 @@ int prepare(bcrown_net* net, LtNet* t) {
     BC_CHECK(upload(t, wd.data(), wd.size() * sizeof(int), &d));
     t->width = reinterpret_cast<int*>(d);
   }
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_RELAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lt_smem(MAX_NP)));
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_CONCRETIZE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lt_smem(MAX_NP)));
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_FWD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lt_smem(MAX_NP)));
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_RELAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lt_smem(MAX_NP)));
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_CONCRETIZE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lt_smem(MAX_NP)));
-  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_FWD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lt_smem(MAX_NP)));
+  int smem_g = 0, smem_t = 0;
+  for (int np = 16; np <= MAX_NP; np += 16) {
+    smem_g = std::max(smem_g, lt_smem(false, np));
+    smem_t = std::max(smem_t, lt_smem(true, np));
+  }
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_RELAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_CONCRETIZE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_FWD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_RELAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_t));
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_CONCRETIZE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_t));
+  BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_FWD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_t));
   t->ready = true;
   return BCROWN_OK;
 }
@@ -1240,9 +1415,14 @@ int launch_pass(bcrown_net* net, const CUtensorMap& mB, Pass q, int mode, const 
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  q.dPm.set(q.Pm);
+  q.dnJ.set(q.nJ);
+  q.dntn.set(q.ntn);
+  q.dHWo.set(q.HWo);
+  q.dCpo.set(q.Cpo);
   const long long ntiles = (q.M + 127) / 128 * q.ntn;
   const int grid = (int)std::min<long long>(ntiles, sms);
-  const int smem = lt_smem(q.Np);
+  const int smem = lt_smem(q.ta != 0, q.Np);
   ProfScope pr(net, BCROWN_PROF_LAYER_GEMM, s);
   // the A operand's map for this launch (the source buffer and the rows of this chunk)
   CUtensorMap mA = mB;   // unused by the gathering kernel
@@ -1322,15 +1502,16 @@ bool lt_supported(const bcrown_net* net) {
 size_t lt_workspace_bytes(const bcrown_net* net, int R, int P, int64_t n_alpha, bool grad) {
   long long act, S, Rc;
   plan_sizes(net, R, &act, &S, &Rc);
-  long long nh = 16;
+  long long nh = 0;
   for (int l = 1; l <= net->L - 1; ++l) {
     const MapDims m = map_of(net, l);
-    nh += (long long)m.HW() * m.Cp;
+    nh += nhwc_elems(m);
   }
   const size_t B = (size_t)R / std::max(net->K, 1);
   size_t bytes = align_up((size_t)Rc * act * 2) * 2 + align_up((size_t)Rc * S * 4);
   bytes += align_up((size_t)R * 16) + align_up(B * BCROWN_MAX_SPLITS * 4) + align_up(B * (net->L + 1) * 4);
-  bytes += align_up((size_t)std::max(P, 1) * nh * 4) + align_up((size_t)std::max(P, 1) * std::max(net->H, 1) * 8);
+  bytes += align_up((size_t)std::max(P, 1) * nh * 4) + align_up((size_t)std::max(P, 1) * nh / 4) +
+           align_up((size_t)std::max(P, 1) * std::max(net->H, 1) * 8);
   if (grad) bytes += align_up((size_t)std::max<int64_t>(n_alpha, 1) * 2);
   return bytes;
 }
@@ -1357,11 +1538,13 @@ int lt_bound(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* bt, 
   uint32_t* ssplit = ar.take<uint32_t>((size_t)bt->B * BCROWN_MAX_SPLITS);
   int* slayer = ar.take<int>((size_t)bt->B * (L + 1));
   uint32_t* ntab = ar.take<uint32_t>((size_t)dom->n_props * t->NH);
+  uint16_t* mtab = ar.take<uint16_t>((size_t)dom->n_props * t->NH / 8);
   float2* chord = ar.take<float2>((size_t)dom->n_props * std::max(net->H, 1));
   __nv_bfloat16* stash = grad ? ar.take<__nv_bfloat16>((size_t)std::max<int64_t>(bt->n_alpha, 1)) : nullptr;
   if (ar.off > ws_bytes) return fail(BCROWN_ERR_OOM, "layer path: workspace plan");
   Ctx cx;
   cx.K = K;
+  cx.dK.set(K);
   cx.P = dom->n_props;
   cx.H = net->H;
   cx.d0 = net->d[0];
@@ -1387,12 +1570,11 @@ int lt_bound(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* bt, 
   cx.NH = t->NH;
   cx.chord = chord;
   // the properties' neurons in NHWC order and their chords by rank, once per call
-  BC_CUDA(cudaMemsetAsync(ntab, 0, (size_t)dom->n_props * t->NH * 4, s));
   for (int l = 1; l <= L - 1; ++l) {
     const MapDims m = map_of(net, l);
-    const long long n = (long long)dom->n_props * m.C * m.HW();
+    const long long n = (long long)dom->n_props * (m.Cp / 8) * m.HW();
     k_lt_ntab<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dom->n_props, net->H, net->hoff[l - 1], m.C, m.HW(), m.Cp,
-                                                         t->NH, t->nhwc_off[l], tb, ntab, chord);
+                                                         t->NH, t->nhwc_off[l], tb, ntab, mtab, chord);
     ++g_launches;
   }
   // the rows' alpha / beta offsets and the subdomains' splits sorted by layer, once per call
@@ -1417,6 +1599,7 @@ int lt_bound(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* bt, 
       for (const PassPrep& pp : P.bwd) {
         Pass q = pp.p;
         q.ntab = i >= 2 ? ntab + t->nhwc_off[i - 1] : nullptr;
+        q.mtab = i >= 2 ? mtab + t->nhwc_off[i - 1] / 8 : nullptr;
         q.src = act[cur];
         q.src_stride = stride;
         q.dst = act[cur ^ 1];
@@ -1436,6 +1619,7 @@ int lt_bound(bcrown_net* net, const bcrown_domain* dom, const bcrown_batch* bt, 
       const LayerPrep& P = t->ly[i];
       Pass q = P.fwd.p;
       q.ntab = ntab + t->nhwc_off[i];
+      q.mtab = mtab + t->nhwc_off[i] / 8;
       q.src = act[cur];
       q.src_stride = stride;
       q.dst = i < L - 1 ? act[cur ^ 1] : nullptr;
