@@ -95,7 +95,8 @@ static_assert(sizeof(Smem<64>) + 1024 <= 232448, "shared memory plan exceeds 227
 
 struct Args {
   int L, K, P, H, R;
-  const int* n_tiles;                 // tiles to process (written by the row planner)
+  int tiles;                          // with one property: its tiles, rows in order (no plan)
+  const int* n_tiles;                 // tiles to process (written by the row planner; null: one property)
   const int* tile_prop;               // [tile] property of every row of the tile
   const int* rowmap;                  // [tile][TR] global row of each slot, -1 when empty
   int d[MAXL + 1];
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
   const uint32_t pad = (1024u - (su32(smem_raw) & 1023u)) & 1023u;
   SM* sm = reinterpret_cast<SM*>(smem_raw + pad);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tiles = *a.n_tiles;
+  const int n_tiles = a.n_tiles ? *a.n_tiles : a.tiles;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSLOT; ++i) {
@@ -441,14 +442,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       // Every row of a tile belongs to one property (the rows are grouped by property before
       // the launch); slots past the property's last row are empty.
-      const int p = a.tile_prop[tile];
+      const int p = a.n_tiles ? a.tile_prop[tile] : 0;
       // ---------------- tile set-up, step 1: per-row scalars (one thread per row)
       if (warp < (TR + 31) / 32) {
         const int row = etid;
         int v = 0, r = -1;
         if (row < TR) {
-          r = a.rowmap[(size_t)tile * TR + row];
+          r = a.n_tiles ? a.rowmap[(size_t)tile * TR + row] : tile * TR + row;
           v = r >= 0 && r < a.R && p >= 0 && p < a.P;
+          if (!a.n_tiles && v && a.bt.prop_of[r / a.K] != 0) {   // (the planner checks the others)
+            atomicCAS(a.status, 0, BCROWN_ERR_ARG);
+            v = 0;
+          }
           int k = 0, cnt = 0, off = 0;
           long long ab = 0, bb = 0;
           if (v) {
@@ -1262,7 +1267,10 @@ static int tc_launch(bcrown_net* net, const bcrown_domain* dom, const bcrown_bat
   carve(ws, B, K, P, net->H, grad, &pl);
   const int tr = tile_rows(B, K, P);
   const long long T = max_tiles_of(B, K, P, tr);
-  if (plan) {
+  // One property: row r is slot r % tr of tile r / tr and no plan is made.  The memset and the four
+  // launches of a plan took 13 us of a 77 us call (16 subdomains of the 784-wide network).
+  const bool single = P == 1;
+  if (plan && !single) {
     BC_CUDA(cudaMemsetAsync(pl.cnt, 0, (size_t)(P + 1) * 4, s));
     const int gb = (int)std::min<long long>((B + 255) / 256, 4096);
     k_plan_count<<<gb, 256, 0, s>>>(B, P, bt->prop_of, pl.cnt, net->status);
@@ -1277,7 +1285,8 @@ static int tc_launch(bcrown_net* net, const bcrown_domain* dom, const bcrown_bat
   A.P = P;
   A.H = net->H;
   A.R = R;
-  A.n_tiles = pl.n_tiles;
+  A.tiles = (int)(((long long)R + tr - 1) / tr);
+  A.n_tiles = single ? nullptr : pl.n_tiles;
   A.tile_prop = pl.tile_prop;
   A.rowmap = pl.rowmap;
   A.stash = pl.stash;
@@ -1301,7 +1310,7 @@ static int tc_launch(bcrown_net* net, const bcrown_domain* dom, const bcrown_bat
   A.n_beta = bt->n_beta;
   A.status = net->status;
   // one CTA per SM at most; the planned tile count (at most T) is read on the device
-  const int grid = (int)std::min<long long>(T, sm_count());
+  const int grid = (int)std::min<long long>(single ? A.tiles : T, sm_count());
   {
     ProfScope ps(net, BCROWN_PROF_FUSED, s);
     if (mode == 2) fused_launch<2>(tr, grid, t->maps, A, s);

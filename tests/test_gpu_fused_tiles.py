@@ -58,3 +58,27 @@ def test_rows_do_not_depend_on_the_tile(widths, n_props):
     # BF16 operands move a bound by a few units of 2^-9 of the magnitudes it sums
     scale = np.maximum(np.abs(ref).max(), 1.0)
     assert np.abs(got[n][0].numpy() - ref).max() <= 2e-2 * scale
+
+
+@pytest.mark.parametrize("B", [5, 700])   # one tile and several
+def test_one_property_needs_no_plan_and_still_refuses_another(B):
+    """With one property the rows stand in the batch's order; a subdomain that names another property is
+    reported and leaves the others' values as they are."""
+    pb = wl.make_problem("single", wl.mlp_layers([30, 96, 64, 3], 4), 1, 0.05, 2, 4)
+    onet, props, unst = oracle_setup(pb)
+    batch = wl.random_batch(pb, unst, B, 0, 6, 3)
+    a, b = wl.random_alpha_beta(batch, 5, 0.5)
+    net = bc.load_net(pb.layers, pb.C)
+    assert bc.path_supported(net, 1)
+    dom = bc.domain_from_host(props["x_lo"], props["x_hi"], props["l"], props["u"])
+    ta, tb = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    lb = bc.bound(net, dom, bc.DeviceBatch.from_host(batch), ta, tb, bc.BF16).reshape(B, -1)
+    assert bc.status(net) == 0
+    prop_of = batch.prop_of.copy()
+    prop_of[B // 2] = 1
+    bad = wl.Batch(prop_of, batch.split_off, batch.split_cnt, batch.split_layer, batch.split_idx, batch.split_sign,
+                   batch.alpha_off, batch.n_alpha, batch.n_beta)
+    got = bc.bound(net, dom, bc.DeviceBatch.from_host(bad), ta, tb, bc.BF16).reshape(B, -1)
+    assert bc.status(net) != 0
+    keep = torch.arange(B) != B // 2
+    assert torch.equal(got[keep.cuda()], lb[keep.cuda()])
