@@ -154,6 +154,18 @@ struct ProfScope {
   ~ProfScope();
 };
 
+// n / d for n < 2^31 by multiplication.
+struct FastDiv {
+  uint32_t d, mul, sh;
+  __host__ void set(uint32_t v) {
+    d = v;
+    sh = 0;
+    while ((1ull << sh) < v) ++sh;
+    mul = (uint32_t)((((1ull << sh) - v) << 32) / v + 1);
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t n) const { return (__umulhi(n, mul) + n) >> sh; }
+};
+
 inline int grid1d(long long n, int block) { return (int)((n + block - 1) / block); }
 
 }  // namespace bcrown

@@ -23,115 +23,183 @@ extern std::atomic<long long> g_launches;
 namespace {
 
 struct SconvPass {
-  long long M;     // rows: R * Pm
+  uint32_t M;      // rows: R * Pm (below 2^31: a chunk's rows hold at least 12 Pm bytes each of 8 GB)
   int Pm, nJ;      // positions per row in this pass, and the pass grid's width
+  FastDiv dPm, dnJ;
   int N, K;        // output channels; terms per output
   int Hs, Ws;      // source map (one channel)
   long long HWs;
   int ms, cy, cx;  // base source position of (i, j): (i ms + cy, j ms + cx)
   int oa, ob, os, Wo;
   long long HWo;   // output position (oa + os i) Wo + ob + os j, channel stride HWo
-  const int4* tab; // [K]: {source offset c HWs + dy Ws + dx, dy, dx, 0}
+  const int4* tab; // [K]: {source offset c HWs + dy Ws + dx, dy, dx, tap = dy nkx + dx of the phase}
   const float* B;  // [K][N] weights
   int ky0, kx0;    // the phase's first tap (B depends on nothing else)
+  int ntap;        // taps of the phase
+};
+// A layer's stride phases, contracted by one launch.
+constexpr int SC_PHASES = 4;
+struct SconvPhases {
+  SconvPass p[SC_PHASES];
 };
 
-constexpr int SC_BM = 128, SC_BK = 16, SC_THREADS = 256;
+// Rows of the output map that a row of the pass belongs to.
+__device__ __forceinline__ long long sc_out(const SconvPass& q, uint32_t m, long long ostride, long long* pos) {
+  const uint32_t rr = q.dPm(m);
+  const int p2 = (int)(m - rr * (uint32_t)q.Pm);
+  const int ii = (int)q.dnJ((uint32_t)p2), jj = p2 - ii * q.nJ;
+  *pos = (long long)(q.oa + q.os * ii) * q.Wo + q.ob + q.os * jj;
+  return (long long)rr * ostride + *pos;
+}
+
+// A 128 x BN tile, 8 x 8 outputs a thread (2 BN threads), FMAs on pairs of neighbouring channels
+// (fma.rn.f32x2, as the GEMM), both operands by cp.async into three stages of 16 K terms: the
+// gathered one in 4-byte pieces (a warp's are one run of positions), zero-filled where a tap falls
+// outside the map.  Bound by the FMA pipe and, for few output channels, by the gather's
+// instructions (each gathered value feeds BN FMAs).  2,997 rows of the 32 -> 64 channel 4x4 stride-2
+// layer backward: 668 us in four launches with 8 x 2 outputs a thread and register staging, 420 now.
+constexpr int SC_BM = 128, SC_BK = 16, SC_STAGES = 3;
+constexpr int SC_AP = SC_BM + 4;
 
 template <int BN>
-__global__ void __launch_bounds__(SC_THREADS) k_sconv(SconvPass q, const float* __restrict__ src, long long sstride,
-                                                      float* __restrict__ out, long long ostride,
-                                                      const float* __restrict__ bias) {
-  constexpr int TN = BN / 16;          // output channels per thread
+__global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const float* __restrict__ src,
+                                                  long long sstride, float* __restrict__ out, long long ostride,
+                                                  const float* __restrict__ bias) {
+  constexpr int NT = 2 * BN;
+  constexpr int RPT = NT >= SC_BM ? 1 : SC_BM / NT;    // tile rows a thread gathers
+  constexpr int KSTEP = NT >= SC_BM ? NT / SC_BM : 1;  // and the stride of its K terms
+  const SconvPass& q = ph.p[blockIdx.z];
+  const uint32_t m0 = blockIdx.x * (uint32_t)SC_BM;
+  if (m0 >= q.M) return;
   extern __shared__ __align__(16) uint8_t sc_raw[];
-  float(*As)[SC_BK][SC_BM + 4] = reinterpret_cast<float(*)[SC_BK][SC_BM + 4]>(sc_raw);
-  float(*Bs)[SC_BK][BN + 4] = reinterpret_cast<float(*)[SC_BK][BN + 4]>(sc_raw + 2 * SC_BK * (SC_BM + 4) * 4);
-  int4* stab = reinterpret_cast<int4*>(sc_raw + 2 * SC_BK * (SC_BM + 4) * 4 + 2 * SC_BK * (BN + 4) * 4);
+  float* As = reinterpret_cast<float*>(sc_raw);                 // [stage][SC_BK][SC_AP]
+  float* Bs = As + SC_STAGES * SC_BK * SC_AP;                   // [stage][SC_BK][BN]
+  int4* stab = reinterpret_cast<int4*>(Bs + SC_STAGES * SC_BK * BN);
   const int tid = threadIdx.x;
-  const int tm = tid & 15, tn = tid >> 4;
-  const long long m0 = (long long)blockIdx.x * SC_BM;
+  const int ty = tid & 15, tx = tid >> 4;
   const int n0 = blockIdx.y * BN;
-  for (int k = tid; k < q.K; k += SC_THREADS) stab[k] = q.tab[k];
-  // the row this thread gathers (fixed across K tiles) and its base source position
-  const long long mg = m0 + (tid & 127);
-  const bool mv = mg < q.M;
-  const long long r = mv ? mg / q.Pm : 0;
-  const int pp = mv ? (int)(mg - r * q.Pm) : 0;
-  const int pi = pp / q.nJ, pj = pp - (pp / q.nJ) * q.nJ;
-  const int y0 = mv ? pi * q.ms + q.cy : -32768, x0 = pj * q.ms + q.cx;
-  const float* srow = src + r * sstride + (mv ? (long long)y0 * q.Ws + x0 : 0);
-  float acc[8][TN];
+  for (int k = tid; k < q.K; k += NT) stab[k] = q.tab[k];
+  // the rows this thread gathers (fixed across K) and their base source positions
+  const float* srow[RPT];
+  int y0[RPT], x0[RPT];
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) {
+    const uint32_t m = m0 + (uint32_t)(tid % SC_BM) + (uint32_t)(u * NT);
+    const bool mv = m < q.M;
+    const uint32_t r = mv ? q.dPm(m) : 0u;
+    const int pp = mv ? (int)(m - r * (uint32_t)q.Pm) : 0;
+    const int pi = (int)q.dnJ((uint32_t)pp), pj = pp - pi * q.nJ;
+    y0[u] = mv ? pi * q.ms + q.cy : -32768;
+    x0[u] = pj * q.ms + q.cx;
+    srow[u] = src + (long long)r * sstride + (mv ? (long long)y0[u] * q.Ws + x0[u] : 0);
+  }
+  const uint32_t sA = (uint32_t)__cvta_generic_to_shared(As), sB = (uint32_t)__cvta_generic_to_shared(Bs);
+  const bool bvec = (q.N & 3) == 0;
+  __syncthreads();
+  auto load = [&](int stage, int k0) {
+    const uint32_t as = sA + (uint32_t)(stage * SC_BK * SC_AP + tid % SC_BM) * 4;
+    const uint32_t bs = sB + (uint32_t)(stage * SC_BK * BN) * 4;
+#pragma unroll
+    for (int kk = tid / SC_BM; kk < SC_BK; kk += KSTEP) {
+      const int k = k0 + kk;
+      const bool kin = k < q.K;
+      const int4 t = stab[kin ? k : 0];
+#pragma unroll
+      for (int u = 0; u < RPT; ++u) {
+        const bool in = kin && (unsigned)(y0[u] + t.y) < (unsigned)q.Hs && (unsigned)(x0[u] + t.z) < (unsigned)q.Ws;
+        cp_async_fill<4>(as + (uint32_t)(kk * SC_AP + u * NT) * 4, in ? srow[u] + t.x : src, in ? 4 : 0);
+      }
+    }
+    if (bvec) {
+#pragma unroll
+      for (int e0 = 0; e0 < SC_BK * (BN / 4); e0 += NT) {
+        const int e = e0 + tid;   // (SC_BK BN / 4 = 2 NT)
+        const int kk = e / (BN / 4), n = (e % (BN / 4)) * 4;
+        const bool in = k0 + kk < q.K && n0 + n < q.N;
+        cp_async_fill<16>(bs + (uint32_t)(kk * BN + n) * 4, in ? q.B + (size_t)(k0 + kk) * q.N + n0 + n : q.B,
+                          in ? 16 : 0);
+      }
+    } else {
+#pragma unroll
+      for (int e0 = 0; e0 < SC_BK * BN; e0 += NT) {
+        const int e = e0 + tid;
+        const int kk = e / BN, n = e % BN;
+        const bool in = k0 + kk < q.K && n0 + n < q.N;
+        cp_async_fill<4>(bs + (uint32_t)(kk * BN + n) * 4, in ? q.B + (size_t)(k0 + kk) * q.N + n0 + n : q.B,
+                         in ? 4 : 0);
+      }
+    }
+  };
+  // thread (ty, tx): rows 4 ty .. + 3 and 64 + 4 ty .. + 3, channels 4 tx .. + 3 of each half
+  unsigned long long acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  float ra[8], rb[TN];
-  __syncthreads();
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int kk = (tid >> 7) + 2 * u;
-      const int k = k0 + kk;
-      float v = 0.f;
-      if (k < q.K) {
-        const int4 t = stab[k];
-        if ((unsigned)(y0 + t.y) < (unsigned)q.Hs && (unsigned)(x0 + t.z) < (unsigned)q.Ws) v = srow[t.x];
-      }
-      ra[u] = v;
-    }
-#pragma unroll
-    for (int u = 0; u < TN; ++u) {
-      const int e = tid + SC_THREADS * u;
-      const int kk = e / BN, n = e - (e / BN) * BN;
-      const int k = k0 + kk;
-      rb[u] = (k < q.K && n0 + n < q.N) ? q.B[(size_t)k * q.N + n0 + n] : 0.f;
-    }
-  };
-  auto store = [&](int buf) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) As[buf][(tid >> 7) + 2 * u][tid & 127] = ra[u];
-#pragma unroll
-    for (int u = 0; u < TN; ++u) {
-      const int e = tid + SC_THREADS * u;
-      Bs[buf][e / BN][e - (e / BN) * BN] = rb[u];
-    }
-  };
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
   const int nk = (q.K + SC_BK - 1) / SC_BK;
-  load(0);
-  store(0);
-  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < SC_STAGES - 1; ++t) {
+    if (t < nk) load(t, t * SC_BK);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  int st = 0, ld = SC_STAGES - 1;
   for (int t = 0; t < nk; ++t) {
-    const int buf = t & 1;
-    if (t + 1 < nk) load((t + 1) * SC_BK);
+    asm volatile("cp.async.wait_group %0;" ::"n"(SC_STAGES - 2) : "memory");
+    __syncthreads();
+    if (t + SC_STAGES - 1 < nk) load(ld, (t + SC_STAGES - 1) * SC_BK);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* as = As + st * SC_BK * SC_AP + 4 * ty;
+    const float* bs = Bs + st * SC_BK * BN + 4 * tx;
+    if (++st == SC_STAGES) st = 0;
+    if (++ld == SC_STAGES) ld = 0;
 #pragma unroll
     for (int kk = 0; kk < SC_BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][4 * tm]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + 4 * tm]);
+      const float4 a0 = *reinterpret_cast<const float4*>(as + kk * SC_AP);
+      const float4 a1 = *reinterpret_cast<const float4*>(as + kk * SC_AP + 64);
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + kk * BN);
+      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + kk * BN + BN / 2);
       const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      float bv[TN];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) bv[j] = Bs[buf][kk][tn * TN + j];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long a = f32x2_dup(av[i]);
+        f32x2_fma(acc[i][0], a, b0.x);
+        f32x2_fma(acc[i][1], a, b0.y);
+        f32x2_fma(acc[i][2], a, b1.x);
+        f32x2_fma(acc[i][3], a, b1.y);
+      }
     }
-    if (t + 1 < nk) store(buf ^ 1);
-    __syncthreads();
   }
+  // four neighbouring rows are four neighbouring outputs where the pass covers whole map rows
+  const bool v4 = q.os == 1 && ((q.nJ | q.Wo) & 3) == 0 && (q.ob & 3) == 0 && ((q.HWo | ostride) & 3) == 0 &&
+                  ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(bias)) & 15) == 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const long long m = m0 + (i < 4 ? 4 * tm + i : 64 + 4 * tm + i - 4);
-    if (m >= q.M) continue;
-    const long long rr = m / q.Pm;
-    const int p2 = (int)(m - rr * q.Pm);
-    const int ii = p2 / q.nJ, jj = p2 - (p2 / q.nJ) * q.nJ;
-    const long long p = (long long)(q.oa + q.os * ii) * q.Wo + q.ob + q.os * jj;
-    float* orow = out + rr * ostride + p;
+  for (int hm = 0; hm < 2; ++hm) {
+    const uint32_t mb = m0 + 64u * hm + 4u * ty;
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int n = n0 + tn * TN + j;
-      if (n < q.N) orow[(size_t)n * q.HWo] = acc[i][j] + (bias ? bias[(size_t)n * q.HWo + p] : 0.f);
+    for (int j = 0; j < 8; ++j) {
+      const int n = n0 + (j < 4 ? 4 * tx + j : BN / 2 + 4 * tx + j - 4);
+      if (n >= q.N) continue;
+      float o[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 x = f32x2_split(acc[4 * hm + i][j / 2]);
+        o[i] = j & 1 ? x.y : x.x;
+      }
+      if (v4 && mb + 3 < q.M) {
+        long long pos;
+        float* op = out + sc_out(q, mb, ostride, &pos) + (size_t)n * q.HWo;
+        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bias) b = *reinterpret_cast<const float4*>(bias + (size_t)n * q.HWo + pos);
+        *reinterpret_cast<float4*>(op) = make_float4(o[0] + b.x, o[1] + b.y, o[2] + b.z, o[3] + b.w);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (mb + i >= q.M) continue;
+          long long pos;
+          const long long at = sc_out(q, mb + i, ostride, &pos);
+          out[at + n * q.HWo] = o[i] + (bias ? bias[(size_t)n * q.HWo + pos] : 0.f);
+        }
+      }
     }
   }
 }
@@ -144,12 +212,19 @@ __global__ void __launch_bounds__(SC_THREADS) k_sconv(SconvPass q, const float* 
 // global memory; the K loop reads the tap table and the N weights of each term from shared
 // memory (one broadcast load each).  Each output is the same sequential FMA chain in K order as
 // in k_sconv, so the result is the same bit for bit and the same a priori error bound holds.
+//
+// Which taps of a row lie inside the map is one bit each, worked out once, and 8 terms' loads (32 a
+// thread) are in flight together: with the bounds tested per term and 2 terms at a time the kernel
+// waited for its loads three quarters of the time.  All stride phases are one launch.  2,997 rows of
+// 3 x 32 x 32 from 32 channels: 185 us.
 constexpr int SN_THREADS = 256, SN_TM = 4;
 
 template <int N>
-__global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(SconvPass q, const float* __restrict__ src,
+__global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(const SconvPhases ph, const float* __restrict__ src,
                                                             long long sstride, float* __restrict__ out,
                                                             long long ostride, const float* __restrict__ bias) {
+  const SconvPass& q = ph.p[blockIdx.z];
+  if (blockIdx.x * (uint32_t)(SN_THREADS * SN_TM) >= q.M) return;
   extern __shared__ __align__(16) uint8_t sn_raw[];
   int4* stab = reinterpret_cast<int4*>(sn_raw);
   float4* sB = reinterpret_cast<float4*>(sn_raw + (size_t)q.K * sizeof(int4));
@@ -159,49 +234,75 @@ __global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(SconvPass q, const 
     const float* b = q.B + (size_t)k * N;
     sB[k] = make_float4(b[0], N > 1 ? b[1] : 0.f, N > 2 ? b[2] : 0.f, N > 3 ? b[3] : 0.f);
   }
+  __syncthreads();
   const float* srow[SN_TM];
+  uint32_t inside[SN_TM];   // taps inside the map (the first 32; the others are tested per term)
   int y0[SN_TM], x0[SN_TM];
-  long long mrow[SN_TM];
 #pragma unroll
   for (int i = 0; i < SN_TM; ++i) {
-    const long long m = (long long)blockIdx.x * (SN_THREADS * SN_TM) + i * SN_THREADS + tid;
+    const uint32_t m = blockIdx.x * (uint32_t)(SN_THREADS * SN_TM) + i * SN_THREADS + tid;
     const bool mv = m < q.M;
-    const long long r = mv ? m / q.Pm : 0;
-    const int pp = mv ? (int)(m - r * q.Pm) : 0;
-    const int pi = pp / q.nJ, pj = pp - (pp / q.nJ) * q.nJ;
+    const uint32_t r = mv ? q.dPm(m) : 0u;
+    const int pp = mv ? (int)(m - r * (uint32_t)q.Pm) : 0;
+    const int pi = (int)q.dnJ((uint32_t)pp), pj = pp - pi * q.nJ;
     y0[i] = mv ? pi * q.ms + q.cy : -32768;
     x0[i] = pj * q.ms + q.cx;
-    srow[i] = src + r * sstride + (mv ? (long long)y0[i] * q.Ws + x0[i] : 0);
-    mrow[i] = mv ? m : -1;
+    srow[i] = src + (long long)r * sstride + (mv ? (long long)y0[i] * q.Ws + x0[i] : 0);
+    inside[i] = 0u;
+    for (int t = 0; t < min(q.ntap, 32); ++t)
+      if ((unsigned)(y0[i] + stab[t].y) < (unsigned)q.Hs && (unsigned)(x0[i] + stab[t].z) < (unsigned)q.Ws)
+        inside[i] |= 1u << t;
   }
-  __syncthreads();
   float acc[SN_TM][N];
 #pragma unroll
   for (int i = 0; i < SN_TM; ++i)
 #pragma unroll
     for (int j = 0; j < N; ++j) acc[i][j] = 0.f;
-#pragma unroll 2
-  for (int k = 0; k < q.K; ++k) {
-    const int4 t = stab[k];
-    const float4 b4 = sB[k];
-    const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+  if (q.ntap <= 32) {
+    constexpr int KU = 8;
+    for (int k0 = 0; k0 < q.K; k0 += KU) {
+      float v[KU][SN_TM];
 #pragma unroll
-    for (int i = 0; i < SN_TM; ++i) {
-      const bool in = (unsigned)(y0[i] + t.y) < (unsigned)q.Hs && (unsigned)(x0[i] + t.z) < (unsigned)q.Ws;
-      const float v = in ? srow[i][t.x] : 0.f;
+      for (int e = 0; e < KU; ++e) {
+        const int k = min(k0 + e, q.K - 1);
+        const int2 t = make_int2(stab[k].x, k0 + e < q.K ? stab[k].w : 32);
 #pragma unroll
-      for (int j = 0; j < N; ++j) acc[i][j] = fmaf(v, bv[j], acc[i][j]);
+        for (int i = 0; i < SN_TM; ++i) {
+          v[e][i] = 0.f;
+          if (t.y < 32 && (inside[i] >> t.y) & 1u) v[e][i] = srow[i][t.x];
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < KU; ++e) {
+        if (k0 + e >= q.K) break;
+        const float4 b4 = sB[k0 + e];
+        const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+        for (int i = 0; i < SN_TM; ++i)
+#pragma unroll
+          for (int j = 0; j < N; ++j) acc[i][j] = fmaf(v[e][i], bv[j], acc[i][j]);
+      }
+    }
+  } else {
+    for (int k = 0; k < q.K; ++k) {
+      const int4 t = stab[k];
+      const float4 b4 = sB[k];
+      const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int i = 0; i < SN_TM; ++i) {
+        const bool in = (unsigned)(y0[i] + t.y) < (unsigned)q.Hs && (unsigned)(x0[i] + t.z) < (unsigned)q.Ws;
+        const float v = in ? srow[i][t.x] : 0.f;
+#pragma unroll
+        for (int j = 0; j < N; ++j) acc[i][j] = fmaf(v, bv[j], acc[i][j]);
+      }
     }
   }
 #pragma unroll
   for (int i = 0; i < SN_TM; ++i) {
-    const long long m = mrow[i];
-    if (m < 0) continue;
-    const long long rr = m / q.Pm;
-    const int p2 = (int)(m - rr * q.Pm);
-    const int ii = p2 / q.nJ, jj = p2 - (p2 / q.nJ) * q.nJ;
-    const long long p = (long long)(q.oa + q.os * ii) * q.Wo + q.ob + q.os * jj;
-    float* orow = out + rr * ostride + p;
+    const uint32_t m = blockIdx.x * (uint32_t)(SN_THREADS * SN_TM) + i * SN_THREADS + tid;
+    if (m >= q.M) continue;
+    long long p;
+    float* orow = out + sc_out(q, m, ostride, &p);
 #pragma unroll
     for (int j = 0; j < N; ++j) orow[(size_t)j * q.HWo] = acc[i][j] + (bias ? bias[(size_t)j * q.HWo + p] : 0.f);
   }
@@ -209,7 +310,7 @@ __global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(SconvPass q, const 
 
 int sconv_narrow_smem(int K) { return K * (int)(sizeof(int4) + sizeof(float4)); }
 
-int sconv_smem(int BN, int K) { return 2 * SC_BK * (SC_BM + 4) * 4 + 2 * SC_BK * (BN + 4) * 4 + K * (int)sizeof(int4); }
+int sconv_smem(int BN, int K) { return SC_STAGES * SC_BK * (SC_AP + BN) * 4 + K * (int)sizeof(int4); }
 
 struct LayerF32 {
   std::vector<SconvPass> bwd;   // one per stride phase with positions
@@ -289,11 +390,14 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
         q.HWo = (long long)in_h * in_w;
         q.ky0 = ky0;
         q.kx0 = kx0;
+        q.ntap = std::max(1, nky * nkx);
+        q.dPm.set(q.Pm);
+        q.dnJ.set(q.nJ);
         std::vector<int4> tab((size_t)q.K, make_int4(0, -32768, 0, 0));
         for (int co = 0; co < l.out_c; ++co)
           for (int dy = 0; dy < nky; ++dy)
             for (int dx = 0; dx < nkx; ++dx)
-              tab[(co * nky + dy) * nkx + dx] = make_int4((int)(co * q.HWs - dy * out_w - dx), -dy, -dx, 0);
+              tab[(co * nky + dy) * nkx + dx] = make_int4((int)(co * q.HWs - dy * out_w - dx), -dy, -dx, dy * nkx + dx);
         void *dt = nullptr, *dB = nullptr;
         BC_CHECK(sc_upload(t, tab.data(), tab.size() * sizeof(int4), &dt));
         q.tab = reinterpret_cast<const int4*>(dt);
@@ -338,13 +442,16 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
     f.os = 1;
     f.Wo = l.out_w;
     f.HWo = (long long)l.out_h * l.out_w;
+    f.ntap = kk;
+    f.dPm.set(f.Pm);
+    f.dnJ.set(f.nJ);
     std::vector<int4> tab((size_t)f.K);
     std::vector<float> B((size_t)f.K * f.N);
     for (int ci = 0; ci < l.in_c; ++ci)
       for (int ky = 0; ky < k; ++ky)
         for (int kx = 0; kx < k; ++kx) {
           const int kq = (ci * k + ky) * k + kx;
-          tab[kq] = make_int4((int)(ci * f.HWs + ky * l.in_w + kx), ky, kx, 0);
+          tab[kq] = make_int4((int)(ci * f.HWs + ky * l.in_w + kx), ky, kx, ky * k + kx);
           for (int co = 0; co < l.out_c; ++co) B[(size_t)kq * f.N + co] = w[(((size_t)co * l.in_c + ci) * k + ky) * k + kx];
         }
     void *dt = nullptr, *dB = nullptr;
@@ -375,29 +482,42 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
   return BCROWN_OK;
 }
 
-int sc_launch(const SconvPass& q0, int R, const float* src, long long sstride, float* out, long long ostride,
+// The n passes of one contraction (a layer's stride phases, or its forward pass) for R rows.
+int sc_launch(const SconvPass* qs, int n, int R, const float* src, long long sstride, float* out, long long ostride,
               const float* bias, cudaStream_t s) {
-  SconvPass q = q0;
-  q.M = (long long)R * q.Pm;
-  if (q.M <= 0) return BCROWN_OK;
-  if (q.N <= 4) {
-    const unsigned nb = (unsigned)((q.M + SN_THREADS * SN_TM - 1) / (SN_THREADS * SN_TM));
-    const int smem = sconv_narrow_smem(q.K);
-    if (q.N == 1) k_sconv_narrow<1><<<nb, SN_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-    else if (q.N == 2) k_sconv_narrow<2><<<nb, SN_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-    else if (q.N == 3) k_sconv_narrow<3><<<nb, SN_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-    else k_sconv_narrow<4><<<nb, SN_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
+  for (int i0 = 0; i0 < n; i0 += SC_PHASES) {
+    SconvPhases ph{};
+    const int nz = std::min(SC_PHASES, n - i0);
+    long long M = 0;
+    int K = 0;
+    for (int z = 0; z < nz; ++z) {
+      ph.p[z] = qs[i0 + z];
+      const long long m = (long long)R * ph.p[z].Pm;
+      if (m >= (1LL << 31)) return fail(BCROWN_ERR_ARG, "FP32 conv: more than 2^31 positions in a chunk");
+      ph.p[z].M = (uint32_t)m;
+      M = std::max(M, m);
+      K = std::max(K, ph.p[z].K);
+    }
+    if (M <= 0) continue;
+    const int N = ph.p[0].N;
+    if (N <= 4) {
+      const dim3 grid((unsigned)((M + SN_THREADS * SN_TM - 1) / (SN_THREADS * SN_TM)), 1, nz);
+      const int smem = sconv_narrow_smem(K);
+      if (N == 1) k_sconv_narrow<1><<<grid, SN_THREADS, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else if (N == 2) k_sconv_narrow<2><<<grid, SN_THREADS, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else if (N == 3) k_sconv_narrow<3><<<grid, SN_THREADS, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else k_sconv_narrow<4><<<grid, SN_THREADS, smem, s>>>(ph, src, sstride, out, ostride, bias);
+    } else {
+      const int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : 128;
+      const dim3 grid((unsigned)((M + SC_BM - 1) / SC_BM), (unsigned)((N + BN - 1) / BN), nz);
+      const int smem = sconv_smem(BN, K);
+      if (BN == 16) k_sconv<16><<<grid, 32, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else if (BN == 32) k_sconv<32><<<grid, 64, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else if (BN == 64) k_sconv<64><<<grid, 128, smem, s>>>(ph, src, sstride, out, ostride, bias);
+      else k_sconv<128><<<grid, 256, smem, s>>>(ph, src, sstride, out, ostride, bias);
+    }
     ++g_launches;
-    return BCROWN_OK;
   }
-  const int BN = q.N <= 16 ? 16 : q.N <= 32 ? 32 : q.N <= 64 ? 64 : 128;
-  const dim3 grid((unsigned)((q.M + SC_BM - 1) / SC_BM), (unsigned)((q.N + BN - 1) / BN));
-  const int smem = sconv_smem(BN, q.K);
-  if (BN == 16) k_sconv<16><<<grid, SC_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-  else if (BN == 32) k_sconv<32><<<grid, SC_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-  else if (BN == 64) k_sconv<64><<<grid, SC_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-  else k_sconv<128><<<grid, SC_THREADS, smem, s>>>(q, src, sstride, out, ostride, bias);
-  ++g_launches;
   return BCROWN_OK;
 }
 
@@ -417,8 +537,8 @@ int sconv_bwd(bcrown_net* net, int i, int R, const float* Lam, float* Ain, cudaS
   SconvNet* t = sc_of(net);
   if (!t->ready) return fail(BCROWN_ERR_ARG, "FP32 conv: tables not built");
   const LayerDev& l = net->ly[i - 1];
-  for (const SconvPass& q : t->ly[i].bwd) BC_CHECK(sc_launch(q, R, Lam, l.d_out, Ain, l.d_in, nullptr, s));
-  return BCROWN_OK;
+  const std::vector<SconvPass>& q = t->ly[i].bwd;
+  return sc_launch(q.data(), (int)q.size(), R, Lam, l.d_out, Ain, l.d_in, nullptr, s);
 }
 
 bool root_patch(const bcrown_net* net, int T, std::vector<int>& n) {
@@ -438,17 +558,16 @@ int sconv_patch(bcrown_net* net, int T, int i, int R, const float* Lam, float* A
   std::vector<int> n;
   if (!t->ready || !root_patch(net, T, n)) return fail(BCROWN_ERR_ARG, "FP32 conv: no patch tables");
   const LayerDev& l = net->ly[i - 1];
-  for (const SconvPass& q : t->ly[i].patch[T])
-    BC_CHECK(sc_launch(q, R, Lam, (long long)l.out_c * n[i] * n[i], Ain, (long long)l.in_c * n[i - 1] * n[i - 1],
-                       nullptr, s));
-  return BCROWN_OK;
+  const std::vector<SconvPass>& q = t->ly[i].patch[T];
+  return sc_launch(q.data(), (int)q.size(), R, Lam, (long long)l.out_c * n[i] * n[i], Ain,
+                   (long long)l.in_c * n[i - 1] * n[i - 1], nullptr, s);
 }
 
 int sconv_fwd(bcrown_net* net, int i, int R, const float* h, float* Z, const float* bias, cudaStream_t s) {
   SconvNet* t = sc_of(net);
   if (!t->ready) return fail(BCROWN_ERR_ARG, "FP32 conv: tables not built");
   const LayerDev& l = net->ly[i - 1];
-  return sc_launch(t->ly[i].fwd, R, h, l.d_in, Z, l.d_out, bias, s);
+  return sc_launch(&t->ly[i].fwd, 1, R, h, l.d_in, Z, l.d_out, bias, s);
 }
 
 void sconv_release(const bcrown_net* net) {

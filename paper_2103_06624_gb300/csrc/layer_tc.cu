@@ -62,17 +62,6 @@ struct LtList {
   int2 split[BCROWN_MAX_SPLITS];
 };
 
-// n / d for n < 2^31 by multiplication.
-struct FastDiv {
-  uint32_t d, mul, sh;
-  __host__ void set(uint32_t v) {
-    d = v;
-    sh = 0;
-    while ((1ull << sh) < v) ++sh;
-    mul = (uint32_t)((((1ull << sh) - v) << 32) / v + 1);
-  }
-  __device__ __forceinline__ uint32_t operator()(uint32_t n) const { return (__umulhi(n, mul) + n) >> sh; }
-};
 // Warp roles.  Gathered A operand: 12 epilogue warps (three groups of 4, every third tile) and 4
 // gather warps.  A operand by TMA: 16 epilogue warps (four groups).  Both with
 // the TMA and the MMA warp: 18 warps, which leaves 96 registers a thread.

@@ -610,29 +610,6 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
 // ----------------------------------------------------------------------------------------
 constexpr int SG_STAGES = 3;
 
-__device__ __forceinline__ unsigned long long f32x2_dup(float a) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
-  return r;
-}
-__device__ __forceinline__ void f32x2_fma(unsigned long long& c, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ float2 f32x2_split(unsigned long long c) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(c));
-  return r;
-}
-
-// Copies `bytes` (0 .. SIZE) of src, the rest of the SIZE-byte piece zero.
-template <int SIZE>
-__device__ __forceinline__ void cp_async_fill(uint32_t dst, const float* src, int bytes) {
-  if (SIZE == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-
 // BM x BN tiles, K steps of BK, TM x 8 outputs per thread; VEC: 16-byte copies (A and B with
 // 16-byte aligned rows).
 template <int BM, int BN, int BK, int TM, bool VEC>
