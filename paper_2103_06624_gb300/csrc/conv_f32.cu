@@ -53,18 +53,21 @@ __device__ __forceinline__ long long sc_out(const SconvPass& q, uint32_t m, long
 }
 
 // A 128 x BN tile, 8 x 8 outputs a thread (2 BN threads), FMAs on pairs of neighbouring channels
-// (fma.rn.f32x2, as the GEMM), both operands by cp.async into three stages of 16 K terms: the
+// (fma.rn.f32x2, as the GEMM), both operands by cp.async into two stages of 16 K terms: the
 // gathered one in 4-byte pieces (a warp's are one run of positions), zero-filled where a tap falls
-// outside the map.  Bound by the FMA pipe and, for few output channels, by the gather's
-// instructions (each gathered value feeds BN FMAs).  2,997 rows of the 32 -> 64 channel 4x4 stride-2
-// layer backward: 668 us in four launches with 8 x 2 outputs a thread and register staging, 420 now.
-constexpr int SC_BM = 128, SC_BK = 16, SC_STAGES = 3;
+// outside the map, which is one bit per tap, worked out once a row.  Bound by the shared-memory pipe
+// (48 % of its peak at 128 channels, 71 % at 32, where a gathered value feeds fewest FMAs) together
+// with the FMA pipe; a third stage costs a resident block and is 3 % slower.  2,997 rows of the
+// 32 -> 64 channel 4x4 stride-2 layer backward: 668 us in four launches with 8 x 2 outputs a thread
+// and register staging, 420 with bounds tested per value and the lanes in row order, 347 now; 576
+// rows of the 128 -> 128 channel 3x3 stride-2 layer 353 -> 271.
+constexpr int SC_BM = 128, SC_BK = 16, SC_STAGES = 2;
 constexpr int SC_AP = SC_BM + 4;
 
 template <int BN>
-__global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const float* __restrict__ src,
-                                                  long long sstride, float* __restrict__ out, long long ostride,
-                                                  const float* __restrict__ bias) {
+__global__ void __launch_bounds__(2 * BN, BN == 32 ? 7 : 256 / BN)
+    k_sconv(const SconvPhases ph, const float* __restrict__ src, long long sstride, float* __restrict__ out,
+            long long ostride, const float* __restrict__ bias) {
   constexpr int NT = 2 * BN;
   constexpr int RPT = NT >= SC_BM ? 1 : SC_BM / NT;    // tile rows a thread gathers
   constexpr int KSTEP = NT >= SC_BM ? NT / SC_BM : 1;  // and the stride of its K terms
@@ -74,14 +77,28 @@ __global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const fl
   extern __shared__ __align__(16) uint8_t sc_raw[];
   float* As = reinterpret_cast<float*>(sc_raw);                 // [stage][SC_BK][SC_AP]
   float* Bs = As + SC_STAGES * SC_BK * SC_AP;                   // [stage][SC_BK][BN]
-  int4* stab = reinterpret_cast<int4*>(Bs + SC_STAGES * SC_BK * BN);
-  const int tid = threadIdx.x;
-  const int ty = tid & 15, tx = tid >> 4;
+  int2* stab = reinterpret_cast<int2*>(Bs + SC_STAGES * SC_BK * BN);   // [K, rounded up]: {offset, tap's bit}
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // A warp's 32 threads are 8 row groups by 4 channel groups (16 by 2 where the block is one warp),
+  // neighbouring lanes in the same row group: a 16-byte shared read then takes 2 wavefronts (4 with
+  // the lanes in row order), and the shared pipe bounds the kernel beside the FMAs.
+  const int ty = BN == 16 ? lane >> 1 : ((lane >> 1) & 7) + 8 * (w & 1);
+  const int tx = BN == 16 ? lane & 1 : (lane & 1) + 2 * (lane >> 4) + 4 * (w >> 1);
   const int n0 = blockIdx.y * BN;
-  for (int k = tid; k < q.K; k += NT) stab[k] = q.tab[k];
-  // the rows this thread gathers (fixed across K) and their base source positions
+  const int nk = (q.K + SC_BK - 1) / SC_BK;
+  const bool bits = q.ntap <= 32;
+  for (int k = tid; k < nk * SC_BK; k += NT) {
+    int2 e = make_int2(0, 0);
+    if (k < q.K) {
+      const int4 t = q.tab[k];
+      e = make_int2(t.x, bits ? (int)(1u << t.w) : 0);
+    }
+    stab[k] = e;
+  }
+  // the rows this thread gathers (fixed across K), their base source positions and their taps in the map
   const float* srow[RPT];
-  int y0[RPT], x0[RPT];
+  int pos[RPT], y0[RPT], x0[RPT];
+  uint32_t inside[RPT];
 #pragma unroll
   for (int u = 0; u < RPT; ++u) {
     const uint32_t m = m0 + (uint32_t)(tid % SC_BM) + (uint32_t)(u * NT);
@@ -91,7 +108,13 @@ __global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const fl
     const int pi = (int)q.dnJ((uint32_t)pp), pj = pp - pi * q.nJ;
     y0[u] = mv ? pi * q.ms + q.cy : -32768;
     x0[u] = pj * q.ms + q.cx;
-    srow[u] = src + (long long)r * sstride + (mv ? (long long)y0[u] * q.Ws + x0[u] : 0);
+    srow[u] = src + (long long)r * sstride;
+    pos[u] = y0[u] * q.Ws + x0[u];
+    inside[u] = 0u;
+    for (int t = 0; bits && t < q.ntap; ++t) {
+      const int4 e = q.tab[t];
+      if ((unsigned)(y0[u] + e.y) < (unsigned)q.Hs && (unsigned)(x0[u] + e.z) < (unsigned)q.Ws) inside[u] |= 1u << t;
+    }
   }
   const uint32_t sA = (uint32_t)__cvta_generic_to_shared(As), sB = (uint32_t)__cvta_generic_to_shared(Bs);
   const bool bvec = (q.N & 3) == 0;
@@ -99,15 +122,26 @@ __global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const fl
   auto load = [&](int stage, int k0) {
     const uint32_t as = sA + (uint32_t)(stage * SC_BK * SC_AP + tid % SC_BM) * 4;
     const uint32_t bs = sB + (uint32_t)(stage * SC_BK * BN) * 4;
+    if (bits) {
 #pragma unroll
-    for (int kk = tid / SC_BM; kk < SC_BK; kk += KSTEP) {
-      const int k = k0 + kk;
-      const bool kin = k < q.K;
-      const int4 t = stab[kin ? k : 0];
+      for (int k1 = 0; k1 < SC_BK; k1 += KSTEP) {
+        const int kk = k1 + tid / SC_BM;
+        const int2 t = stab[k0 + kk];
 #pragma unroll
-      for (int u = 0; u < RPT; ++u) {
-        const bool in = kin && (unsigned)(y0[u] + t.y) < (unsigned)q.Hs && (unsigned)(x0[u] + t.z) < (unsigned)q.Ws;
-        cp_async_fill<4>(as + (uint32_t)(kk * SC_AP + u * NT) * 4, in ? srow[u] + t.x : src, in ? 4 : 0);
+        for (int u = 0; u < RPT; ++u) {
+          const bool in = (inside[u] & (uint32_t)t.y) != 0u;
+          cp_async_fill<4>(as + (uint32_t)(kk * SC_AP + u * NT) * 4, srow[u] + (in ? pos[u] + t.x : 0), in ? 4 : 0);
+        }
+      }
+    } else {
+      for (int kk = tid / SC_BM; kk < SC_BK; kk += KSTEP) {
+        const int k = k0 + kk;
+        const int4 t = q.tab[min(k, q.K - 1)];
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+          const bool in = k < q.K && (unsigned)(y0[u] + t.y) < (unsigned)q.Hs && (unsigned)(x0[u] + t.z) < (unsigned)q.Ws;
+          cp_async_fill<4>(as + (uint32_t)(kk * SC_AP + u * NT) * 4, srow[u] + (in ? pos[u] + t.x : 0), in ? 4 : 0);
+        }
       }
     }
     if (bvec) {
@@ -136,7 +170,6 @@ __global__ void __launch_bounds__(2 * BN) k_sconv(const SconvPhases ph, const fl
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-  const int nk = (q.K + SC_BK - 1) / SC_BK;
 #pragma unroll
   for (int t = 0; t < SC_STAGES - 1; ++t) {
     if (t < nk) load(t, t * SC_BK);
@@ -310,7 +343,9 @@ __global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(const SconvPhases p
 
 int sconv_narrow_smem(int K) { return K * (int)(sizeof(int4) + sizeof(float4)); }
 
-int sconv_smem(int BN, int K) { return SC_STAGES * SC_BK * (SC_AP + BN) * 4 + K * (int)sizeof(int4); }
+int sconv_smem(int BN, int K) {
+  return SC_STAGES * SC_BK * (SC_AP + BN) * 4 + (K + SC_BK - 1) / SC_BK * SC_BK * (int)sizeof(int2);
+}
 
 struct LayerF32 {
   std::vector<SconvPass> bwd;   // one per stride phase with positions
