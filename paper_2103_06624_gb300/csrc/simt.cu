@@ -304,9 +304,7 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
   constexpr int RPB = RELAX_WARPS / WPR;   // rows per block
   __shared__ SplitSlot slots[RPB][BCROWN_MAX_SPLITS];
   __shared__ int nslots[RPB];
-  // split bitmask of a wide row (a whole block's row, up to SPLIT_MASK_WORDS * 32 neurons)
-  constexpr int MW = WPR > 1 ? SPLIT_MASK_WORDS : 1;
-  __shared__ uint32_t smask[RPB][MW];
+  extern __shared__ uint32_t relax_mask[];   // split bitmask of each row (up to SPLIT_MASK_WORDS * 32 neurons)
   __shared__ float red[RELAX_WARPS][3];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rs = w / WPR, sub = w - rs * WPR;   // row slot in the block, warp within the row
@@ -347,16 +345,17 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
   }
   if (WPR > 1) __syncthreads();
   else __syncwarp();
-  const bool use_mask = WPR > 1 && d <= MW * 32;
+  const bool use_mask = d <= SPLIT_MASK_WORDS * 32;
+  uint32_t* const smask = relax_mask + rs * ((d + 31) / 32);
   if (use_mask) {
     if (live)
-      for (int q = sub * 32 + lane; q < (d + 31) / 32; q += 32 * WPR) smask[rs][q] = 0u;
+      for (int q = sub * 32 + lane; q < (d + 31) / 32; q += 32 * WPR) smask[q] = 0u;
     if (WPR > 1) __syncthreads();
     else __syncwarp();
     if (live)
       for (int q = sub * 32 + lane; q < nslots[rs]; q += 32 * WPR) {
         const int jj = slots[rs][q].idx;
-        atomicOr(&smask[rs][jj >> 5], 1u << (jj & 31));
+        atomicOr(&smask[jj >> 5], 1u << (jj & 31));
       }
     if (WPR > 1) __syncthreads();
     else __syncwarp();
@@ -373,10 +372,89 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
     // CERT: acc is a lower bound of sum_j Lambda_j b_j + A_j lambda_j (every operation rounded
     // down); e1, e2 are upper bounds (rounded up) of the error terms below.
     const size_t n0 = (size_t)p * c.tb.H + hoff;
-    // Rows of up to 2048 neurons (one warp each): one neuron per lane per step, the split list
-    // scanned per neuron (short for these rows); measured faster there than the wide-row code
-    // below, which the wide (conv) layers need.
-    if (WPR == 1) {
+    // Rows whose neurons lie on 16-byte boundaries in every array: 4 consecutive neurons per lane
+    // (float4 A, bias, Lambda and, certified, error weights; uchar4 codes), 1024 or 128 a step of the
+    // row's warps; a group of stable, unsplit neurons needs no other load.
+    const long long aend = abase + Up;
+    const bool alpha_ok = abase >= 0 && aend <= n_alpha;   // the row's alpha block, checked once
+    const uintptr_t mis = reinterpret_cast<uintptr_t>(a_row) | reinterpret_cast<uintptr_t>(lam_row) |
+                          reinterpret_cast<uintptr_t>(bias) |
+                          (CERT ? reinterpret_cast<uintptr_t>(wm + n0) | reinterpret_cast<uintptr_t>(c.l + n0) |
+                                      reinterpret_cast<uintptr_t>(c.u + n0)
+                                : 0);
+    const bool vec4 = ((d | (int)(n0 & 3)) & 3) == 0 && (mis & 15) == 0 && ((WPR > 1 && !CERT) || alpha_ok);
+    if (vec4) {
+      const uchar4* code4 = reinterpret_cast<const uchar4*>(c.tb.code + n0);
+      const float* alpha_row = alpha_ok ? alpha + abase : nullptr;
+      if (!alpha_row && Up > 0 && lane == 0 && sub == 0) flag(c.status, BCROWN_ERR_ARG);
+#pragma unroll 2
+      for (int q = sub * 32 + lane; q < d / 4; q += 32 * WPR) {
+        const int j = 4 * q;
+        const float4 a4 = reinterpret_cast<const float4*>(a_row)[q];
+        const float4 b4 = reinterpret_cast<const float4*>(bias)[q];
+        const float4 w4 = CERT ? reinterpret_cast<const float4*>(wm + n0)[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const uchar4 c4 = code4[q];
+        const uint32_t sb = ns == 0 ? 0u : (use_mask ? (smask[j >> 5] >> (j & 31)) & 0xFu : 0xFu);
+        const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+        const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
+        float Lv[4];
+        if (sb == 0u && stable4(c4)) {
+          const float dv[4] = {d01(c4.x), d01(c4.y), d01(c4.z), d01(c4.w)};
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            Lv[v] = fmaf(av[v], dv[v], 0.f);
+            if (CERT) {
+              acc = __fadd_rd(acc, __fadd_rd(__fmul_rd(Lv[v], bv[v]), __fmul_rd(av[v], 0.f)));
+              e2 = __fadd_ru(e2, __fmul_ru(fabsf(Lv[v]), wv[v]));
+            } else {
+              acc = fmaf(Lv[v], bv[v], fmaf(av[v], 0.f, acc));
+            }
+          }
+        } else {
+          float D[4], lm[4], zl[4], zu[4];
+          int rk[4];
+          if (CERT) {
+            const float4 l4 = *reinterpret_cast<const float4*>(c.l + n0 + j);
+            const float4 u4 = *reinterpret_cast<const float4*>(c.u + n0 + j);
+            zl[0] = l4.x, zl[1] = l4.y, zl[2] = l4.z, zl[3] = l4.w;
+            zu[0] = u4.x, zu[1] = u4.y, zu[2] = u4.z, zu[3] = u4.w;
+          }
+          group4(c.tb, n0 + j, av, c4, alpha_row, D, lm, rk);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            float bs = 0.f;
+            int s = 0;
+            if ((sb >> v) & 1u)   // a split of the row may sit here
+              for (int qq = 0; qq < ns; ++qq)
+                if (sl_[qq].idx == j + v) {
+                  const long long bi = bbase + sl_[qq].t;
+                  s = sl_[qq].sign;
+                  if (bi >= 0 && bi < n_beta) bs = fmaxf(beta[bi], 0.f) * (float)s;
+                  else flag(c.status, BCROWN_ERR_ARG);
+                  D[v] = s == -1 ? 1.f : 0.f;
+                  lm[v] = 0.f;
+                }
+            Lv[v] = fmaf(av[v], D[v], bs);
+            if (CERT) {
+              acc = __fadd_rd(acc, __fadd_rd(__fmul_rd(Lv[v], bv[v]), __fmul_rd(av[v], lm[v])));
+              if (!(s == 0 && (D[v] == 0.f || D[v] == 1.f))) {
+                // Lambda_j was rounded once: |error| <= 2^-23 |Lambda_j| (+ an underflow margin),
+                // acting on |z_j| <= max(|l_j|, |u_j|)
+                const float zmax = fmaxf(fabsf(zl[v]), fabsf(zu[v]));
+                e1 = __fadd_ru(e1, __fmul_ru(__fmaf_ru(fabsf(Lv[v]), 0x1p-23f, 0x1p-140f), zmax));
+              }
+              e2 = __fadd_ru(e2, __fmul_ru(fabsf(Lv[v]), wv[v]));
+            } else {
+              acc = fmaf(Lv[v], bv[v], fmaf(av[v], lm[v], acc));
+            }
+          }
+        }
+        reinterpret_cast<float4*>(lam_row)[q] = make_float4(Lv[0], Lv[1], Lv[2], Lv[3]);
+      }
+    }
+    // Other rows of up to 2048 neurons (one warp each): one neuron per lane per step, the split list
+    // scanned per neuron (short for these rows).
+    if (WPR == 1 && !vec4) {
   #pragma unroll 4
       for (int j = sub * 32 + lane; j < d; j += 32 * WPR) {
         const float a = a_row[j];
@@ -428,57 +506,6 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
         }
       }
     }
-    // FP32 form with 16-byte aligned rows: 4 consecutive neurons per lane (float4 A, bias and
-    // Lambda, uchar4 codes); a group of stable, unsplit neurons needs no other load
-    const bool vec4 = WPR > 1 && !CERT && ((d | (int)(n0 & 3)) & 3) == 0 &&
-                      ((reinterpret_cast<uintptr_t>(a_row) | reinterpret_cast<uintptr_t>(lam_row) |
-                        reinterpret_cast<uintptr_t>(bias)) & 15) == 0;
-    if (vec4) {
-      const uchar4* code4 = reinterpret_cast<const uchar4*>(c.tb.code + n0);
-      // the row's alpha block, checked once against the array
-      const float* alpha_row = (abase >= 0 && abase + Up <= n_alpha) ? alpha + abase : nullptr;
-      if (!alpha_row && Up > 0 && lane == 0 && sub == 0) flag(c.status, BCROWN_ERR_ARG);
-      for (int q = sub * 32 + lane; q < d / 4; q += 32 * WPR) {
-        const int j = 4 * q;
-        const float4 a4 = reinterpret_cast<const float4*>(a_row)[q];
-        const float4 b4 = reinterpret_cast<const float4*>(bias)[q];
-        const uchar4 c4 = code4[q];
-        const uint32_t sb = ns == 0 ? 0u : (use_mask ? (smask[rs][j >> 5] >> (j & 31)) & 0xFu : 0xFu);
-        float4 L;
-        if (sb == 0u && stable4(c4)) {
-          L.x = fmaf(a4.x, d01(c4.x), 0.f);
-          L.y = fmaf(a4.y, d01(c4.y), 0.f);
-          L.z = fmaf(a4.z, d01(c4.z), 0.f);
-          L.w = fmaf(a4.w, d01(c4.w), 0.f);
-          acc = fmaf(L.x, b4.x, fmaf(a4.x, 0.f, acc));
-          acc = fmaf(L.y, b4.y, fmaf(a4.y, 0.f, acc));
-          acc = fmaf(L.z, b4.z, fmaf(a4.z, 0.f, acc));
-          acc = fmaf(L.w, b4.w, fmaf(a4.w, 0.f, acc));
-        } else {
-          const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
-          float D[4], lm[4], Lv[4];
-          int rk[4];
-          group4(c.tb, n0 + j, av, c4, alpha_row, D, lm, rk);
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            float bs = 0.f;
-            if ((sb >> v) & 1u)   // a split of the row may sit here
-              for (int qq = 0; qq < ns; ++qq)
-                if (sl_[qq].idx == j + v) {
-                  const long long bi = bbase + sl_[qq].t;
-                  if (bi >= 0 && bi < n_beta) bs = fmaxf(beta[bi], 0.f) * (float)sl_[qq].sign;
-                  else flag(c.status, BCROWN_ERR_ARG);
-                  D[v] = sl_[qq].sign == -1 ? 1.f : 0.f;
-                  lm[v] = 0.f;
-                }
-            Lv[v] = fmaf(av[v], D[v], bs);
-            acc = fmaf(Lv[v], bv[v], fmaf(av[v], lm[v], acc));
-          }
-          L = make_float4(Lv[0], Lv[1], Lv[2], Lv[3]);
-        }
-        reinterpret_cast<float4*>(lam_row)[q] = L;
-      }
-    }
     // RELAX_V neurons per lane per step, their loads issued in three rounds (A, code, bias; then
     // the unstable neurons' rank and chord; then alpha) instead of one dependent chain each
     constexpr int RELAX_V = 4;
@@ -519,7 +546,7 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
         const size_t n = n0 + j;
         int s = 0;
         float bet = 0.f;
-        if (ns > 0 && (!use_mask || split_bit(smask[rs], j)))
+        if (ns > 0 && (!use_mask || split_bit(smask, j)))
           for (int q = 0; q < ns; ++q)
             if (sl_[q].idx == j) {
               s = sl_[q].sign;
@@ -1448,19 +1475,20 @@ void launch_relax(bool cert, const RowsCtx& c, int layer, int d, long long hoff,
                   const float* bias, const float* alpha, int64_t n_alpha, const float* beta, int64_t n_beta, float* cf,
                   double* cd, double* E, const float* wm, double gamma, cudaStream_t s) {
   if (c.R <= 0) return;
-  // one warp per row up to 2048 neurons, a whole block per row beyond
+  // One warp per row up to 2048 neurons, a whole block per row beyond.
   const bool wide = d > 2048;
   const int rpb = wide ? 1 : RELAX_WARPS;
   const int grid = (c.R + rpb - 1) / rpb;
-  if (cert && wide)
-    k_relax<true, RELAX_WARPS><<<grid, 32 * RELAX_WARPS, 0, s>>>(c, layer, d, hoff, Ain, Lam, bias, alpha, n_alpha, beta, n_beta, cf, cd, E, wm, gamma);
-  else if (cert)
-    k_relax<true, 1><<<grid, 32 * RELAX_WARPS, 0, s>>>(c, layer, d, hoff, Ain, Lam, bias, alpha, n_alpha, beta, n_beta, cf, cd, E, wm, gamma);
-  else if (wide)
-    k_relax<false, RELAX_WARPS><<<grid, 32 * RELAX_WARPS, 0, s>>>(c, layer, d, hoff, Ain, Lam, bias, alpha, n_alpha, beta, n_beta, cf, cd, E, wm, gamma);
-  else
-    k_relax<false, 1><<<grid, 32 * RELAX_WARPS, 0, s>>>(c, layer, d, hoff, Ain, Lam, bias, alpha, n_alpha, beta, n_beta, cf, cd, E, wm, gamma);
-  ++g_launches;
+  const size_t smem = d <= SPLIT_MASK_WORDS * 32 ? (size_t)rpb * ((d + 31) / 32) * sizeof(uint32_t) : 0;
+  auto go = [&](auto* kernel) {
+    kernel<<<grid, 32 * RELAX_WARPS, smem, s>>>(c, layer, d, hoff, Ain, Lam, bias, alpha, n_alpha, beta, n_beta, cf,
+                                                cd, E, wm, gamma);
+    ++g_launches;
+  };
+  if (cert && wide) go(k_relax<true, RELAX_WARPS>);
+  else if (cert) go(k_relax<true, 1>);
+  else if (wide) go(k_relax<false, RELAX_WARPS>);
+  else go(k_relax<false, 1>);
 }
 
 template <int BM, int BN, int BK, int TM>
