@@ -533,7 +533,7 @@ extern "C" int bcrown_root_bounds(bcrown_net* net, int n_props, const float* x_l
                     T >= 3 ? net->hoff[T - 3] : -1, u, x_lo, x_hi, net->d[0], pl.wm, s);
     std::vector<int> n;
     const bool patch = root_patch(net, T, n);
-    std::vector<RootMap> map(T, RootMap{0, 0, 0, 0, 0});
+    std::vector<RootMap> map(T, RootMap{});
     std::vector<int> d(T);
     for (int m = T - 1, os = 1, oo = 0; m >= 0; --m) {
       d[m] = net->d[m];
@@ -541,7 +541,9 @@ extern "C" int bcrown_root_bounds(bcrown_net* net, int n_props, const float* x_l
       const LayerDev& ly = net->ly[m];   // layer m + 1: from map m to map m + 1
       os *= ly.stride;
       oo = oo * ly.stride + ly.pad;
-      map[m] = RootMap{n[m], ly.in_h, ly.in_w, os, oo};
+      map[m] = RootMap{n[m], ly.in_h, ly.in_w, os, oo, {}, {}};
+      map[m].dnn.set(n[m] * n[m]);
+      map[m].dn.set(n[m]);
       d[m] = ly.in_c * n[m] * n[m];
     }
     const long long rows = 2LL * c.d_top * n_props;

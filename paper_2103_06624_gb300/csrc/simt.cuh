@@ -73,6 +73,7 @@ struct RootCtx {
 // origin is (position in layer T) * os - oo, over an Hm x Wm map.
 struct RootMap {
   int n, Hm, Wm, os, oo;
+  FastDiv dnn, dn;   // by n n and by n (n > 0)
 };
 void launch_root_first(bool cert, const RootCtx& c, int P, const LayerGeom& g, const float* W, const float* b,
                        cudaStream_t s);
