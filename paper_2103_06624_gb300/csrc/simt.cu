@@ -167,39 +167,92 @@ __device__ __forceinline__ uint32_t ld_u8(const uint8_t* p, bool pred, uint32_t 
 __device__ __forceinline__ float hmax_hidden(float uv) { return fmaxf(uv, 0.f); }
 
 // wm[p][hoff_i + j] = sum_m |W^(i)_jm| M^(i-1)_m, every product and sum rounded up (FP32),
-// for the a priori contraction error of layer i.  One warp per output neuron.
-__global__ void __launch_bounds__(256) k_absw_m(LayerGeom g, const float* __restrict__ W, int P, int H,
+// for the a priori contraction error of layer i.  One warp per output neuron, or, of a convolution,
+// per 4 neighbouring positions of an output channel: they share the weight's load and the term's
+// index arithmetic, and their 4 chains of rounded sums run side by side.  The loads of 4 terms (of 8
+// for a fully connected layer) are issued together.  Every neuron's sum has the same order whatever
+// the grouping.  576 terms x 32,768 neurons: 65 us, a neuron and a term at a time.
+struct AbswDiv {
+  FastDiv hw, ow, kk, k, groups;
+};
+constexpr int ABSW_G = 4;
+__global__ void __launch_bounds__(256) k_absw_m(LayerGeom g, AbswDiv dv, const float* __restrict__ W, int P, int H,
                                                 long long hoff_i, long long hoff_prev, const float* __restrict__ u,
                                                 const float* __restrict__ x_lo, const float* __restrict__ x_hi,
-                                                int d0, float* __restrict__ wm) {
-  const long long id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+                                                int d0, float* __restrict__ wm, uint32_t total) {
+  const uint32_t id = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  const long long total = (long long)P * g.d_out;
   if (id >= total) return;
-  const int p = (int)(id / g.d_out);
-  const int j = (int)(id - (long long)p * g.d_out);
+  const int p = (int)dv.groups(id);
+  const int grp = (int)(id - (uint32_t)p * dv.groups.d);
+  const float* up = hoff_prev < 0 ? nullptr : u + (size_t)p * H + hoff_prev;
+  const float *xl = x_lo + (size_t)p * d0, *xh = x_hi + (size_t)p * d0;
   auto M = [&](int m) -> float {
-    if (hoff_prev < 0) return fmaxf(fabsf(x_lo[(size_t)p * d0 + m]), fabsf(x_hi[(size_t)p * d0 + m]));
-    return hmax_hidden(u[(size_t)p * H + hoff_prev + m]);
+    if (!up) return fmaxf(fabsf(xl[m]), fabsf(xh[m]));
+    return hmax_hidden(up[m]);
   };
-  float s = 0.f;
   if (g.kind == BCROWN_LAYER_FC) {
-    const float* w = W + (size_t)j * g.d_in;
-    for (int m = lane; m < g.d_in; m += 32) s = __fadd_ru(s, __fmul_ru(fabsf(w[m]), M(m)));
-  } else {
-    const int hw = g.out_h * g.out_w;
-    const int co = j / hw, rem = j - co * hw, oy = rem / g.out_w, ox = rem - oy * g.out_w;
-    const int kk = g.k * g.k;
-    for (int t = lane; t < g.in_c * kk; t += 32) {
-      const int ci = t / kk, r = t - ci * kk, ky = r / g.k, kx = r - ky * g.k;
-      const int iy = oy * g.stride - g.pad + ky, ix = ox * g.stride - g.pad + kx;
-      if (iy < 0 || iy >= g.in_h || ix < 0 || ix >= g.in_w) continue;
-      const float w = fabsf(W[(((size_t)co * g.in_c + ci) * g.k + ky) * g.k + kx]);
-      s = __fadd_ru(s, __fmul_ru(w, M((ci * g.in_h + iy) * g.in_w + ix)));
+    const float* w = W + (size_t)grp * g.d_in;
+    float s = 0.f;
+    constexpr int V = 8;
+    for (int m0 = lane; m0 < g.d_in; m0 += 32 * V) {
+      float wv[V], mv[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int m = m0 + 32 * v;
+        wv[v] = m < g.d_in ? fabsf(w[m]) : 0.f;
+        mv[v] = m < g.d_in ? M(m) : 0.f;
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (m0 + 32 * v < g.d_in) s = __fadd_ru(s, __fmul_ru(wv[v], mv[v]));
     }
+    for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(0xffffffffu, s, o));
+    if (lane == 0) wm[(size_t)p * H + hoff_i + grp] = s;
+    return;
   }
-  for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(0xffffffffu, s, o));
-  if (lane == 0) wm[(size_t)p * H + hoff_i + j] = s;
+  const int hw = g.out_h * g.out_w, gc = (hw + ABSW_G - 1) / ABSW_G, kk = g.k * g.k;
+  const int co = grp / gc, pos0 = (grp - co * gc) * ABSW_G;
+  int y0[ABSW_G], x0[ABSW_G];
+  float s[ABSW_G];
+#pragma unroll
+  for (int q = 0; q < ABSW_G; ++q) {
+    const int pos = pos0 + q, oy = (int)dv.ow((uint32_t)pos), ox = pos - oy * g.out_w;
+    y0[q] = pos < hw ? oy * g.stride - g.pad : -32768;   // (out of the map for every tap)
+    x0[q] = ox * g.stride - g.pad;
+    s[q] = 0.f;
+  }
+  const float* wr = W + (size_t)co * g.in_c * kk;
+  const int T = g.in_c * kk;
+  constexpr int V = 4;
+  for (int t0 = lane; t0 < T; t0 += 32 * V) {
+    float wv[V], mv[V][ABSW_G];
+    bool in[V][ABSW_G];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int t = t0 + 32 * v;
+      const bool tin = t < T;
+      const int tt = tin ? t : 0;
+      const int ci = (int)dv.kk((uint32_t)tt), r = tt - ci * kk, ky = (int)dv.k((uint32_t)r), kx = r - ky * g.k;
+      wv[v] = fabsf(wr[tt]);
+#pragma unroll
+      for (int q = 0; q < ABSW_G; ++q) {
+        const int iy = y0[q] + ky, ix = x0[q] + kx;
+        in[v][q] = tin && (unsigned)iy < (unsigned)g.in_h && (unsigned)ix < (unsigned)g.in_w;
+        mv[v][q] = in[v][q] ? M((ci * g.in_h + iy) * g.in_w + ix) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int q = 0; q < ABSW_G; ++q)
+        if (in[v][q]) s[q] = __fadd_ru(s[q], __fmul_ru(wv[v], mv[v][q]));
+  }
+#pragma unroll
+  for (int q = 0; q < ABSW_G; ++q) {
+    for (int o = 16; o > 0; o >>= 1) s[q] = __fadd_ru(s[q], __shfl_xor_sync(0xffffffffu, s[q], o));
+    if (lane == 0 && pos0 + q < hw) wm[(size_t)p * H + hoff_i + (size_t)co * hw + pos0 + q] = s[q];
+  }
 }
 
 // ----------------------------------------------------------------------------------------
@@ -1138,8 +1191,11 @@ __device__ __forceinline__ float adam_alpha(float th, float g, float& m, float& 
   return __saturatef(th);
 }
 
-// One warp per row: the row's alphas in 16-byte accesses where the arrays allow it.
+// One warp per row, or a block for rows of many alphas (WPR warps: launch_adam): the row's alphas in
+// 16-byte accesses where the arrays allow it.  Bound by memory: 32 bytes an alpha, 36 where the row
+// improved.  576 rows of 12,000 alphas: 96 us a warp per row (72 blocks).
 constexpr int ADAM_ROWS_PER_BLOCK = 8;
+template <int WPR>
 __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(
     int R, int K, BatchView bt, const int32_t* __restrict__ U, int P, const float* __restrict__ lb_t,
     float* __restrict__ best_lb, float* __restrict__ a_cur, float* __restrict__ a_best,
@@ -1147,14 +1203,15 @@ __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(
     float* __restrict__ b_best, const float* __restrict__ gb, float* __restrict__ mb, float* __restrict__ vb,
     float lr_a, float lr_b, float beta1, float beta2, float eps, float bc1, float bc2, int64_t n_alpha,
     int64_t n_beta) {
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * ADAM_ROWS_PER_BLOCK + (threadIdx.x >> 5);
+  constexpr int LANES = 32 * WPR;
+  const int lane = threadIdx.x % LANES;
+  const int r = blockIdx.x * (ADAM_ROWS_PER_BLOCK / WPR) + threadIdx.x / LANES;
   if (r >= R) return;
   const int b = r / K, k = r - b * K;
   const int p = bt.prop_of[b];
   if (p < 0 || p >= P) return;
   const float cur = lb_t[r];
-  const bool improved = cur > best_lb[r];
+  const bool improved = cur > best_lb[r];   // (before the row's last lines change it)
   const float ib1 = 1.f / bc1, ib2 = 1.f / bc2;
   const int Up = U[p];
   const long long abase = bt.alpha_off[b] + (long long)k * Up;
@@ -1176,10 +1233,10 @@ __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(
     v0 = min(aend, (abase + 3) & ~3LL);
     v1 = v0 + ((aend - v0) & ~3LL);
   }
-  for (long long i = abase + lane; i < v0; i += 32) one(i);
-  for (long long i = v1 + lane; i < aend; i += 32) one(i);
+  for (long long i = abase + lane; i < v0; i += LANES) one(i);
+  for (long long i = v1 + lane; i < aend; i += LANES) one(i);
 #pragma unroll 2
-  for (long long i = v0 + 4 * lane; i < v1; i += 128) {
+  for (long long i = v0 + 4 * lane; i < v1; i += 4 * LANES) {
     const float4 th = *reinterpret_cast<const float4*>(a_cur + i);
     const float4 g = *reinterpret_cast<const float4*>(ga + i);
     float4 m = *reinterpret_cast<const float4*>(ma + i);
@@ -1196,7 +1253,7 @@ __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(
   }
   const int cnt = bt.split_cnt[b];
   const long long bbase = (long long)bt.split_off[b] * K + (long long)k * cnt;
-  for (int t = lane; t < cnt; t += 32) {
+  for (int t = lane; t < cnt; t += LANES) {
     const long long i = bbase + t;
     if (i < 0 || i >= n_beta) break;
     float th = b_cur[i];
@@ -1209,7 +1266,8 @@ __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(
     th += lr_b * (m / bc1) / (sqrtf(v / bc2) + eps);
     b_cur[i] = fmaxf(th, 0.f);
   }
-  __syncwarp();
+  if (WPR > 1) __syncthreads();   // (one row a block: no thread has left)
+  else __syncwarp();
   if (lane == 0 && improved) best_lb[r] = cur;
 }
 
@@ -1456,8 +1514,27 @@ void launch_tables(int P, int H, const float* l, const float* u, Tables& t, uint
 
 void launch_absw_m(const LayerGeom& g, const float* W, int P, int H, long long hoff_i, long long hoff_prev,
                    const float* u, const float* x_lo, const float* x_hi, int d0, float* wm, cudaStream_t s) {
-  long long n = (long long)P * g.d_out;
-  if (n > 0) { k_absw_m<<<grid1d(n * 32, 256), 256, 0, s>>>(g, W, P, H, hoff_i, hoff_prev, u, x_lo, x_hi, d0, wm); ++g_launches; }
+  const bool fc = g.kind == BCROWN_LAYER_FC;
+  const int hw = fc ? 1 : g.out_h * g.out_w;
+  const long long per = fc ? g.d_out : (long long)g.out_c * ((hw + ABSW_G - 1) / ABSW_G);
+  AbswDiv dv{};
+  dv.groups.set((uint32_t)per);
+  if (!fc) {
+    dv.ow.set(g.out_w);
+    dv.kk.set(g.k * g.k);
+    dv.k.set(g.k);
+  }
+  // whole properties per launch, so that a warp's index stays below 2^31
+  const int step = (int)std::max<long long>(1, ((1LL << 31) - 1) / std::max<long long>(1, per));
+  for (int p0 = 0; p0 < P; p0 += step) {
+    const int np = std::min(step, P - p0);
+    const long long n = per * np;
+    if (n <= 0) continue;
+    k_absw_m<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(g, dv, W, np, H, hoff_i, hoff_prev, u + (size_t)p0 * H,
+                                                     x_lo + (size_t)p0 * d0, x_hi + (size_t)p0 * d0, d0,
+                                                     wm + (size_t)p0 * H, (uint32_t)n);
+    ++g_launches;
+  }
 }
 
 void launch_init_top(bool cert, const RowsCtx& c, int dtop, const bcrown_net* net, long long hoff_top, float* A,
@@ -1587,12 +1664,16 @@ void launch_adam(int R, int K, const BatchView& bt, const int32_t* U, int P, con
                  const float* gb, float* mb, float* vb, float lr_a, float lr_b, float beta1, float beta2, float eps,
                  float bc1, float bc2, int64_t n_alpha, int64_t n_beta, cudaStream_t s) {
   if (R <= 0) return;
-  if (R > 0) {
-    k_adam<<<(R + ADAM_ROWS_PER_BLOCK - 1) / ADAM_ROWS_PER_BLOCK, 32 * ADAM_ROWS_PER_BLOCK, 0, s>>>(
+  // a block per row where rows have many alphas (a warp would walk them 128 at a time)
+  if (n_alpha >= 2048LL * R)
+    k_adam<ADAM_ROWS_PER_BLOCK><<<R, 32 * ADAM_ROWS_PER_BLOCK, 0, s>>>(
         R, K, bt, U, P, lb_t, best_lb, a_cur, a_best, ga, ma, va, b_cur, b_best, gb, mb, vb, lr_a, lr_b, beta1, beta2,
         eps, bc1, bc2, n_alpha, n_beta);
-    ++g_launches;
-  }
+  else
+    k_adam<1><<<(R + ADAM_ROWS_PER_BLOCK - 1) / ADAM_ROWS_PER_BLOCK, 32 * ADAM_ROWS_PER_BLOCK, 0, s>>>(
+        R, K, bt, U, P, lb_t, best_lb, a_cur, a_best, ga, ma, va, b_cur, b_best, gb, mb, vb, lr_a, lr_b, beta1, beta2,
+        eps, bc1, bc2, n_alpha, n_beta);
+  ++g_launches;
 }
 
 void launch_adam16(int R, int K, const BatchView& bt, const int32_t* U, int P, const float* lb_t, float* best_lb,
