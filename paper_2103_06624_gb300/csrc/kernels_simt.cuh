@@ -81,6 +81,8 @@ __device__ __forceinline__ void split_mask_block(const SplitSlot* slots, int ns,
 }
 __device__ __forceinline__ bool split_bit(const uint32_t* mask, int j) { return (mask[j >> 5] >> (j & 31)) & 1u; }
 
+__device__ __forceinline__ bool is_unstable(float lv, float uv) { return lv < 0.f && uv > 0.f; }
+
 // Valid-layer check for splits across all layers (done once per row by the init kernel).
 __device__ __forceinline__ bool row_prop(const RowsCtx& c, int rl, int* b, int* k, int* p) {
   int r = c.r0 + rl;

@@ -1,0 +1,291 @@
+// The FP32 bound and gradient of a small fully connected network in one launch: a row (subdomain,
+// specification) walks its whole chain -- the tables of its property, relaxation and contraction of
+// every layer, concretisation, the minimising corner and the adjoint pass -- with everything but the
+// weights in shared memory.
+//
+// Layer by layer the path is a launch or two per layer and pass, each of a few blocks: 16-32-32-4,
+// 192 rows, bound and gradient: 12 launches, 57 us, of which no kernel has 2 us of work.  Here a
+// warp takes the row (four rows a block) where no layer is wider than ROWS_WARP_WIDTH, else a block
+// of 256 threads; a thread owns every 32nd or 256th output of a contraction and runs its sum in the
+// order of the GEMM (one chain of FMAs over k), the weights' loads of 8 terms in flight.
+#include <algorithm>
+#include <atomic>
+
+#include "simt.cuh"
+
+namespace bcrown {
+
+extern std::atomic<long long> g_launches;
+
+namespace {
+
+constexpr int ROWS_MAXL = 16;          // layers
+constexpr int ROWS_H = 2048;           // hidden neurons
+constexpr int ROWS_D0 = 2048;          // inputs
+constexpr int ROWS_WIDTH = 512;        // widest hidden layer
+constexpr int ROWS_WARP_WIDTH = 64;    // widest layer of the form with one warp per row
+constexpr int ROWS_BLOCK = 256, ROWS_WARP_ROWS = 4;
+
+struct RowsNet {
+  int L, H, mw;                        // mw: widest layer, the input included
+  int d[ROWS_MAXL + 1], hoff[ROWS_MAXL + 1];
+  const float *W[ROWS_MAXL + 1], *Wt[ROWS_MAXL + 1], *b[ROWS_MAXL + 1];
+  const float *Wbar, *bbar;
+};
+
+__host__ __device__ constexpr int rows_floats(int H, int mw) { return 5 * H + 3 * mw; }
+
+template <int T>
+__device__ __forceinline__ void row_sync() {
+  if (T > 32) __syncthreads();
+  else __syncwarp();
+}
+
+// y[n] = sum_k x[k] w[k][n] over n = t, t + T, ..: store(n, sum).  One chain over k, 8 loads in flight.
+// (16, or two batches of 16 in turn, or outputs side by side cost more in resident rows than they
+// gained: 37-300-260-5, 512 rows 53 us with this one, 75 to 95 with those.)
+template <int T, class F>
+__device__ __forceinline__ void row_product(const float* x, const float* __restrict__ w, int K, int N, int t, F store) {
+  for (int n = t; n < N; n += T) {
+    const float* wp = w + n;
+    float acc = 0.f;
+    int k = 0;
+    for (; k + 8 <= K; k += 8) {
+      float wv[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) wv[e] = __ldg(wp + (size_t)(k + e) * N);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc = fmaf(x[k + e], wv[e], acc);
+    }
+    for (; k < K; ++k) acc = fmaf(x[k], __ldg(wp + (size_t)k * N), acc);
+    store(n, acc);
+  }
+}
+
+template <int T>   // threads per row: 32 (ROWS_WARP_ROWS rows a block) or the block
+__global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T)
+    k_rows(const RowsNet net, RowsCtx c, const float* __restrict__ alpha, int64_t n_alpha,
+           const float* __restrict__ beta, int64_t n_beta, float* __restrict__ lb, float* __restrict__ xstar,
+           bool grad, float* __restrict__ dalpha, float* __restrict__ dbeta) {
+  extern __shared__ __align__(16) float rows_smem[];
+  __shared__ float red[T / 32];
+  __shared__ int tot[T / 32];
+  const int t = threadIdx.x % T, lane = threadIdx.x & 31, w = t >> 5;
+  const int rl = blockIdx.x * (T == 32 ? ROWS_WARP_ROWS : 1) + threadIdx.x / T;
+  if (rl >= c.R) return;   // (whole rows: a warp, or no thread of the block)
+  const int H = net.H, L = net.L;
+  float* A = rows_smem + (size_t)(threadIdx.x / T) * rows_floats(H, net.mw);
+  float *D = A + H, *lm = D + H;
+  int *rank = reinterpret_cast<int*>(lm + H), *sp = rank + H;
+  float *Lam = reinterpret_cast<float*>(sp + H), *h = Lam + net.mw, *z = h + net.mw;
+
+  int b, k, p;
+  const bool ok = row_prop(c, rl, &b, &k, &p);
+  if (!ok) {
+    if (t == 0) flag(c.status, BCROWN_ERR_ARG);
+    p = 0;
+  }
+  const int off = c.bt.split_off[b], cnt = c.bt.split_cnt[b];
+  if ((cnt < 0 || cnt > BCROWN_MAX_SPLITS) && t == 0) flag(c.status, BCROWN_ERR_ARG);
+  const int ns = cnt < 0 || cnt > BCROWN_MAX_SPLITS ? 0 : cnt;
+
+  // the property's table (as k_tables): D, lambda of a stable neuron, the chord and the rank of an unstable one
+  const float *lp = c.l + (size_t)p * H, *up = c.u + (size_t)p * H;
+  int U = 0;
+  for (int n0 = 0; n0 < H; n0 += T) {
+    const int n = n0 + t;
+    const float lv = n < H ? lp[n] : 0.f, uv = n < H ? up[n] : 0.f;
+    const bool un = n < H && is_unstable(lv, uv);
+    const unsigned m = __ballot_sync(0xffffffffu, un);
+    int r = U + __popc(m & ((1u << lane) - 1u));
+    U += __popc(m);
+    if (T > 32) {
+      U -= __popc(m);
+      if (lane == 0) tot[w] = __popc(m);
+      __syncthreads();
+      int all = 0;
+#pragma unroll
+      for (int q = 0; q < T / 32; ++q) {
+        if (q < w) r += tot[q];
+        all += tot[q];
+      }
+      U += all;
+      __syncthreads();
+    }
+    if (n < H) {
+      const float sl = un ? __fdiv_ru(uv, __fsub_rd(uv, lv)) : (lv >= 0.f ? 1.f : 0.f);
+      rank[n] = un ? r : -1;
+      D[n] = sl;
+      lm[n] = un ? __fmul_ru(sl, -lv) : 0.f;
+      sp[n] = 0;
+    }
+  }
+  for (int j = t; j < net.d[L - 1]; j += T) (L > 1 ? A + net.hoff[L - 1] : h)[j] = net.Wbar[(size_t)k * net.d[L - 1] + j];
+  row_sync<T>();
+  // the row's splits: sp = 2 (place in the list + 1) + (sign > 0), the last of a neuron's
+  for (int q = t; q < ns; q += T) {
+    const int ly = c.bt.split_layer[off + q], sg = c.bt.split_sign[off + q];
+    const long long j = c.bt.split_idx[off + q];
+    if (sg != -1 && sg != 1) flag(c.status, BCROWN_ERR_ARG);
+    else if (ly >= 1 && ly < L) {
+      if (j >= net.d[ly]) flag(c.status, BCROWN_ERR_ARG);
+      else atomicMax(sp + net.hoff[ly] + (int)j, 2 * (q + 1) + (sg > 0 ? 1 : 0));
+    }
+  }
+  row_sync<T>();
+
+  const long long abase = c.bt.alpha_off[b] + (long long)k * U;
+  const long long bbase = (long long)off * c.K + (long long)k * cnt;
+  float acc = 0.f;
+  for (int i = L - 1; i >= 1; --i) {
+    const int d = net.d[i], o = net.hoff[i];
+    for (int j = t; j < d; j += T) {
+      const int n = o + j, s2 = sp[n];
+      const float a = A[n];
+      float Dn = D[n], ln = lm[n], bs = 0.f;
+      if (s2) {
+        const long long bi = bbase + (s2 >> 1) - 1;
+        const float sg = s2 & 1 ? 1.f : -1.f;
+        if (bi >= 0 && bi < n_beta) bs = fmaxf(beta[bi], 0.f) * sg;
+        else flag(c.status, BCROWN_ERR_ARG);
+        Dn = s2 & 1 ? 0.f : 1.f;
+        ln = 0.f;
+      } else if (rank[n] >= 0 && a >= 0.f) {
+        const long long ai = abase + rank[n];
+        ln = 0.f;
+        if (ai < 0 || ai >= n_alpha) {
+          flag(c.status, BCROWN_ERR_ARG);
+          Dn = 0.f;
+        } else {
+          Dn = fminf(fmaxf(alpha[ai], 0.f), 1.f);
+        }
+      }
+      D[n] = Dn;
+      lm[n] = ln;
+      const float lam = fmaf(a, Dn, bs);
+      Lam[j] = lam;
+      acc = fmaf(lam, net.b[i][j], fmaf(a, ln, acc));
+    }
+    row_sync<T>();
+    float* out = i > 1 ? A + net.hoff[i - 1] : h;
+    row_product<T>(Lam, net.W[i], d, net.d[i - 1], t, [&](int n, float v) { out[n] = v; });
+    row_sync<T>();
+  }
+  // concretisation, and the corner that attains it
+  const float *xl = c.x_lo + (size_t)p * net.d[0], *xh = c.x_hi + (size_t)p * net.d[0];
+  for (int m = t; m < net.d[0]; m += T) {
+    const float a = h[m];
+    acc += fminf(a * xl[m], a * xh[m]);
+    const float x = a >= 0.f ? xl[m] : xh[m];
+    if (xstar) xstar[(size_t)(c.r0 + rl) * net.d[0] + m] = x;
+    h[m] = x;
+  }
+  acc = warp_sum(acc);
+  if (T > 32) {
+    if (lane == 0) red[w] = acc;
+    __syncthreads();
+    acc = 0.f;
+#pragma unroll
+    for (int q = 0; q < T / 32; ++q) acc += red[q];
+  } else {
+    __syncwarp();
+  }
+  if (t == 0) {
+    float out = (ok ? net.bbar[k] : -INFINITY) + acc;
+    if (!isfinite(out)) {
+      flag(c.status, BCROWN_ERR_NONFINITE);
+      out = -INFINITY;
+    }
+    lb[c.r0 + rl] = out;
+  }
+  if (!grad) return;
+  for (int i = 1; i < L; ++i) {
+    const int o = net.hoff[i];
+    row_product<T>(h, net.Wt[i], net.d[i - 1], net.d[i], t, [&](int j, float v) {
+      const int n = o + j, s2 = sp[n];
+      const float zj = v + net.b[i][j], a = A[n];
+      if (rank[n] >= 0) {
+        const long long ai = abase + rank[n];
+        if (ai < 0 || ai >= n_alpha) flag(c.status, BCROWN_ERR_ARG);
+        else dalpha[ai] = !s2 && a >= 0.f ? a * zj : 0.f;
+      }
+      if (s2) {
+        const long long bi = bbase + (s2 >> 1) - 1;
+        if (bi >= 0 && bi < n_beta) dbeta[bi] = s2 & 1 ? zj : -zj;
+        else flag(c.status, BCROWN_ERR_ARG);
+      }
+      z[j] = fmaf(D[n], zj, lm[n]);
+    });
+    row_sync<T>();
+    float* sw = h;
+    h = z;
+    z = sw;
+  }
+}
+
+int widest(const bcrown_net* net) {
+  int w = net->d[0];
+  for (int i = 1; i < net->L; ++i) w = std::max(w, net->d[i]);
+  return w;
+}
+
+}  // namespace
+
+int rows_load() {
+  const int smem = rows_floats(ROWS_H, ROWS_D0) * 4;
+  for (cudaError_t e : {cudaFuncSetAttribute(k_rows<ROWS_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                        cudaFuncSetAttribute(k_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)})
+    if (e != cudaSuccess) return fail(BCROWN_ERR_CUDA, "row kernel: shared memory");
+  return BCROWN_OK;
+}
+
+// Which calls take it (times of calls, bound and gradient, this kernel / layer by layer).  The warp
+// form, always: a pass per layer over rows this short costs more than the whole chain (16-32-32-4:
+// 192 rows 30 us / 58, 3,072 33 / 70, 196,608 288 / 1,176; the first two are the host's time for a
+// call).  The block form reads the weights once per row, so it is for the rows that leave the GEMM's
+// tiles empty, up to 2^27 FMAs per pass: 37-300-260-5, 64 rows 43 / 103, 2,048 rows (1.8e8 FMAs)
+// 140 / 134; 64-128x3-10, 2,304 rows (0.9e8) 75 / 118, 9,216 (3.8e8) 257 / 191; 784-256x6-10, 72 rows
+// 107 / 252, 1,152 (6.1e8) 344 / 280.  Layers over 512 neurons stay with the GEMM: a thread's chains
+// follow one another there (100-1000-900-10, 9 rows 194 / 172).  A bound and a gradient of the same
+// batch take the same kernel.
+constexpr long long ROWS_FMAS = 1LL << 27;
+
+static bool warp_form(const bcrown_net* net) { return widest(net) <= ROWS_WARP_WIDTH && net->H <= ROWS_H / 4; }
+
+bool rows_supported(const bcrown_net* net, long long R) {
+  if (net->L > ROWS_MAXL || net->H > ROWS_H || net->d[0] > ROWS_D0) return false;
+  long long fma = 0;
+  for (int i = 1; i < net->L; ++i) {
+    if (net->ly[i - 1].kind != BCROWN_LAYER_FC || net->d[i] > ROWS_WIDTH) return false;
+    fma += (long long)net->d[i] * net->d[i - 1];
+  }
+  return warp_form(net) || R * fma <= ROWS_FMAS;
+}
+
+int rows_bound(const bcrown_net* net, const RowsCtx& c, const float* alpha, int64_t n_alpha, const float* beta,
+               int64_t n_beta, float* lb, float* xstar, bool grad, float* dalpha, float* dbeta, cudaStream_t s) {
+  RowsNet n{};
+  n.L = net->L;
+  n.H = net->H;
+  n.mw = widest(net);
+  n.Wbar = net->Wbar;
+  n.bbar = net->bbar;
+  for (int i = 0; i < net->L; ++i) n.d[i] = net->d[i];
+  for (int i = 1; i < net->L; ++i) {
+    n.hoff[i] = (int)net->hoff[i - 1];
+    n.W[i] = net->ly[i - 1].W;
+    n.Wt[i] = net->ly[i - 1].Wt;
+    n.b[i] = net->ly[i - 1].b;
+  }
+  const int smem = rows_floats(n.H, n.mw) * 4;
+  if (warp_form(net))
+    k_rows<32><<<(c.R + ROWS_WARP_ROWS - 1) / ROWS_WARP_ROWS, 32 * ROWS_WARP_ROWS, ROWS_WARP_ROWS * smem, s>>>(
+        n, c, alpha, n_alpha, beta, n_beta, lb, xstar, grad, dalpha, dbeta);
+  else
+    k_rows<ROWS_BLOCK><<<c.R, ROWS_BLOCK, smem, s>>>(n, c, alpha, n_alpha, beta, n_beta, lb, xstar, grad, dalpha,
+                                                     dbeta);
+  ++g_launches;
+  return BCROWN_OK;
+}
+
+}  // namespace bcrown

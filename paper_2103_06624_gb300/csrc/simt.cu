@@ -22,8 +22,6 @@ std::atomic<long long> g_launches{0};
 // from the offset in its first slot, which only its own block reads and overwrites.
 constexpr int TAB_SEG = 4096;
 
-__device__ __forceinline__ bool is_unstable(float lv, float uv) { return lv < 0.f && uv > 0.f; }
-
 __global__ void __launch_bounds__(1024) k_tables_count(int H, const float* __restrict__ l,
                                                        const float* __restrict__ u, int32_t* rank) {
   __shared__ int tot;

@@ -46,6 +46,13 @@ void launch_fill(float* p, long long n, float v, cudaStream_t s);
 // into stride phases (backward), and the convolution plus bias (forward), for R rows.
 constexpr int SCONV_MAX_K = 4096;   // terms per output the staged gather table holds
 bool sconv_supported(const bcrown_net* net, int i);
+// rows.cu: the FP32 bound (and gradient, and minimising corner) of a small fully connected network in
+// one launch.  c.tb is not read: a row works out its property's table itself.
+int rows_load();
+bool rows_supported(const bcrown_net* net, long long R);
+int rows_bound(const bcrown_net* net, const RowsCtx& c, const float* alpha, int64_t n_alpha, const float* beta,
+               int64_t n_beta, float* lb, float* xstar, bool grad, float* dalpha, float* dbeta, cudaStream_t s);
+
 int sconv_load(bcrown_net* net);   // builds the tables (at bcrown_load_net)
 int sconv_bwd(bcrown_net* net, int i, int R, const float* Lam, float* Ain, cudaStream_t s);
 int sconv_fwd(bcrown_net* net, int i, int R, const float* h, float* Z, const float* bias, cudaStream_t s);

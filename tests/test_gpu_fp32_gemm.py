@@ -48,3 +48,15 @@ def test_gemm_tiles(widths, B):
         want = np.asarray(want).reshape(-1)
         if want.size:   # entry by entry within 1e-3 of |g| + 1e-3 max |g|, as the gradient tests hold it
             assert (np.abs(got - want) <= 1e-3 * (np.abs(want) + 1e-3 * np.abs(want).max())).all()
+
+
+@pytest.mark.parametrize("widths", [[7, 33, 31, 3], [33, 65, 63, 5], [32, 64, 128, 4], [36, 68, 132, 4], [8, 129, 4, 3]])
+@pytest.mark.parametrize("n", [1, 31, 33, 192])
+def test_gemm_tiles_forward(widths, n):
+    """The plain forward pass takes the GEMM at every size (bounds of small networks do not)."""
+    pb = wl.make_problem("gemm", wl.mlp_layers(widths, 5), 1, 0.08, 2, 5)
+    net = bc.load_net(pb.layers, pb.C)
+    x = np.random.default_rng(n).uniform(0, 1, (n, widths[0])).astype(np.float32)
+    ref = O.OracleNet(pb.layers, pb.C).forward(x)
+    got = bc.forward(net, torch.from_numpy(x).cuda()).cpu().numpy()
+    assert got.shape == ref.shape and np.max(rel_err(got, ref)) <= RTOL
