@@ -36,6 +36,7 @@ struct SconvPass {
   const float* B;  // [K][N] weights
   int ky0, kx0;    // the phase's first tap (B depends on nothing else)
   int ntap;        // taps of the phase
+  int nky, nkx;    // its rows and columns of taps, 0 in a forward pass
 };
 // A layer's stride phases, contracted by one launch.
 constexpr int SC_PHASES = 4;
@@ -59,7 +60,7 @@ __device__ __forceinline__ long long sc_out(const SconvPass& q, uint32_t m, long
 // (48 % of its peak at 128 channels, 71 % at 32, where a gathered value feeds fewest FMAs) together
 // with the FMA pipe; a third stage costs a resident block and is 3 % slower.  2,997 rows of the
 // 32 -> 64 channel 4x4 stride-2 layer backward: 668 us in four launches with 8 x 2 outputs a thread
-// and register staging, 420 with bounds tested per value and the lanes in row order, 347 now; 576
+// and register staging, 420 with bounds tested per value and the lanes in row order, 335 now; 576
 // rows of the 128 -> 128 channel 3x3 stride-2 layer 353 -> 271.
 constexpr int SC_BM = 128, SC_BK = 16, SC_STAGES = 2;
 constexpr int SC_AP = SC_BM + 4;
@@ -248,8 +249,8 @@ __global__ void __launch_bounds__(2 * BN, BN == 32 ? 7 : 256 / BN)
 //
 // Which taps of a row lie inside the map is one bit each, worked out once, and 8 terms' loads (32 a
 // thread) are in flight together: with the bounds tested per term and 2 terms at a time the kernel
-// waited for its loads three quarters of the time.  All stride phases are one launch.  2,997 rows of
-// 3 x 32 x 32 from 32 channels: 185 us.
+// waited for its loads three quarters of the time.  All stride phases are one launch.  Layers whose taps
+// share a window go to k_sconv_cells.
 constexpr int SN_THREADS = 256, SN_TM = 4;
 
 template <int N>
@@ -341,6 +342,139 @@ __global__ void __launch_bounds__(SN_THREADS) k_sconv_narrow(const SconvPhases p
   }
 }
 
+// The common first layers' backward pass (3x3 stride 1, 4x4 stride 2; at most 4 input channels): a
+// thread takes cells of 2 x 2 outputs, whose taps lie in one (T + SH) x (T + SH) window of the source,
+// so a value is loaded once for the outputs that share it (9 loads a channel instead of 16 with 4x4
+// stride 2, 16 instead of 36 with 3x3): k_sconv_narrow is bound by its loads and what surrounds them.
+// Output (2 i + a, 2 j + b), tap (dy, dx) reads window row SH a + T - 1 - dy and column SH b + T - 1 - dx:
+// T = 3, SH = 1 for 3x3 stride 1, T = 2 for 4x4 stride 2 with SH the padding's parity.  Every output's
+// sum has the order of the general pass.  2,997 rows of 3 x 32 x 32 from 32 channels (4x4 stride 2):
+// k_sconv_narrow 183 us, here 109; 576 rows from 64 channels (3x3) 169 / 83; 1,024 rows of 18 x 18
+// patches (padding 0) 57 / 28.
+struct SconvCells {
+  uint32_t M;        // cells of all rows
+  int Pm, nJ;        // cells of a row, and of a row of cells
+  FastDiv dPm, dnJ;
+  int Hs, Ws, C;     // source map, its channels
+  long long HWs;
+  int ms, cy, cx;    // window origin of cell (i, j): (i ms + cy, j ms + cx)
+  int Ho, Wo;
+  long long HWo;
+  const float* B[4]; // [C T T][N] weights of output (a, b) of a cell, at 2 a + b (stride 1: one for all)
+};
+constexpr int SL_THREADS = 128, SL_CELLS = 2;   // cells a thread
+
+template <int N, int T, int SH>
+__global__ void __launch_bounds__(SL_THREADS) k_sconv_cells(const SconvCells q, const float* __restrict__ src,
+                                                           long long sstride, float* __restrict__ out,
+                                                           long long ostride) {
+  constexpr int W = T + SH, TT = T * T, NP = T == 3 ? 1 : 4;
+  extern __shared__ __align__(16) uint8_t sl_raw[];
+  float4* sB = reinterpret_cast<float4*>(sl_raw);   // [C][NP][T T]
+  for (int e = threadIdx.x; e < q.C * NP * TT; e += SL_THREADS) {
+    const int t = e % TT, ph = e / TT % NP, c = e / (TT * NP);
+    const float* b = (ph == 0 ? q.B[0] : ph == 1 ? q.B[1] : ph == 2 ? q.B[2] : q.B[3]) + (size_t)(c * TT + t) * N;
+    sB[e] = make_float4(b[0], N > 1 ? b[1] : 0.f, N > 2 ? b[2] : 0.f, N > 3 ? b[3] : 0.f);
+  }
+  __syncthreads();
+  const float* win[SL_CELLS];
+  uint32_t in[SL_CELLS];
+  long long at[SL_CELLS];
+  int edge[SL_CELLS];   // bit 0: a second row of outputs, bit 1: a second column, bit 2: any
+#pragma unroll
+  for (int u = 0; u < SL_CELLS; ++u) {
+    const uint32_t m = blockIdx.x * (uint32_t)(SL_THREADS * SL_CELLS) + u * SL_THREADS + threadIdx.x;
+    const bool mv = m < q.M;
+    const uint32_t r = mv ? q.dPm(m) : 0u;
+    const int pp = mv ? (int)(m - r * (uint32_t)q.Pm) : 0;
+    const int ci = (int)q.dnJ((uint32_t)pp), cj = pp - ci * q.nJ;
+    const int y0 = ci * q.ms + q.cy, x0 = cj * q.ms + q.cx;
+    win[u] = src + (long long)r * sstride + ((long long)y0 * q.Ws + x0);
+    in[u] = 0u;
+#pragma unroll
+    for (int y = 0; y < W; ++y)
+#pragma unroll
+      for (int x = 0; x < W; ++x)
+        if (mv && (unsigned)(y0 + y) < (unsigned)q.Hs && (unsigned)(x0 + x) < (unsigned)q.Ws) in[u] |= 1u << (y * W + x);
+    at[u] = (long long)r * ostride + (long long)(2 * ci) * q.Wo + 2 * cj;
+    edge[u] = mv ? 4 | (2 * ci + 1 < q.Ho ? 1 : 0) | (2 * cj + 1 < q.Wo ? 2 : 0) : 0;
+  }
+  float acc[SL_CELLS][4][N];
+#pragma unroll
+  for (int u = 0; u < SL_CELLS; ++u)
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+      for (int n = 0; n < N; ++n) acc[u][o][n] = 0.f;
+  for (int c = 0; c < q.C; ++c) {
+    float v[SL_CELLS][W * W];
+#pragma unroll
+    for (int u = 0; u < SL_CELLS; ++u) {
+#pragma unroll
+      for (int y = 0; y < W; ++y) {
+        const float* row = win[u] + (long long)y * q.Ws;
+#pragma unroll
+        for (int x = 0; x < W; ++x) {
+          v[u][y * W + x] = 0.f;
+          if ((in[u] >> (y * W + x)) & 1u) v[u][y * W + x] = row[x];
+        }
+      }
+      win[u] += q.HWs;
+    }
+    const float4* wc = sB + c * NP * TT;
+#pragma unroll
+    for (int ph = 0; ph < NP; ++ph)
+#pragma unroll
+      for (int dy = 0; dy < T; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < T; ++dx) {
+          const float4 b4 = wc[ph * TT + dy * T + dx];
+          const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            if (NP == 4 && o != ph) continue;
+            const int a = o >> 1, b = o & 1;
+            const int e = (SH * a + T - 1 - dy) * W + SH * b + T - 1 - dx;
+#pragma unroll
+            for (int u = 0; u < SL_CELLS; ++u)
+#pragma unroll
+              for (int n = 0; n < N; ++n) acc[u][o][n] = fmaf(v[u][e], bv[n], acc[u][o][n]);
+          }
+        }
+  }
+  const bool pairs = ((q.Wo | (int)(q.HWo & 1) | (int)(ostride & 1)) & 1) == 0 &&
+                     (reinterpret_cast<uintptr_t>(out) & 7) == 0;
+#pragma unroll
+  for (int u = 0; u < SL_CELLS; ++u) {
+    if (!edge[u]) continue;
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        if (a && !(edge[u] & 1)) continue;
+        float* o = out + at[u] + n * q.HWo + (long long)a * q.Wo;
+        if (pairs) {
+          *reinterpret_cast<float2*>(o) = make_float2(acc[u][2 * a][n], acc[u][2 * a + 1][n]);
+        } else {
+          o[0] = acc[u][2 * a][n];
+          if (edge[u] & 2) o[1] = acc[u][2 * a + 1][n];
+        }
+      }
+  }
+}
+
+constexpr int SL_SMEM = 96 * 1024;
+int sconv_cells_smem(int C, int T) { return C * (T == 3 ? 9 : 16) * (int)sizeof(float4); }
+
+template <int T, int SH>
+cudaError_t cells_attr() {
+  cudaError_t e = cudaFuncSetAttribute(k_sconv_cells<1, T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sconv_cells<2, T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sconv_cells<3, T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sconv_cells<4, T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
+  return e;
+}
+
 int sconv_narrow_smem(int K) { return K * (int)(sizeof(int4) + sizeof(float4)); }
 
 int sconv_smem(int BN, int K) {
@@ -426,6 +560,8 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
         q.ky0 = ky0;
         q.kx0 = kx0;
         q.ntap = std::max(1, nky * nkx);
+        q.nky = nky;
+        q.nkx = nkx;
         q.dPm.set(q.Pm);
         q.dnJ.set(q.nJ);
         std::vector<int4> tab((size_t)q.K, make_int4(0, -32768, 0, 0));
@@ -505,6 +641,9 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
       if (e != cudaSuccess)
         return fail(BCROWN_ERR_CUDA, std::string("FP32 conv: smem attribute: ") + cudaGetErrorString(e));
   }
+  for (cudaError_t e : {cells_attr<3, 1>(), cells_attr<2, 1>(), cells_attr<2, 0>()})
+    if (e != cudaSuccess)
+      return fail(BCROWN_ERR_CUDA, std::string("FP32 conv: smem attribute: ") + cudaGetErrorString(e));
   for (int BN : {16, 32, 64, 128}) {
     const int smem = sconv_smem(BN, SCONV_MAX_K);
     cudaError_t e = BN == 16    ? cudaFuncSetAttribute(k_sconv<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
@@ -517,9 +656,59 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
   return BCROWN_OK;
 }
 
+template <int T, int SH>
+void cells_launch(int N, unsigned grid, int smem, const SconvCells& c, const float* src, long long sstride, float* out,
+                  long long ostride, cudaStream_t s) {
+  auto go = [&](auto* k) { k<<<grid, SL_THREADS, smem, s>>>(c, src, sstride, out, ostride); };
+  if (N == 1) go(k_sconv_cells<1, T, SH>);
+  else if (N == 2) go(k_sconv_cells<2, T, SH>);
+  else if (N == 3) go(k_sconv_cells<3, T, SH>);
+  else go(k_sconv_cells<4, T, SH>);
+}
+
+// A backward contraction that the cells' kernel takes (its geometry is in the passes); false: it does not.
+bool cells_try(const SconvPass* q, int n, int R, const float* src, long long sstride, float* out, long long ostride,
+               cudaStream_t s) {
+  if (q[0].N > 4) return false;
+  const bool s1 = n == 1 && q[0].os == 1 && q[0].nky == 3 && q[0].nkx == 3;
+  bool s2 = n == 4 && q[0].os == 2;
+  for (int z = 0; s2 && z < 4; ++z) s2 = q[z].nky == 2 && q[z].nkx == 2 && q[z].oa == z / 2 && q[z].ob == z % 2;
+  if (!s1 && !s2) return false;
+  const int T = s1 ? 3 : 2, SH = s1 ? 1 : q[2].cy - q[0].cy;
+  if (s2 && (q[1].cx - q[0].cx != SH || (SH != 0 && SH != 1))) return false;
+  SconvCells c{};
+  c.C = q[0].K / (T * T);
+  const int smem = sconv_cells_smem(c.C, T);
+  if (smem > SL_SMEM) return false;
+  c.Wo = q[0].Wo;
+  c.HWo = q[0].HWo;
+  c.Ho = (int)(c.HWo / c.Wo);
+  c.nJ = (c.Wo + 1) / 2;
+  c.Pm = (c.Ho + 1) / 2 * c.nJ;
+  const long long M = (long long)R * c.Pm;
+  if (M <= 0 || M >= (1LL << 31)) return false;
+  c.M = (uint32_t)M;
+  c.dPm.set(c.Pm);
+  c.dnJ.set(c.nJ);
+  c.Hs = q[0].Hs;
+  c.Ws = q[0].Ws;
+  c.HWs = q[0].HWs;
+  c.ms = s1 ? 2 : 1;
+  c.cy = q[0].cy - (T - 1);
+  c.cx = q[0].cx - (T - 1);
+  for (int z = 0; z < 4; ++z) c.B[z] = q[s1 ? 0 : z].B;
+  const unsigned grid = (unsigned)((M + SL_THREADS * SL_CELLS - 1) / (SL_THREADS * SL_CELLS));
+  if (s1) cells_launch<3, 1>(q[0].N, grid, smem, c, src, sstride, out, ostride, s);
+  else if (SH) cells_launch<2, 1>(q[0].N, grid, smem, c, src, sstride, out, ostride, s);
+  else cells_launch<2, 0>(q[0].N, grid, smem, c, src, sstride, out, ostride, s);
+  ++g_launches;
+  return true;
+}
+
 // The n passes of one contraction (a layer's stride phases, or its forward pass) for R rows.
 int sc_launch(const SconvPass* qs, int n, int R, const float* src, long long sstride, float* out, long long ostride,
               const float* bias, cudaStream_t s) {
+  if (!bias && cells_try(qs, n, R, src, sstride, out, ostride, s)) return BCROWN_OK;
   for (int i0 = 0; i0 < n; i0 += SC_PHASES) {
     SconvPhases ph{};
     const int nz = std::min(SC_PHASES, n - i0);

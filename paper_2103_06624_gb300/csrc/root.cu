@@ -146,8 +146,8 @@ __device__ __forceinline__ void root_origin(const RootCtx& c, const RootMap& m, 
 // Bound by the latency of its loads (A, l, u, bias and the error weight per element).  A thread takes
 // four elements at a time with all their loads issued together: four neighbours by 16-byte loads
 // where the row is the whole map and every array lies on a 16-byte boundary (VEC), else four a block
-// apart.  1,024 rows of 8,192 neurons, certified: 62 us one element at a time; of 8,192 patches of
-// 512 elements 44.
+// apart.  1,024 rows of 8,192 neurons, certified: 62 us one element at a time, 28 now; 8,192 patches
+// of 512 elements 44, 46 now.
 template <bool CERT, bool VEC>
 __global__ void __launch_bounds__(256) k_root_relax(RootCtx c, RootMap m, int d, long long hoff, int rule,
                                                     float rule_value, const float* __restrict__ Ain,

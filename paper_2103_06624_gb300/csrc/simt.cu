@@ -169,7 +169,8 @@ __device__ __forceinline__ float hmax_hidden(float uv) { return fmaxf(uv, 0.f); 
 // per 4 neighbouring positions of an output channel: they share the weight's load and the term's
 // index arithmetic, and their 4 chains of rounded sums run side by side.  The loads of 4 terms (of 8
 // for a fully connected layer) are issued together.  Every neuron's sum has the same order whatever
-// the grouping.  576 terms x 32,768 neurons: 65 us, a neuron and a term at a time.
+// the grouping.  576 terms x 32,768 neurons: 65 us
+// a neuron and a term at a time, 23 now.
 struct AbswDiv {
   FastDiv hw, ow, kk, k, groups;
 };
@@ -294,8 +295,11 @@ __global__ void __launch_bounds__(256) k_init_top(RowsCtx c, int dtop, const flo
 // ----------------------------------------------------------------------------------------
 // Relaxation + beta shift + bias (Eq. definition_D, definition_lowerb, definition_A):
 //   Lambda_j = A_j D_j + beta_j S_jj ;  c += Lambda_j b_j + A_j lambda_j
-// One warp per row (RELAX_ROWS rows per block): the row's splits of this layer are compacted
-// into shared memory by ballots, neurons are strided over the lanes, sums are warp reductions.
+// One warp per row (8 rows per block), or a block per row for wide layers: the row's splits of this
+// layer are compacted into shared memory by ballots, with one bit per neuron; a lane takes four
+// neighbouring neurons where the arrays are aligned.  Bound by memory and its latency.  2,997 rows,
+// certified, of 8,192 / 4,096 / 512 neurons: 126 / 80 / 34 us a neuron per lane, 101 / 65 / 19 now;
+// 4,608 rows of 256, not certified, 16.6 / 12.
 // CERT: outward chord constants (from the tables), c summed rounded down, error terms rounded up.
 // ----------------------------------------------------------------------------------------
 constexpr int RELAX_WARPS = 8;   // warps per block; WPR of them share a row (wide layers: all 8)
@@ -1191,7 +1195,7 @@ __device__ __forceinline__ float adam_alpha(float th, float g, float& m, float& 
 
 // One warp per row, or a block for rows of many alphas (WPR warps: launch_adam): the row's alphas in
 // 16-byte accesses where the arrays allow it.  Bound by memory: 32 bytes an alpha, 36 where the row
-// improved.  576 rows of 12,000 alphas: 96 us a warp per row (72 blocks).
+// improved.  576 rows of 12,000 alphas: 96 us a warp per row (72 blocks), 37 a block per row.
 constexpr int ADAM_ROWS_PER_BLOCK = 8;
 template <int WPR>
 __global__ void __launch_bounds__(32 * ADAM_ROWS_PER_BLOCK) k_adam(

@@ -1,6 +1,7 @@
 """The FP32 convolution passes against the FP64 oracle (needs a GB300): output channels at each tile
 width and past it, terms that leave a remainder, maps whose rows are no multiple of four, more stride
-phases than a launch takes, phases without a tap, more than 32 taps in front of a narrow layer."""
+phases than a launch takes, phases without a tap, more than 32 taps in front of a narrow layer, and
+the cells of 2 x 2 outputs over odd and even maps and paddings."""
 import numpy as np
 import pytest
 import torch
@@ -20,6 +21,10 @@ NETS = {
     "nine_phases": ((3, 13, 10), [(5, 4, 3, 1), (6, 3, 1, 1)]),
     "empty_phases": ((4, 9, 9), [(5, 2, 3, 0), (3, 2, 1, 0)]),
     "many_taps": ((2, 9, 11), [(3, 7, 1, 3), (8, 3, 2, 0)]),
+    "cells_stride_2": ((3, 13, 11), [(6, 4, 2, 1), (5, 3, 1, 1)]),   # odd maps: cells half outside
+    "cells_even_padding": ((4, 9, 10), [(5, 4, 2, 0), (3, 2, 1, 0)]),
+    "cells_padding_2": ((1, 8, 8), [(7, 4, 2, 2), (3, 3, 1, 1)]),
+    "cells_stride_1": ((2, 7, 5), [(4, 3, 1, 0), (4, 4, 2, 1)]),
     "pointwise": ((3, 6, 6), [(8, 1, 1, 0), (20, 1, 2, 0)]),
 }
 
