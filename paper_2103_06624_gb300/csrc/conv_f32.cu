@@ -525,9 +525,11 @@ void sc_phase(int a, int k, int s, int pad, int in, int* k0, int* nk, int* off, 
 int sc_prepare(bcrown_net* net, SconvNet* t) {
   if (t->ready) return BCROWN_OK;
   t->ly.assign(net->L, LayerF32());
+  bool any = false;
   for (int i = 1; i <= net->L - 1; ++i) {
     const LayerDev& l = net->ly[i - 1];
     if (!sconv_supported(net, i)) continue;
+    any = true;
     const int k = l.k, s = l.stride, kk = k * k;
     std::vector<float> w((size_t)l.out_c * l.in_c * kk);
     if (cudaMemcpy(w.data(), l.W, w.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -631,6 +633,10 @@ int sc_prepare(bcrown_net* net, SconvNet* t) {
     f.tab = reinterpret_cast<const int4*>(dt);
     f.B = reinterpret_cast<const float*>(dB);
     P.fwd = f;
+  }
+  if (!any) {   // (the attributes below load every kernel, which a net without convolutions need not wait for)
+    t->ready = true;
+    return BCROWN_OK;
   }
   {
     const int smem = sconv_narrow_smem(SCONV_MAX_K);

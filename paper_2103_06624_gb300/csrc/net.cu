@@ -268,7 +268,7 @@ extern "C" int bcrown_load_net(const bcrown_layer* layers, int n_layers, const f
   // (the allocation-free bound included) allocates them
   if (st == BCROWN_OK) st = sconv_load(net);
   if (st == BCROWN_OK) st = sgemm_load();
-  if (st == BCROWN_OK) st = rows_load();
+  if (st == BCROWN_OK) st = rows_load(net);
   if (st != BCROWN_OK) {
     bcrown_free_net(net);
     return st;

@@ -231,7 +231,8 @@ int widest(const bcrown_net* net) {
 
 }  // namespace
 
-int rows_load() {
+int rows_load(const bcrown_net* net) {
+  if (!rows_supported(net, 0)) return BCROWN_OK;
   const int smem = rows_floats(ROWS_H, ROWS_D0) * 4;
   for (cudaError_t e : {cudaFuncSetAttribute(k_rows<ROWS_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                         cudaFuncSetAttribute(k_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)})
