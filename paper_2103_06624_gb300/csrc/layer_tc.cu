@@ -34,6 +34,7 @@
 #include <mutex>
 #include <vector>
 
+#include "layer_ring.h"
 #include "layer_tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -45,11 +46,6 @@ namespace lt {
 
 using namespace tc;
 
-// Pipeline stages of one K block (A: 128 x 64, B: Np x 64); the gathering form has one per gather warp.
-constexpr int NS_MAX = 5, NS_GATHER = 4;
-__host__ __device__ constexpr int lt_stages(bool ta, int Np) {
-  return Np > 128 ? 3 : !ta ? NS_GATHER : Np <= 64 ? 5 : 4;
-}
 // An epilogue warp's list of special elements (32 lanes x at most 16 columns, or 64 columns that hold
 // fewer) and its lanes' rows.
 constexpr int CAP = 512;
@@ -346,8 +342,8 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
     }
   } else if (!TA && warp >= RL::GATHER0) {
     // ------------------------------------------------------------ operand (A) gather
-    // warp g takes the K blocks g, g + 4, ... of the (tile, K block) order, each into the ring slot
-    // its number falls on; it writes chunks CPW part .. CPW part + CPW - 1 (of 8 per row)
+    // warp g takes the K blocks g, g + NS, ... of the (tile, K block) order, all of them in ring slot g
+    // (lt_gather_warp); it writes chunks CPW part .. CPW part + CPW - 1 (of 8 per row)
     const int g = (warp - RL::GATHER0) % NS_GATHER, part = 0;
     constexpr int CPW = 8;
     constexpr int GW = RL::GW > 0 ? RL::GW : 1;
@@ -372,16 +368,15 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         srow[q] = ps.src + r * ps.src_stride + (mv ? ((long long)y0[q] * ps.Ws + x0[q]) * ps.Cps : 0);
       }
       for (int kb = 0; kb < nkb; ++kb, ++seq) {
-        if ((int)(seq % NS_GATHER) != g) continue;
-        const uint32_t slot = seq % (uint32_t)NS;
+        if (lt_gather_warp((int)seq, NS) != g) continue;
         int okw = 1;
-        if (lane == 0) okw = lt_wait(&empty[slot], ((seq / (uint32_t)NS) & 1) ^ 1, abort, cx.status) ? 1 : 0;
+        if (lane == 0) okw = lt_wait(&empty[g], ((seq / (uint32_t)NS) & 1) ^ 1, abort, cx.status) ? 1 : 0;
         okw = __shfl_sync(0xffffffffu, okw, 0);
         if (!okw) {
           ok = false;
           break;
         }
-        uint8_t* stage = sA + slot * 16384;
+        uint8_t* stage = sA + g * 16384;
         // 4 chunks (of 4 rows each) in flight at a time: 16 loads of 16 bytes per lane
 #pragma unroll
         for (int c0 = 0; c0 < CPW; c0 += 4) {
@@ -409,7 +404,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         }
         fence_proxy_async();   // generic-proxy stores of the stage, before the MMA reads it
         __syncwarp();
-        if (lane == 0) mbar_arrive(&full[slot]);
+        if (lane == 0) mbar_arrive(&full[g]);
       }
     }
   } else {
@@ -985,10 +980,16 @@ __global__ void k_lt_ntab(int P, long long H, long long hoff, int C, int HW, int
   mtab[o / 8] = (uint16_t)(act | uns << 8);
 }
 
-inline int lt_smem(bool ta, int Np) {
+constexpr int lt_smem(bool ta, int Np) {
   return 1024 + lt_stages(ta, Np) * (16384 + Np * 128) + 256 + (MAX_KP / 8) * (int)sizeof(int2) +
          MAX_NP * (int)sizeof(float) + (ta ? LtRoles<true>::EPI : LtRoles<false>::EPI) * (int)sizeof(LtList);
 }
+constexpr int lt_smem_max(bool ta) {
+  int most = 0;
+  for (int np = 16; np <= MAX_NP; np += 16) most = lt_smem(ta, np) > most ? lt_smem(ta, np) : most;
+  return most;
+}
+static_assert(lt_smem_max(false) <= 232448 && lt_smem_max(true) <= 232448, "shared memory plan exceeds 227 KB per CTA");
 
 }  // namespace lt
 
@@ -1383,11 +1384,7 @@ int prepare(bcrown_net* net, LtNet* t) {
     BC_CHECK(upload(t, wd.data(), wd.size() * sizeof(int), &d));
     t->width = reinterpret_cast<int*>(d);
   }
-  int smem_g = 0, smem_t = 0;
-  for (int np = 16; np <= MAX_NP; np += 16) {
-    smem_g = std::max(smem_g, lt_smem(false, np));
-    smem_t = std::max(smem_t, lt_smem(true, np));
-  }
+  const int smem_g = lt_smem_max(false), smem_t = lt_smem_max(true);
   BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_RELAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
   BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_CONCRETIZE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
   BC_CUDA(cudaFuncSetAttribute(k_lt<EPI_FWD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_g));
