@@ -50,7 +50,7 @@ using namespace tc;
 // fewer) and its lanes' rows.
 constexpr int CAP = 512;
 struct LtList {
-  int4 row[32][2];           // {alpha base lo, hi, neuron table offset lo, hi}, {output offset lo, hi, chord base, -}
+  int4 row[32][2];           // {alpha base lo, hi, neuron table offset lo, hi}, {output offset lo, hi, chord base lo, hi}
   float val[CAP];
   uint16_t ent[CAP];         // column | lane << 8 | split << 15
   // the splits of the warp's row in this layer, where its positions lie in one row of a convolution
@@ -537,9 +537,9 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         const int lim = ps.npos ? ps.N : ps.Cpo;                  // elements that exist in the map
         __syncwarp();
         {
-          const long long dofs = (long long)rl * ps.dst_stride + nhwc0;
+          const long long dofs = (long long)rl * ps.dst_stride + nhwc0, cofs = (long long)prop * cx.H;
           wl.row[lane][0] = make_int4(ri.x, ri.y, (int)(uint32_t)tofs, (int)(tofs >> 32));
-          wl.row[lane][1] = make_int4((int)(uint32_t)dofs, (int)(dofs >> 32), prop * cx.H, 0);
+          wl.row[lane][1] = make_int4((int)(uint32_t)dofs, (int)(dofs >> 32), (int)(uint32_t)cofs, (int)(cofs >> 32));
         }
         const bool mvec = ((ps.Cpo | ps.N) & 63) == 0 && !(nlo & 63);   // 64 columns' masks in one 16-byte load
         bool waited = false;
@@ -694,7 +694,9 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
                 ch[q] = make_float2(0.f, 0.f);
-                if (rk[q] >= 0) ch[q] = cx.chord[wl.row[wl.ent[first + lane + 32 * q] >> 8][1].z + rk[q]];
+                if (rk[q] < 0) continue;
+                const int4 x = wl.row[wl.ent[first + lane + 32 * q] >> 8][1];
+                ch[q] = cx.chord[(((long long)x.w << 32) | (uint32_t)x.z) + rk[q]];
               }
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
