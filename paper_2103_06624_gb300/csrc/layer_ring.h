@@ -18,12 +18,12 @@ LT_HD constexpr int lt_stages(bool ta, int Np) {
   return ta ? (Np > 128 ? 3 : Np <= 64 ? 5 : 4) : (Np > 208 ? 3 : NS_GATHER);
 }
 
-// K block seq of a CTA's (tile, K block) order lies in stage seq % ns, and one gather warp owns each
+// K block s of a CTA's (tile, K block) order lies in stage s % stages, and one gather warp owns each
 // stage; with fewer stages than warps the others gather nothing.  A barrier's phase is told by one
 // parity bit, so a warp may only wait for a stage whose previous block it has written itself: a warp
 // that took the blocks of several stages in turn could come to one two rounds ahead, where the
 // wait's parity is that of a round that has passed.
-LT_HD constexpr int lt_gather_warp(int seq, int ns) { return seq % ns; }
+LT_HD constexpr int lt_gather_warp(int stage) { return stage; }
 
 }  // namespace lt
 }  // namespace bcrown

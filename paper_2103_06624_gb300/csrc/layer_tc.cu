@@ -351,7 +351,8 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
     if (!linear)
       for (int k = threadIdx.x - RL::GATHER0 * 32; k < ps.kchunks; k += GW * 32) stab[k] = ps.tab[k];
     asm volatile("bar.sync 2, %0;" ::"n"(GW * 32) : "memory");
-    uint32_t seq = 0;
+    int next = 0;       // stage of the next block, and the parity of its empty barrier
+    uint32_t par = 1;
     bool ok = true;
     for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
       const __nv_bfloat16* srow[4];
@@ -367,10 +368,13 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         x0[q] = j * ps.ms + ps.cx;
         srow[q] = ps.src + r * ps.src_stride + (mv ? ((long long)y0[q] * ps.Ws + x0[q]) * ps.Cps : 0);
       }
-      for (int kb = 0; kb < nkb; ++kb, ++seq) {
-        if (lt_gather_warp((int)seq, NS) != g) continue;
+      for (int kb = 0; kb < nkb; ++kb) {
+        const bool mine = lt_gather_warp(next) == g;
+        const uint32_t ph = par;
+        if (++next == NS) next = 0, par ^= 1;
+        if (!mine) continue;
         int okw = 1;
-        if (lane == 0) okw = lt_wait(&empty[g], ((seq / (uint32_t)NS) & 1) ^ 1, abort, cx.status) ? 1 : 0;
+        if (lane == 0) okw = lt_wait(&empty[g], ph, abort, cx.status) ? 1 : 0;
         okw = __shfl_sync(0xffffffffu, okw, 0);
         if (!okw) {
           ok = false;

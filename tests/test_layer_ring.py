@@ -32,7 +32,7 @@ int main() {
   for (int np = 16; np <= 256; np += 16) {
     const int ns = lt_stages(false, np);
     std::printf("%%d %%d %%d", np, ns, NS_GATHER);
-    for (int s = 0; s < %d; ++s) std::printf(" %%d", lt_gather_warp(s, ns));
+    for (int s = 0; s < %d; ++s) std::printf(" %%d", lt_gather_warp(s %% ns));
     std::printf("\\n");
   }
 }
