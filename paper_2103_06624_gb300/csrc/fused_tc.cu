@@ -148,6 +148,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, SM* sm, 
     }
   }
 }
+// The TMA and the MMA warp (one warp each) wait with all lanes.
+template <class SM>
+__device__ __forceinline__ bool mbar_wait_all(uint64_t* b, uint32_t parity, SM* sm, int* status) {
+  return mbar_wait_together(b, parity, [&] { return *(volatile int*)&sm->abort_flag != 0; },
+                            [&] {
+                              atomicCAS(status, 0, BCROWN_ERR_TIMEOUT);
+                              *(volatile int*)&sm->abort_flag = 1;
+                            });
+}
 // Wait by a whole warp: one lane polls the barrier (512 polling threads would flood the
 // shared-memory pipe every other warp needs), then the warp reconverges.
 template <class SM>
@@ -306,7 +315,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
     bool ok = true;
     // K pair kp of M chunk mc of a layer's weights
     auto put = [&](const CUtensorMap* map, uint32_t bytes, int mc, int kp, int nkb) -> bool {
-      if (!mbar_wait(&sm->w_empty[st], ph, sm, a.status)) return false;
+      if (!mbar_wait_all(&sm->w_empty[st], ph, sm, a.status)) return false;
       if (lane == 0) {
         const bool two = 2 * kp + 1 < nkb;
         mbar_expect_tx(&sm->w_full[st], two ? 2 * bytes : bytes);
@@ -362,8 +371,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
     bool ok = true;
     // one K pair (or its first block) of a chunk: weights of stage st, activations of slot s
     auto pair = [&](uint32_t dt, uint32_t s, bool first, bool two) -> bool {
-      if (!mbar_wait(&sm->w_full[st], wph, sm, a.status)) return false;
-      __syncwarp();
+      if (!mbar_wait_all(&sm->w_full[st], wph, sm, a.status)) return false;
       tc_fence_after();
       umma_kpair<(STAGE_BYTES >> 4), (SLOT_BYTES >> 4)>(dt, w0 + st * WSTEP, a0 + s * ASTEP, idesc, first ? 0u : 1u,
                                                         two ? 1u : 0u, b_wempty + 8 * st);
@@ -373,14 +381,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
     // chunk mc of nmc of a contraction with a resident operand (slots half, half + 1) of nkb K blocks
     auto chunk = [&](int mc, int nmc, int nkb) -> bool {
       const bool last = mc == nmc - 1;
-      if (!mbar_wait(&sm->acc_empty[buf], cph, sm, a.status)) return false;
+      if (!mbar_wait_all(&sm->acc_empty[buf], cph, sm, a.status)) return false;
       tc_fence_after();
       const uint32_t dt = tmem + buf * TR;
-      if (mc == 0 && !mbar_wait(&sm->act_full[half], (fpar >> half) & 1, sm, a.status)) return false;
+      if (mc == 0 && !mbar_wait_all(&sm->act_full[half], (fpar >> half) & 1, sm, a.status)) return false;
       if (!pair(dt, half, true, nkb > 1)) return false;
       if (last) umma_commit_warp(b_aempty + 8 * half);
       if (nkb > 2) {
-        if (mc == 0 && !mbar_wait(&sm->act_full[half + 1], (fpar >> (half + 1)) & 1, sm, a.status)) return false;
+        if (mc == 0 && !mbar_wait_all(&sm->act_full[half + 1], (fpar >> (half + 1)) & 1, sm, a.status)) return false;
         if (!pair(dt, half + 1, false, nkb > 3)) return false;
         if (last) umma_commit_warp(b_aempty + 8 * (half + 1));
       }
@@ -408,7 +416,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
         if (MODE == 0 || m < XLAG) continue;
         const int e = m - XLAG;
         const uint32_t s = xhalf + (uint32_t)(e & 1);
-        if (!(ok = mbar_wait(&sm->act_full[s], (fpar >> s) & 1, sm, a.status))) break;
+        if (!(ok = mbar_wait_all(&sm->act_full[s], (fpar >> s) & 1, sm, a.status))) break;
         for (int mc = 0; mc < nmc1 && ok; ++mc)
           ok = pair(tmem + (uint32_t)((NACC + mc) * TR), s, e == 0, 2 * e + 1 < nkbx);
         if (!ok) break;
@@ -427,7 +435,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(const __grid_constant__ M
     }
     __syncwarp();
     umma_commit_warp(su32(&sm->done));
-    mbar_wait(&sm->done, 0, sm, a.status);
+    mbar_wait_all(&sm->done, 0, sm, a.status);
   } else {
     // ---------------------------------------------------------------- epilogue (warps 0..15)
     const int q = warp & 3;          // TMEM lane quadrant: neurons 32q..32q+31 of an M chunk

@@ -155,6 +155,15 @@ __device__ __forceinline__ bool lt_wait(uint64_t* b, uint32_t parity, volatile i
   }
 }
 
+// The TMA and the MMA warp wait with all lanes.
+__device__ __forceinline__ bool lt_wait_all(uint64_t* b, uint32_t parity, volatile int* abort, int* status) {
+  return mbar_wait_together(b, parity, [&] { return *abort != 0; },
+                            [&] {
+                              atomicCAS(status, 0, BCROWN_ERR_TIMEOUT);
+                              *abort = 1;
+                            });
+}
+
 __device__ __forceinline__ uint4 ldg_nc_v4(const void* p, bool pred) {
   uint4 v;
   asm volatile(
@@ -270,11 +279,10 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         }
       }
       for (int kb = 0; kb < nkb; ++kb, ++seq) {
-        if (!lt_wait(&empty[st], ph ^ 1, abort, cx.status)) {
+        if (!lt_wait_all(&empty[st], ph ^ 1, abort, cx.status)) {
           ok = false;
           break;
         }
-        __syncwarp();
         if (lane == 0) {
           mbar_expect_tx(&full[st], (TA ? 16384u : 0u) + (uint32_t)bbytes);
           if constexpr (TA) {
@@ -319,15 +327,14 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
     const uint32_t a0 = plain ? ((su32(sA) >> 4) & 0x3FFFu) | ((2048u >> 4) << 16) : sdesc_lo(su32(sA));
     const uint32_t b_empty = su32(empty), b_acc = su32(acc_full);
     for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-      if (!lt_wait(&acc_empty[buf], cph, abort, cx.status)) break;
+      if (!lt_wait_all(&acc_empty[buf], cph, abort, cx.status)) break;
       tc_fence_after();
       const uint32_t dt = tmem + buf * (uint32_t)Np;
       for (int kb = 0; kb < nkb; ++kb) {
-        if (!lt_wait(&full[st], wph, abort, cx.status)) {
+        if (!lt_wait_all(&full[st], wph, abort, cx.status)) {
           ok = false;
           break;
         }
-        __syncwarp();
         tc_fence_after();
         const uint32_t al = a0 + (uint32_t)st * (16384 >> 4), bl = b0 + (uint32_t)st * bstep;
         if (plain)

@@ -50,6 +50,34 @@ __device__ __forceinline__ bool mbar_try_sleep(uint64_t* b, uint32_t parity, uin
       : "memory");
   return ok != 0;
 }
+// Wait by a whole warp whose lanes all poll.  Their answers are combined, so that they leave the wait
+// together and take the same branch, also where the time (about 2 s) runs out for some of them only: what
+// follows elects a lane among all 32, or keeps the warp at one place of a ring, where a lane left
+// behind would wait for a parity that has passed.  The phase stays complete while the warp waits for it, so
+// a lane that has seen it sees it again.  aborted(): whether another warp gave up; give_up(): records it.
+__device__ __forceinline__ bool mbar_try_together(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "vote.sync.all.pred q, p, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(ok)
+      : "r"(su32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+template <class Aborted, class GiveUp>
+__device__ __forceinline__ bool mbar_wait_together(uint64_t* b, uint32_t parity, Aborted aborted, GiveUp give_up) {
+  if (mbar_try_together(b, parity)) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_sleep(b, parity, 20000u))) return true;
+    const bool late = clock64() - t0 > 4000000000LL;
+    if (__any_sync(0xffffffffu, late || aborted())) {
+      if (late) give_up();
+      return false;
+    }
+  }
+}
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
