@@ -6,8 +6,12 @@
 // Layer by layer the path is a launch or two per layer and pass, each of a few blocks: 16-32-32-4,
 // 192 rows, bound and gradient: 12 launches, 57 us, of which no kernel has 2 us of work.  Here a
 // warp takes the row (four rows a block) where no layer is wider than ROWS_WARP_WIDTH, else a block
-// of 256 threads; a thread owns every 32nd or 256th output of a contraction and runs its sum in the
-// order of the GEMM (one chain of FMAs over k), the weights' loads of 8 terms in flight.
+// of 256 threads; a thread owns every 32nd or 256th output of a contraction.  Bound by the latency of the
+// weights' loads, so 16 of them are in flight per thread (8 where the rows fill the chip).
+//
+// Every sum has the order that the layers' kernels give it (the GEMM's chain over k, the relaxation's
+// lanes, the concretisation's 256 threads), so a row's bits do not depend on the kernel, and with it
+// on the batch.
 #include <algorithm>
 #include <atomic>
 
@@ -33,7 +37,9 @@ struct RowsNet {
   const float *Wbar, *bbar;
 };
 
-__host__ __device__ constexpr int rows_floats(int H, int mw) { return 5 * H + 3 * mw; }
+// H and mw rounded up to a multiple of 4, so that Lam, h and z lie on 16-byte boundaries
+__host__ __device__ constexpr int rows_pad(int x) { return (x + 3) & ~3; }
+__host__ __device__ constexpr int rows_floats(int H, int mw) { return 5 * rows_pad(H) + 3 * rows_pad(mw); }
 
 template <int T>
 __device__ __forceinline__ void row_sync() {
@@ -41,43 +47,80 @@ __device__ __forceinline__ void row_sync() {
   else __syncwarp();
 }
 
-// y[n] = sum_k x[k] w[k][n] over n = t, t + T, ..: store(n, sum).  One chain over k, 8 loads in flight.
-// (16, or two batches of 16 in turn, or outputs side by side cost more in resident rows than they
-// gained: 37-300-260-5, 512 rows 53 us with this one, 75 to 95 with those.)
-template <int T, class F>
+// y[n] = sum_k x[k] w[k][n] over n = t, t + T, ..: store(n, sum).  One chain over k whatever V, the loads
+// of V terms in flight (x 16-byte aligned, read 4 terms at a time).
+template <int T, int V, class F>
 __device__ __forceinline__ void row_product(const float* x, const float* __restrict__ w, int K, int N, int t, F store) {
+#pragma unroll 1
   for (int n = t; n < N; n += T) {
     const float* wp = w + n;
     float acc = 0.f;
     int k = 0;
-    for (; k + 8 <= K; k += 8) {
-      float wv[8];
+#pragma unroll 1
+    for (; k + V <= K; k += V, wp += (size_t)V * N) {
+      float wv[V];
+      float4 xv[V / 4];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) wv[e] = __ldg(wp + (size_t)(k + e) * N);
+      for (int e = 0; e < V; ++e) wv[e] = __ldg(wp + (size_t)e * N);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc = fmaf(x[k + e], wv[e], acc);
+      for (int e = 0; e < V / 4; ++e) xv[e] = *reinterpret_cast<const float4*>(x + k + 4 * e);
+#pragma unroll
+      for (int e = 0; e < V / 4; ++e) {
+        acc = fmaf(xv[e].x, wv[4 * e], acc);
+        acc = fmaf(xv[e].y, wv[4 * e + 1], acc);
+        acc = fmaf(xv[e].z, wv[4 * e + 2], acc);
+        acc = fmaf(xv[e].w, wv[4 * e + 3], acc);
+      }
     }
-    for (; k < K; ++k) acc = fmaf(x[k], __ldg(wp + (size_t)k * N), acc);
+    if (k < K) {   // the rest, its loads together as well
+      float wv[V];
+#pragma unroll
+      for (int e = 0; e < V; ++e) wv[e] = k + e < K ? __ldg(wp + (size_t)e * N) : 0.f;
+#pragma unroll
+      for (int e = 0; e < V; ++e)
+        if (k + e < K) acc = fmaf(x[k + e], wv[e], acc);
+    }
     store(n, acc);
   }
 }
 
-template <int T>   // threads per row: 32 (ROWS_WARP_ROWS rows a block) or the block
-__global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T)
+// sum_j Lam[j] b[j] + a[j] lm[j] over the lanes of a warp, in the order of the layers' relaxation pass: 4
+// neighbours at a time per lane where d is a multiple of 4, else every 32nd, then the same exchange.
+// All operands lie in shared memory.
+__device__ __forceinline__ float row_bias_sum(const float* Lam, const float* b, const float* a, const float* lm, int d,
+                                              int lane) {
+  float acc = 0.f;
+  if ((d & 3) == 0) {
+    for (int j = 4 * lane; j < d; j += 128)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc = fmaf(Lam[j + v], b[j + v], fmaf(a[j + v], lm[j + v], acc));
+  } else {
+    for (int j = lane; j < d; j += 32) acc = fmaf(Lam[j], b[j], fmaf(a[j], lm[j], acc));
+  }
+  return warp_sum(acc);
+}
+
+// T: threads per row, 32 (ROWS_WARP_ROWS rows a block) or the block.  V: weights in flight a thread; the
+// block form with 16 asks for 3 blocks an SM only (62 registers, 4 fit): without that the compiler keeps to
+// the registers of more blocks and issues fewer of the loads together.
+template <int T, int V>
+__global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T, T > 32 && V == 16 ? 3 : 0)
     k_rows(const RowsNet net, RowsCtx c, const float* __restrict__ alpha, int64_t n_alpha,
            const float* __restrict__ beta, int64_t n_beta, float* __restrict__ lb, float* __restrict__ xstar,
            bool grad, float* __restrict__ dalpha, float* __restrict__ dbeta) {
   extern __shared__ __align__(16) float rows_smem[];
-  __shared__ float red[T / 32];
+  __shared__ float red[T > 32 ? 32 : 1];
+  __shared__ float part[T > 32 ? ROWS_MAXL + 1 : 1];   // the layers' bias sums
   __shared__ int tot[T / 32];
   const int t = threadIdx.x % T, lane = threadIdx.x & 31, w = t >> 5;
   const int rl = blockIdx.x * (T == 32 ? ROWS_WARP_ROWS : 1) + threadIdx.x / T;
   if (rl >= c.R) return;   // (whole rows: a warp, or no thread of the block)
   const int H = net.H, L = net.L;
   float* A = rows_smem + (size_t)(threadIdx.x / T) * rows_floats(H, net.mw);
-  float *D = A + H, *lm = D + H;
-  int *rank = reinterpret_cast<int*>(lm + H), *sp = rank + H;
-  float *Lam = reinterpret_cast<float*>(sp + H), *h = Lam + net.mw, *z = h + net.mw;
+  const int Hp = rows_pad(H), mwp = rows_pad(net.mw);
+  float *D = A + Hp, *lm = D + Hp;
+  int *rank = reinterpret_cast<int*>(lm + Hp), *sp = rank + Hp;
+  float *Lam = reinterpret_cast<float*>(sp + Hp), *h = Lam + mwp, *z = h + mwp;
 
   int b, k, p;
   const bool ok = row_prop(c, rl, &b, &k, &p);
@@ -136,12 +179,13 @@ __global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T)
 
   const long long abase = c.bt.alpha_off[b] + (long long)k * U;
   const long long bbase = (long long)off * c.K + (long long)k * cnt;
-  float acc = 0.f;
+  float c0 = ok ? net.bbar[k] : -INFINITY;
   for (int i = L - 1; i >= 1; --i) {
     const int d = net.d[i], o = net.hoff[i];
     for (int j = t; j < d; j += T) {
       const int n = o + j, s2 = sp[n];
       const float a = A[n];
+      z[j] = net.b[i][j];   // (z is free until the adjoint pass)
       float Dn = D[n], ln = lm[n], bs = 0.f;
       if (s2) {
         const long long bi = bbase + (s2 >> 1) - 1;
@@ -162,36 +206,40 @@ __global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T)
       }
       D[n] = Dn;
       lm[n] = ln;
-      const float lam = fmaf(a, Dn, bs);
-      Lam[j] = lam;
-      acc = fmaf(lam, net.b[i][j], fmaf(a, ln, acc));
+      Lam[j] = fmaf(a, Dn, bs);
     }
     row_sync<T>();
+    if (T == 32) {
+      c0 += row_bias_sum(Lam, z, A + o, lm + o, d, lane);
+    } else if (w == i % (T / 32)) {   // one warp of the block, another each layer
+      const float sum = row_bias_sum(Lam, z, A + o, lm + o, d, lane);
+      if (lane == 0) part[i] = sum;
+    }
     float* out = i > 1 ? A + net.hoff[i - 1] : h;
-    row_product<T>(Lam, net.W[i], d, net.d[i - 1], t, [&](int n, float v) { out[n] = v; });
+    row_product<T, V>(Lam, net.W[i], d, net.d[i - 1], t, [&](int n, float v) { out[n] = v + 0.f; });   // (-0 as the GEMM's 0)
     row_sync<T>();
   }
   // concretisation, and the corner that attains it
   const float *xl = c.x_lo + (size_t)p * net.d[0], *xh = c.x_hi + (size_t)p * net.d[0];
+  // (summed as by 256 threads: in the warp's form, whose inputs are at most 64, by two warps of them)
+  float s0 = 0.f, s1 = 0.f;
   for (int m = t; m < net.d[0]; m += T) {
-    const float a = h[m];
-    acc += fminf(a * xl[m], a * xh[m]);
+    const float a = h[m], v = fminf(a * xl[m], a * xh[m]);
+    if (T > 32 || m < 32) s0 += v;
+    else s1 += v;
     const float x = a >= 0.f ? xl[m] : xh[m];
     if (xstar) xstar[(size_t)(c.r0 + rl) * net.d[0] + m] = x;
     h[m] = x;
   }
-  acc = warp_sum(acc);
   if (T > 32) {
-    if (lane == 0) red[w] = acc;
-    __syncthreads();
-    acc = 0.f;
-#pragma unroll
-    for (int q = 0; q < T / 32; ++q) acc += red[q];
+    s0 = block_sum(s0, red);
+    for (int i = L - 1; i >= 1; --i) c0 += part[i];
   } else {
+    s0 = (warp_sum(s0) + 0.f) + (warp_sum(s1) + 0.f);
     __syncwarp();
   }
   if (t == 0) {
-    float out = (ok ? net.bbar[k] : -INFINITY) + acc;
+    float out = c0 + s0;
     if (!isfinite(out)) {
       flag(c.status, BCROWN_ERR_NONFINITE);
       out = -INFINITY;
@@ -201,7 +249,7 @@ __global__ void __launch_bounds__(T == 32 ? 32 * ROWS_WARP_ROWS : T)
   if (!grad) return;
   for (int i = 1; i < L; ++i) {
     const int o = net.hoff[i];
-    row_product<T>(h, net.Wt[i], net.d[i - 1], net.d[i], t, [&](int j, float v) {
+    row_product<T, V>(h, net.Wt[i], net.d[i - 1], net.d[i], t, [&](int j, float v) {
       const int n = o + j, s2 = sp[n];
       const float zj = v + net.b[i][j], a = A[n];
       if (rank[n] >= 0) {
@@ -234,11 +282,16 @@ int widest(const bcrown_net* net) {
 int rows_load(const bcrown_net* net) {
   if (!rows_supported(net, 0)) return BCROWN_OK;
   const int smem = rows_floats(ROWS_H, ROWS_D0) * 4;
-  for (cudaError_t e : {cudaFuncSetAttribute(k_rows<ROWS_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
-                        cudaFuncSetAttribute(k_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)})
+  for (cudaError_t e : {cudaFuncSetAttribute(k_rows<ROWS_BLOCK, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                        cudaFuncSetAttribute(k_rows<ROWS_BLOCK, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                        cudaFuncSetAttribute(k_rows<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)})
     if (e != cudaSuccess) return fail(BCROWN_ERR_CUDA, "row kernel: shared memory");
   return BCROWN_OK;
 }
+
+// Rows of the block form that are resident at once with 16 loads in flight (4 blocks on each of 152 SMs);
+// more go 8 at a time, in more blocks.
+constexpr int ROWS_DEEP = 608;
 
 // Which calls take it (times of calls, bound and gradient, this kernel / layer by layer).  The warp
 // form, always: a pass per layer over rows this short costs more than the whole chain (16-32-32-4:
@@ -247,8 +300,8 @@ int rows_load(const bcrown_net* net) {
 // tiles empty, up to 2^27 FMAs per pass: 37-300-260-5, 64 rows 43 / 103, 2,048 rows (1.8e8 FMAs)
 // 140 / 134; 64-128x3-10, 2,304 rows (0.9e8) 75 / 118, 9,216 (3.8e8) 257 / 191; 784-256x6-10, 72 rows
 // 107 / 252, 1,152 (6.1e8) 344 / 280.  Layers over 512 neurons stay with the GEMM: a thread's chains
-// follow one another there (100-1000-900-10, 9 rows 194 / 172).  A bound and a gradient of the same
-// batch take the same kernel.
+// follow one another there (100-1000-900-10, 9 rows 194 / 172).  A row's bits
+// are the same either way.
 constexpr long long ROWS_FMAS = 1LL << 27;
 
 static bool warp_form(const bcrown_net* net) { return widest(net) <= ROWS_WARP_WIDTH && net->H <= ROWS_H / 4; }
@@ -279,12 +332,13 @@ int rows_bound(const bcrown_net* net, const RowsCtx& c, const float* alpha, int6
     n.b[i] = net->ly[i - 1].b;
   }
   const int smem = rows_floats(n.H, n.mw) * 4;
-  if (warp_form(net))
-    k_rows<32><<<(c.R + ROWS_WARP_ROWS - 1) / ROWS_WARP_ROWS, 32 * ROWS_WARP_ROWS, ROWS_WARP_ROWS * smem, s>>>(
-        n, c, alpha, n_alpha, beta, n_beta, lb, xstar, grad, dalpha, dbeta);
-  else
-    k_rows<ROWS_BLOCK><<<c.R, ROWS_BLOCK, smem, s>>>(n, c, alpha, n_alpha, beta, n_beta, lb, xstar, grad, dalpha,
-                                                     dbeta);
+  auto go = [&](auto* kernel, int rows, int threads) {
+    kernel<<<(c.R + rows - 1) / rows, threads, rows * smem, s>>>(n, c, alpha, n_alpha, beta, n_beta, lb, xstar, grad,
+                                                                 dalpha, dbeta);
+  };
+  if (warp_form(net)) go(k_rows<32, 16>, ROWS_WARP_ROWS, 32 * ROWS_WARP_ROWS);
+  else if (c.R <= ROWS_DEEP) go(k_rows<ROWS_BLOCK, 16>, 1, ROWS_BLOCK);
+  else go(k_rows<ROWS_BLOCK, 8>, 1, ROWS_BLOCK);
   ++g_launches;
   return BCROWN_OK;
 }

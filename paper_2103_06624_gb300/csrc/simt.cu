@@ -427,9 +427,14 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
     // CERT: acc is a lower bound of sum_j Lambda_j b_j + A_j lambda_j (every operation rounded
     // down); e1, e2 are upper bounds (rounded up) of the error terms below.
     const size_t n0 = (size_t)p * c.tb.H + hoff;
-    // Rows whose neurons lie on 16-byte boundaries in every array: 4 consecutive neurons per lane
-    // (float4 A, bias, Lambda and, certified, error weights; uchar4 codes), 1024 or 128 a step of the
-    // row's warps; a group of stable, unsplit neurons needs no other load.
+    // A lane takes 4 consecutive neurons at a time (1024 or 128 a step of the row's warps) where the
+    // layer's width is a multiple of 4, else every 32nd or 256th neuron: the order of its sums depends on
+    // the width alone, so a row's bits depend neither on its property's place in the arrays nor on
+    // their alignment.
+    const bool quads = (d & 3) == 0;
+    // Rows whose neurons lie on 16-byte boundaries in every array: 16-byte accesses (float4 A, bias,
+    // Lambda and, certified, error weights; uchar4 codes); a group of stable, unsplit neurons needs no
+    // other load.
     const long long aend = abase + Up;
     const bool alpha_ok = abase >= 0 && aend <= n_alpha;   // the row's alpha block, checked once
     const uintptr_t mis = reinterpret_cast<uintptr_t>(a_row) | reinterpret_cast<uintptr_t>(lam_row) |
@@ -437,7 +442,7 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
                           (CERT ? reinterpret_cast<uintptr_t>(wm + n0) | reinterpret_cast<uintptr_t>(c.l + n0) |
                                       reinterpret_cast<uintptr_t>(c.u + n0)
                                 : 0);
-    const bool vec4 = ((d | (int)(n0 & 3)) & 3) == 0 && (mis & 15) == 0 && ((WPR > 1 && !CERT) || alpha_ok);
+    const bool vec4 = quads && (n0 & 3) == 0 && (mis & 15) == 0 && ((WPR > 1 && !CERT) || alpha_ok);
     if (vec4) {
       const uchar4* code4 = reinterpret_cast<const uchar4*>(c.tb.code + n0);
       const float* alpha_row = alpha_ok ? alpha + abase : nullptr;
@@ -511,7 +516,9 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
     // scanned per neuron (short for these rows).
     if (WPR == 1 && !vec4) {
   #pragma unroll 4
-      for (int j = sub * 32 + lane; j < d; j += 32 * WPR) {
+      for (int t = 0;; ++t) {
+        const int j = quads ? 4 * (lane + 32 * (t >> 2)) + (t & 3) : lane + 32 * t;
+        if (j >= d) break;
         const float a = a_row[j];
         const size_t n = (size_t)p * c.tb.H + hoff + j;
         int s = 0;
@@ -564,13 +571,14 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
     // RELAX_V neurons per lane per step, their loads issued in three rounds (A, code, bias; then
     // the unstable neurons' rank and chord; then alpha) instead of one dependent chain each
     constexpr int RELAX_V = 4;
-    for (int j0 = sub * 32 + lane; WPR > 1 && !vec4 && j0 < d; j0 += RELAX_V * 32 * WPR) {
+    const int jstep = quads ? 1 : 32 * WPR;
+    for (int j0 = (sub * 32 + lane) * (quads ? 4 : 1); WPR > 1 && !vec4 && j0 < d; j0 += RELAX_V * 32 * WPR) {
       float av[RELAX_V], bv[RELAX_V], sl[RELAX_V], ic[RELAX_V], al[RELAX_V];
       uint8_t cv[RELAX_V];
       int32_t rk[RELAX_V];
 #pragma unroll
       for (int v = 0; v < RELAX_V; ++v) {
-        const int j = j0 + v * 32 * WPR;
+        const int j = j0 + v * jstep;
         const bool in = j < d;
         av[v] = ld_f32(a_row + j, in);
         bv[v] = ld_f32(bias + j, in);
@@ -578,7 +586,7 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
       }
 #pragma unroll
       for (int v = 0; v < RELAX_V; ++v) {
-        const int j = j0 + v * 32 * WPR;
+        const int j = j0 + v * jstep;
         const bool un = cv[v] == CODE_UNSTABLE;
         rk[v] = ld_s32(c.tb.rank + n0 + j, un && av[v] >= 0.f);
         sl[v] = ld_f32(c.tb.slope + n0 + j, un && av[v] < 0.f);
@@ -595,7 +603,7 @@ __global__ void __launch_bounds__(32 * RELAX_WARPS) k_relax(RowsCtx c, int layer
       }
 #pragma unroll
       for (int v = 0; v < RELAX_V; ++v) {
-        const int j = j0 + v * 32 * WPR;
+        const int j = j0 + v * jstep;
         if (j >= d) break;
         const float a = av[v];
         const size_t n = n0 + j;
