@@ -272,8 +272,8 @@ static int chunk_simt(bcrown_net* net, const bcrown_domain* dom, const bcrown_ba
 }
 
 // Whether a call takes the one-launch row kernel (which needs no tables).
-static bool takes_rows(const bcrown_net* net, int precision, long long R) {
-  return precision == BCROWN_FP32 && rows_supported(net, R);
+static bool takes_rows(const bcrown_net* net, int precision, long long R, bool grad) {
+  return precision == BCROWN_FP32 && rows_supported(net, R, grad);
 }
 
 // tc_plan: group the batch's rows into property tiles first (false when an earlier call on the
@@ -293,7 +293,7 @@ static int run_bound(bcrown_net* net, const bcrown_domain* dom, const bcrown_bat
   // BF16 beyond the fused kernel (conv layers, wide fc layers): the contractions on the tensor
   // cores, the rest of the layer-by-layer path in FP32; planned when the plan has an im2col buffer
   const bool tc_layers = precision == BCROWN_BF16 && pl.col != nullptr;
-  if (takes_rows(net, precision, R)) {
+  if (takes_rows(net, precision, R, grad)) {
     ProfScope ps(net, BCROWN_PROF_FUSED, s);
     return rows_bound(net, ctx_of(net, dom, bt, pl, 0, R), alpha, bt->n_alpha, beta, bt->n_beta, lb, nullptr, grad,
                       dalpha, dbeta, s);
@@ -355,7 +355,7 @@ extern "C" int bcrown_bound(bcrown_net* net, const bcrown_domain* dom, const bcr
   size_t tcb = fused_bytes(net, precision, batch, dom->n_props, false);
   BC_CHECK(make_plan(net, dom->n_props, R, precision == BCROWN_CERTIFY, false, 0, 0, tcb, pl,
                      layer_tc_col(net, precision, R), layer_lt_bytes(net, precision, R, dom->n_props, batch->n_alpha, false)));
-  if (!takes_rows(net, precision, R)) build_tables(net, dom, pl, s);
+  if (!takes_rows(net, precision, R, false)) build_tables(net, dom, pl, s);
   if (precision == BCROWN_CERTIFY) build_wm(net, dom, pl, s);
   BC_CHECK(run_bound(net, dom, batch, pl, precision, false, alpha, beta, lb, nullptr, nullptr, s));
   BC_CUDA(cudaGetLastError());
@@ -379,7 +379,7 @@ extern "C" int bcrown_bound_grad(bcrown_net* net, const bcrown_domain* dom, cons
   size_t tcb = fused_bytes(net, precision, batch, dom->n_props, true);
   BC_CHECK(make_plan(net, dom->n_props, R, false, false, 0, 0, tcb, pl,
                      layer_tc_col(net, precision, R), layer_lt_bytes(net, precision, R, dom->n_props, batch->n_alpha, true)));
-  if (!takes_rows(net, precision, R)) build_tables(net, dom, pl, s);
+  if (!takes_rows(net, precision, R, true)) build_tables(net, dom, pl, s);
   BC_CHECK(run_bound(net, dom, batch, pl, precision, true, alpha, beta, lb, dalpha, dbeta, s));
   BC_CUDA(cudaGetLastError());
   return BCROWN_OK;
@@ -633,7 +633,7 @@ extern "C" int bcrown_bound_xstar(bcrown_net* net, const bcrown_domain* dom, con
   Plan pl;
   const int R = batch->B * net->K;
   BC_CHECK(make_plan(net, dom->n_props, R, false, false, 0, 0, 0, pl));
-  if (takes_rows(net, BCROWN_FP32, R)) {
+  if (takes_rows(net, BCROWN_FP32, R, false)) {
     ProfScope ps(net, BCROWN_PROF_FUSED, s);
     BC_CHECK(rows_bound(net, ctx_of(net, dom, batch, pl, 0, R), alpha, batch->n_alpha, beta, batch->n_beta, lb, xstar,
                         false, nullptr, nullptr, s));

@@ -280,7 +280,7 @@ int widest(const bcrown_net* net) {
 }  // namespace
 
 int rows_load(const bcrown_net* net) {
-  if (!rows_supported(net, 0)) return BCROWN_OK;
+  if (!rows_supported(net, 0, false) && !rows_supported(net, 0, true)) return BCROWN_OK;
   const int smem = rows_floats(ROWS_H, ROWS_D0) * 4;
   for (cudaError_t e : {cudaFuncSetAttribute(k_rows<ROWS_BLOCK, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                         cudaFuncSetAttribute(k_rows<ROWS_BLOCK, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
@@ -293,27 +293,42 @@ int rows_load(const bcrown_net* net) {
 // more go 8 at a time, in more blocks.
 constexpr int ROWS_DEEP = 608;
 
-// Which calls take it (times of calls, bound and gradient, this kernel / layer by layer).  The warp
-// form, always: a pass per layer over rows this short costs more than the whole chain (16-32-32-4:
-// 192 rows 30 us / 58, 3,072 33 / 70, 196,608 288 / 1,176; the first two are the host's time for a
-// call).  The block form reads the weights once per row, so it is for the rows that leave the GEMM's
-// tiles empty, up to 2^27 FMAs per pass: 37-300-260-5, 64 rows 43 / 103, 2,048 rows (1.8e8 FMAs)
-// 140 / 134; 64-128x3-10, 2,304 rows (0.9e8) 75 / 118, 9,216 (3.8e8) 257 / 191; 784-256x6-10, 72 rows
-// 107 / 252, 1,152 (6.1e8) 344 / 280.  Layers over 512 neurons stay with the GEMM: a thread's chains
-// follow one another there (100-1000-900-10, 9 rows 194 / 172).  A row's bits
-// are the same either way.
-constexpr long long ROWS_FMAS = 1LL << 27;
+// Which calls take it.  A row's bits are the same either way: the sums have the layers' order.
+// Times of calls, bound / bound and gradient, here and layer by layer (us; below 26 the host's time):
+//   16-32-32-4       192 rows 23 / 29, 40 / 57;  8,192 22 / 30, 59 / 102;  196,608 217 / 293, 618 / 1,337
+//   64x4-10          2,048 rows 24 / 35, 55 / 104;  196,608 698 / 1,249, 1,023 / 2,445
+//   64x9-10          8,192 rows 134 / 238, 157 / 344;  32,768 506 / 929, 396 / 958
+//   37-300-260-5     64 rows 24 / 36, 63 / 102;  1,024 40 / 76, 67 / 106;  1,400 64 / 117, 69 / 113
+//   784-256x6-10     8 rows 51 / 88, 125 / 246;  72 53 / 90, 120 / 240
+//   784-20-10        2,048 rows 23 / 61, 39 / 80;  8,192 67 / 195, 59 / 131
+//   2048-16-10       1,024 rows 24 / 67, 37 / 117;  2,048 31 / 130, 38 / 129
+//   2048-20-512-3    1,024 rows 61 / 162, 63 / 160;  2,048 91 / 244, 71 / 178
+//   1024-512-10      8 rows 41 / 75, 42 / 88;  2048-512-4  8 rows 73 / 138, 44 / 118
+// The warp form gains everywhere but where many hidden neurons leave few rows resident (64x9: 11 KB a
+// row), from 2^28 FMAs a pass on.  The block form reads the weights once per row: it is for the rows that
+// leave the GEMM's tiles empty, by their FMAs a pass (a layer's launches buy 2^26 of them) and the terms
+// of their chains; and for layers whose own chains (one after the other over the outputs that a thread
+// owns) are not longer than a layer's launches take, the bound's and the gradient's apart.
+constexpr long long ROWS_FMAS = 1LL << 27, ROWS_LAYER_FMAS = 1LL << 26, ROWS_WARP_FMAS = 1LL << 28;
+constexpr long long ROWS_TERMS = 3LL << 20;
+constexpr int ROWS_BOUND_TERMS = 1536, ROWS_GRAD_TERMS = 4096;
 
 static bool warp_form(const bcrown_net* net) { return widest(net) <= ROWS_WARP_WIDTH && net->H <= ROWS_H / 4; }
 
-bool rows_supported(const bcrown_net* net, long long R) {
+bool rows_supported(const bcrown_net* net, long long R, bool grad) {
   if (net->L > ROWS_MAXL || net->H > ROWS_H || net->d[0] > ROWS_D0) return false;
-  long long fma = 0;
+  long long fma = 0, back = 0, fwd = 0;   // FMAs of a pass; terms in a row's chains, one after the other
   for (int i = 1; i < net->L; ++i) {
-    if (net->ly[i - 1].kind != BCROWN_LAYER_FC || net->d[i] > ROWS_WIDTH) return false;
-    fma += (long long)net->d[i] * net->d[i - 1];
+    const int in = net->d[i - 1], out = net->d[i];
+    if (net->ly[i - 1].kind != BCROWN_LAYER_FC || out > ROWS_WIDTH) return false;
+    fma += (long long)out * in;
+    back += (long long)((in + ROWS_BLOCK - 1) / ROWS_BLOCK) * out;
+    fwd += (long long)((out + ROWS_BLOCK - 1) / ROWS_BLOCK) * in;
   }
-  return warp_form(net) || R * fma <= ROWS_FMAS;
+  const int n = net->L - 1;
+  if (warp_form(net)) return widest(net) <= 32 || net->H <= 256 || R * fma <= ROWS_WARP_FMAS;
+  return R * fma <= std::min(n * ROWS_LAYER_FMAS, ROWS_FMAS) && R * (back + fwd) <= ROWS_TERMS &&
+         (grad ? back + fwd <= (long long)n * ROWS_GRAD_TERMS : back <= (long long)n * ROWS_BOUND_TERMS);
 }
 
 int rows_bound(const bcrown_net* net, const RowsCtx& c, const float* alpha, int64_t n_alpha, const float* beta,

@@ -49,7 +49,7 @@ bool sconv_supported(const bcrown_net* net, int i);
 // rows.cu: the FP32 bound (and gradient, and minimising corner) of a small fully connected network in
 // one launch.  c.tb is not read: a row works out its property's table itself.
 int rows_load(const bcrown_net* net);   // shared-memory sizes (at bcrown_load_net)
-bool rows_supported(const bcrown_net* net, long long R);
+bool rows_supported(const bcrown_net* net, long long R, bool grad);
 int rows_bound(const bcrown_net* net, const RowsCtx& c, const float* alpha, int64_t n_alpha, const float* beta,
                int64_t n_beta, float* lb, float* xstar, bool grad, float* dalpha, float* dbeta, cudaStream_t s);
 

@@ -90,3 +90,28 @@ def test_rows_refuse_what_the_layers_refuse():
         assert bc.status(net) != 0
     lb = bc.bound(net, dom, bc.DeviceBatch.from_host(batch), _t(a), _t(b), bc.FP32)
     assert bc.status(net) == 0 and torch.isfinite(lb).all()
+
+
+@pytest.mark.parametrize("widths,B,bound,grad", [
+    ([2048, 512, 4], 4, False, False),    # long chains of one layer
+    ([2048, 256, 4], 4, False, True),     # long in the bound, made up for in the gradient
+    ([784, 20, 10], 4000, False, False),  # many rows of one layer
+    ([784, 20, 10], 1000, True, True),
+    ([64] * 9 + [10], 9000, False, False),   # a warp per row, few of them resident
+    ([64] * 9 + [10], 4, True, True),
+])
+def test_which_calls_take_the_one_launch(widths, B, bound, grad):
+    """Shapes that the layers' kernels do faster go to them, the bound and the gradient each by its own time."""
+    pb = wl.make_problem("rows", wl.mlp_layers(widths, 3), 1, 0.02, 2, 4)
+    onet = O.OracleNet(pb.layers, pb.C)
+    l, u = (x.astype(np.float32) for x in O.interval_bounds(onet, pb.x_lo, pb.x_hi))
+    batch = wl.random_batch(pb, [np.nonzero(O.unstable_mask(l[0], u[0]))[0]], B, 0, 2, 5)
+    a, b = (_t(x) for x in wl.random_alpha_beta(batch, 6, 1.0))
+    net, dom, db = bc.load_net(pb.layers, pb.C), bc.domain_from_host(pb.x_lo, pb.x_hi, l, u), bc.DeviceBatch.from_host(batch)
+    n0 = bc.kernel_launches()
+    lb = bc.bound(net, dom, db, a, b, bc.FP32)
+    n1 = bc.kernel_launches()
+    lb_g, _, _ = bc.bound_grad(net, dom, db, a, b, bc.FP32)
+    assert (n1 - n0 == 1, bc.kernel_launches() - n1 == 1) == (bound, grad)
+    assert torch.equal(lb, lb_g)
+    assert bc.status(net) == 0
