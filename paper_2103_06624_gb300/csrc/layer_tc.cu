@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         if (!okw) break;
         tc_fence_after();
       }
-      float acc = 0.f;
+      float acc = 0.f, acc_special = 0.f;
       const uint32_t tacc = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(buf * Np);
       __nv_bfloat16* dst_r = ps.dst ? ps.dst + (long long)rl * ps.dst_stride : nullptr;
       // the NHWC index of element n of this thread's position (fully connected over a map: n itself)
@@ -739,23 +739,14 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
                 }
               }
             }
-            if (MODE == EPI_RELAX && !warp_sum_ok) {
-              // each lane adds up its own row's terms, in order
-              __syncwarp();
-              unsigned long long mask = spec64 & range;
-              for (int i = off; mask; ++i) {
-                const int bit = __ffsll((long long)mask) - 1;
-                if (!((split64 >> bit) & 1ull)) acc += wl.val[i];
-                mask &= mask - 1;
-              }
-            }
             // split elements: rare, by their own lane
             unsigned long long todo = split64 & range;
             while (todo) {
               const int bit = __ffsll((long long)todo) - 1;
               todo &= todo - 1;
               const int n = nb0 + bit;
-              const float a = wl.val[off + __popcll(spec64 & range & ((1ull << bit) - 1ull))];
+              const int at = off + __popcll(spec64 & range & ((1ull << bit) - 1ull));
+              const float a = wl.val[at];
               const uint32_t ent = ps.ntab[tofs + n];
               const int code = (int)(ent & 3u), rank = (int)(ent >> 2);
               int s = 0, ts = 0;   // its sign and list position (the last entry, as everywhere)
@@ -774,7 +765,8 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
                 const float bn = sb_smem ? sbias[n] : ps.bnhwc[n];
                 const float bs = bi < cx.n_beta ? fmaxf(cx.beta[bi], 0.f) * (float)s : 0.f;
                 out = fmaf(a, s == -1 ? 1.f : 0.f, bs);
-                acc = fmaf(out, bn, acc);
+                if (warp_sum_ok) acc = fmaf(out, bn, acc);
+                else wl.val[at] = out * bn;
               } else {
                 if (bi < cx.n_beta) cx.dbeta[bi] = (float)s * a;
                 out = s == -1 ? a : 0.f;
@@ -782,6 +774,13 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
                 if (code == CODE_UNSTABLE) cx.dalpha[abase + rank] = 0.f;
               }
               if (dst_r) dst_r[nhwc0 + n] = __float2bfloat16_rn(out);
+            }
+            if (MODE == EPI_RELAX && !warp_sum_ok) {
+              // each lane adds up its own row's terms in column order, apart from the stable columns': how
+              // many columns a list holds depends on the rows that share the warp, the sums do not
+              __syncwarp();
+              const int end = off + __popcll(spec64 & range);
+              for (int i = off; i < end; ++i) acc_special += wl.val[i];
             }
           }
         }
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
           if (lane == 0 && mv)
             cx.cpart[(size_t)rl * cx.S + ps.slot0 + ((size_t)nt * ps.Pm + pp) / 32] = sw;
         } else if (mv) {
-          cx.cpart[(size_t)rl * cx.S + ps.slot0 + (size_t)nt * ps.Pm + pp] = acc;
+          cx.cpart[(size_t)rl * cx.S + ps.slot0 + (size_t)nt * ps.Pm + pp] = acc + acc_special;
         }
       }
     }

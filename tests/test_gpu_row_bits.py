@@ -1,4 +1,4 @@
-"""What a row's FP32 and certified bits depend on: its own data only (needs a GB300).  A small network's rows
+"""What a row's bits depend on: its own data only (needs a GB300).  A small network's rows
 have the same bits whichever kernel the batch's size takes and in bcrown_bound_static; a property's place
 among the others, which moves its tables off the 16-byte boundaries, changes nothing either."""
 import numpy as np
@@ -87,3 +87,31 @@ def test_a_row_does_not_depend_on_its_property_s_place(which, precision):
     assert bc.status(net) == 0
     for g in got[1:]:
         assert torch.equal(g, got[0])
+
+
+@pytest.mark.parametrize("which", ["mlp", "odd_maps"])
+def test_a_bf16_layer_path_row_does_not_depend_on_the_batch(which):
+    """Subdomains of a property with few unstable neurons, alone in a ragged tile and among those of one with
+    many: bound and gradient.  Both networks have warps that hold several rows."""
+    layers = {"mlp": lambda: wl.mlp_layers([37, 300, 260, 5], 11),
+              "odd_maps": lambda: wl.conv_layers((4, 7, 7), [(24, 3, 1, 1), (72, 3, 2, 1)], [40, 4], 3)}[which]()
+    pb = wl.make_problem("bits", layers, 2, 0.02, 3, 4)
+    pb.x_lo[1] -= 0.5
+    pb.x_hi[1] += 0.5
+    _, props, unst = oracle_setup(pb)
+    U = np.array([len(u) for u in unst])
+    assert U[0] < 0.25 * props["l"].shape[1] < 0.5 * U[1]
+    net = bc.load_net(pb.layers, pb.C)
+    bc.set_launch(net, bc.N.PATH_LAYER_EPI)
+    dom = bc.domain_from_host(props["x_lo"], props["x_hi"], props["l"], props["u"])
+    n = 7
+    big = wl.random_batch(pb, unst, 150, 1, 8, 5, props=np.where(np.arange(150) < n, 0, np.arange(150) % 2))
+    na, ns = int((U[big.prop_of[:n]] * pb.K).sum()), int(big.split_cnt[:n].sum())
+    small = wl.Batch(big.prop_of[:n], big.split_off[:n], big.split_cnt[:n], big.split_layer[:ns], big.split_idx[:ns],
+                     big.split_sign[:ns], big.alpha_off[:n], na, ns * pb.K)
+    a, b = (_t(x) for x in wl.random_alpha_beta(big, 6, 1.0))
+    got = [bc.bound_grad(net, dom, bc.DeviceBatch.from_host(x), y, z, bc.BF16)
+           for x, y, z in ((small, a[:na], b[:ns * pb.K]), (big, a, b))]
+    assert bc.status(net) == 0
+    for s, l in zip(*got):
+        assert torch.equal(s, l[:s.numel()])
