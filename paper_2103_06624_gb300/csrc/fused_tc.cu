@@ -1130,9 +1130,8 @@ bool tc_supported(const bcrown_net* net) {
     words += (net->d[i] + 31) / 32;
   }
   if (words > MAX_MASK_WORDS || net->H > MAX_H) return false;
-  // the forward contraction of layer 1 streams d0 in K blocks: its M chunks must fit the
-  // accumulator ring (hidden widths <= 256 give at most 2)
-  if ((net->d[1] + MCH - 1) / MCH > NACC) return false;
+  // the forward contraction of layer 1 streams d0 in K blocks into accumulators of its own, one per M chunk
+  static_assert(MAX_HIDDEN <= NFACC * MCH, "forward layer 1 needs an accumulator per M chunk");
   int dev = 0, major = 0, minor = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
