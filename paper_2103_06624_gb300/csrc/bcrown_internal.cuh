@@ -154,7 +154,8 @@ struct ProfScope {
   ~ProfScope();
 };
 
-// n / d for n < 2^31 by multiplication.
+// n / d for n < 2^31 by multiplication with a rounded-up reciprocal (Granlund and Montgomery, Division by
+// Invariant Integers using Multiplication, PLDI 1994).
 struct FastDiv {
   uint32_t d, mul, sh;
   __host__ void set(uint32_t v) {

@@ -100,19 +100,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-template <int MODE>  // 0 nearest, 1 toward -inf, 2 toward +inf
-__device__ __forceinline__ double dadd(double a, double b) {
-  if (MODE == 1) return __dadd_rd(a, b);
-  if (MODE == 2) return __dadd_ru(a, b);
-  return a + b;
-}
-
-template <int MODE>
-__device__ __forceinline__ double warp_dsum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = dadd<MODE>(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // FP32 sums with a rounding direction: MODE 0 nearest, 1 down (toward -inf), 2 up.  Directed
 // rounding at every step makes the result a lower (1) or upper (2) bound of the exact sum.
 template <int MODE>
@@ -147,21 +134,6 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
   int nw = (blockDim.x + 31) >> 5;
   float s = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.f;
   if (w == 0) s = warp_sum(s);
-  if (threadIdx.x == 0) sh[0] = s;
-  __syncthreads();
-  return sh[0];
-}
-
-template <int MODE>
-__device__ __forceinline__ double block_dsum(double v, double* sh) {
-  v = warp_dsum<MODE>(v);
-  int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
-  __syncthreads();
-  if (ln == 0) sh[w] = v;
-  __syncthreads();
-  int nw = (blockDim.x + 31) >> 5;
-  double s = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-  if (w == 0) s = warp_dsum<MODE>(s);
   if (threadIdx.x == 0) sh[0] = s;
   __syncthreads();
   return sh[0];

@@ -90,12 +90,10 @@ struct Pass {
   // output position of (row, pp): (oa + os * i) * Wo + ob + os * j; npos: position from n
   int oa, ob, os, Wo, npos;
   int Co, HWo, Cpo;          // output map: channels, positions, padded channels
-  FastDiv dPm, dnJ, dntn, dHWo, dCpo;   // (set at the launch)
+  FastDiv dPm, dnJ, dntn, dHWo;   // (set at the launch)
   __nv_bfloat16* dst;        // NHWC BF16 output (null: none)
   long long dst_stride;
   int layer;                 // hidden layer of the epilogue (0: the input)
-  long long hoff;            // its first global hidden index
-  const float* bias;         // its bias, expanded per neuron (channel-major)
   const float* bnhwc;        // its bias in NHWC order (padded channels 0)
   const uint32_t* ntab;      // its neurons in NHWC order, property 0 (stride Ctx::NH per property):
                              // code (0 inactive, 1 active, 2 unstable) | rank among the unstable << 2
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
     const uint32_t idesc = idesc_bf16(Np);
     const uint32_t b0 = sdesc_lo(su32(sB)), bstep = (uint32_t)bbytes >> 4;
     const bool plain = TA && ps.ta == 8;   // A without swizzle: core matrices 128 B apart along M, 2 KB along K
-    const uint32_t a0 = plain ? ((su32(sA) >> 4) & 0x3FFFu) | ((2048u >> 4) << 16) : sdesc_lo(su32(sA));
+    const uint32_t a0 = plain ? sdesc_plain_lo(su32(sA), 2048) : sdesc_lo(su32(sA));
     const uint32_t b_empty = su32(empty), b_acc = su32(acc_full);
     for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
       if (!lt_wait_all(&acc_empty[buf], cph, abort, cx.status)) break;
@@ -350,9 +348,8 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
   } else if (!TA && warp >= RL::GATHER0) {
     // ------------------------------------------------------------ operand (A) gather
     // warp g takes the K blocks g, g + NS, ... of the (tile, K block) order, all of them in ring slot g
-    // (lt_gather_warp); it writes chunks CPW part .. CPW part + CPW - 1 (of 8 per row)
-    const int g = (warp - RL::GATHER0) % NS_GATHER, part = 0;
-    constexpr int CPW = 8;
+    // (lt_gather_warp); a block is 8 chunks of 16 bytes per row
+    const int g = warp - RL::GATHER0;
     constexpr int GW = RL::GW > 0 ? RL::GW : 1;
     const bool linear = ps.tab == nullptr;
     if (!linear)
@@ -390,11 +387,11 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
         uint8_t* stage = sA + g * 16384;
         // 4 chunks (of 4 rows each) in flight at a time: 16 loads of 16 bytes per lane
 #pragma unroll
-        for (int c0 = 0; c0 < CPW; c0 += 4) {
+        for (int c0 = 0; c0 < 8; c0 += 4) {
           uint4 v[4][4];
 #pragma unroll
           for (int cc = 0; cc < 4; ++cc) {
-            const int kc = kb * 8 + CPW * part + c0 + cc;
+            const int kc = kb * 8 + c0 + cc;
             const int2 t = kc < ps.kchunks ? (linear ? make_int2(8 * kc, 0) : stab[kc]) : make_int2(0, 0x8000);
             const int dy = (int)(short)(t.y & 0xffff), dx = t.y >> 16;
 #pragma unroll
@@ -405,7 +402,7 @@ __global__ void __launch_bounds__(LtRoles<TA>::THREADS, 1)
           }
 #pragma unroll
           for (int cc = 0; cc < 4; ++cc) {
-            const int c = CPW * part + c0 + cc;
+            const int c = c0 + cc;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const int m = lane + 32 * q;
@@ -1234,8 +1231,6 @@ int prepare(bcrown_net* net, LtNet* t) {
           q.HWo = mo.HW();
           q.Cpo = mo.Cp;
           q.layer = i - 1;
-          q.hoff = i >= 2 ? net->hoff[i - 2] : 0;
-          q.bias = i >= 2 ? net->ly[i - 2].b : nullptr;
           q.bnhwc = i >= 2 ? t->bnhwc[i - 1] : nullptr;
           std::vector<int2> tab((size_t)kph / 8, kNoChunk);
           for (int dy = 0; dy < py.nk; ++dy)
@@ -1299,8 +1294,6 @@ int prepare(bcrown_net* net, LtNet* t) {
       q.HWo = mi.HW();
       q.Cpo = mi.Cp;
       q.layer = i;
-      q.hoff = net->hoff[i - 1];
-      q.bias = l.b;
       q.bnhwc = t->bnhwc[i];
       q.slot0 = 0;
       BC_CHECK(finish_pass(P.fwd, tab));
@@ -1343,8 +1336,6 @@ int prepare(bcrown_net* net, LtNet* t) {
       q.HWo = mo.HW();
       q.Cpo = mo.Cp;
       q.layer = i - 1;
-      q.hoff = i >= 2 ? net->hoff[i - 2] : 0;
-      q.bias = i >= 2 ? net->ly[i - 2].b : nullptr;
       q.bnhwc = i >= 2 ? t->bnhwc[i - 1] : nullptr;
       q.kchunks = mi.Cp / 8;   // K chunks past the layer's padded width read as zero
       q.tab = nullptr;
@@ -1380,8 +1371,6 @@ int prepare(bcrown_net* net, LtNet* t) {
       f.Cpo = mi.Cp;
       f.Wo = 1;
       f.layer = i;
-      f.hoff = net->hoff[i - 1];
-      f.bias = l.b;
       f.bnhwc = t->bnhwc[i];
       f.slot0 = 0;
       void* df = nullptr;
@@ -1417,7 +1406,6 @@ int launch_pass(bcrown_net* net, const CUtensorMap& mB, Pass q, int mode, const 
   q.dnJ.set(q.nJ);
   q.dntn.set(q.ntn);
   q.dHWo.set(q.HWo);
-  q.dCpo.set(q.Cpo);
   const long long ntiles = (q.M + 127) / 128 * q.ntn;
   const int grid = (int)std::min<long long>(ntiles, sms);
   const int smem = lt_smem(q.ta != 0, q.Np);

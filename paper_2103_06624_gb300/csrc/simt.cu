@@ -172,7 +172,7 @@ __device__ __forceinline__ float hmax_hidden(float uv) { return fmaxf(uv, 0.f); 
 // the grouping.  576 terms x 32,768 neurons: 65 us
 // a neuron and a term at a time, 23 now.
 struct AbswDiv {
-  FastDiv hw, ow, kk, k, groups;
+  FastDiv ow, kk, k, groups;
 };
 constexpr int ABSW_G = 4;
 __global__ void __launch_bounds__(256) k_absw_m(LayerGeom g, AbswDiv dv, const float* __restrict__ W, int P, int H,

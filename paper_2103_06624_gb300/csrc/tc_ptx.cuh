@@ -171,35 +171,17 @@ __device__ __forceinline__ void umma_kblock_warp(uint32_t dtmem, uint32_t alo, u
 #undef BC_UMMA1
 }
 constexpr uint32_t SDESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);         // sdesc's high word
-__host__ __device__ constexpr uint32_t SDESC_PLAIN_HI(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }   // sdesc_plain's
+// High and low word of a K-major descriptor without swizzle: 8-row x 16-byte core matrices of 128 contiguous
+// bytes, `sbo` bytes apart along M and `lbo` bytes apart along K.
+__host__ __device__ constexpr uint32_t SDESC_PLAIN_HI(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+__device__ __forceinline__ uint32_t sdesc_plain_lo(uint32_t saddr, uint32_t lbo) {
+  return ((saddr >> 4) & 0x3FFFu) | ((lbo >> 4) << 16);
+}
 // A commit by one lane of a converged warp.
 __device__ __forceinline__ void umma_commit_warp(uint32_t bar) {
   asm volatile(
       "{\n\t.reg .pred l;\n\t.reg .b32 d;\n\telect.sync d|l, 0xffffffff;\n\t"
       "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
-      : "memory");
-}
-// Shared-memory descriptor, K-major, no swizzle: 8-row x 16-byte core matrices stored as 128
-// contiguous bytes, `sbo` bytes apart along M and `lbo` bytes apart along K.
-__device__ __forceinline__ uint64_t sdesc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;                 // descriptor version; layout type 0 (no swizzle)
-  return d;
-}
-// As umma_kblock, with the A descriptor advanced by `astep` (16-byte units) per K step of 16.
-__device__ __forceinline__ void umma_kblock_astep(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                                  uint32_t acc, uint32_t astep) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, q;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, q;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, q;\n\t}" ::"r"(dtmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "l"(ad + astep), "l"(bd + 2), "l"(ad + 2 * astep), "l"(bd + 4),
-      "l"(ad + 3 * astep), "l"(bd + 6)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
