@@ -23,6 +23,9 @@
  *    which is sound, and sets BCROWN_ERR_NONFINITE; the other rows are written.
  *  - Calls on one net share the net's device workspace, so calls on the same
  *    net issued to different streams must not overlap.
+ *  - A row's bound, gradient and minimiser depend on the row alone, bit for bit: not on the
+ *    other rows of the batch, their number, or the place of its property in the domain.
+ *    (BF16: at one launch configuration, see bcrown_set_launch.)
  *
  * Index conventions (paper notation): layers i = 1..L are the linear layers;
  * hidden layers are i = 1..L-1 with d_i neurons (for a convolution, flattened
@@ -265,7 +268,8 @@ enum {
   BCROWN_PROF_CONCRETIZE = 2, /* concretisation over the box */
   BCROWN_PROF_ADJOINT = 3,    /* adjoint epilogue (gradients) */
   BCROWN_PROF_ADAM = 4,       /* projected Adam */
-  BCROWN_PROF_FUSED = 5,      /* fused tensor-core iteration kernel */
+  BCROWN_PROF_FUSED = 5,      /* fused tensor-core iteration kernel; the FP32 pass of small fully connected
+                                 networks in one launch */
   BCROWN_PROF_LAYER_GEMM = 6, /* tensor-core GEMMs of the BF16 layer paths (LAYER_EPI: with the fused epilogues) */
   BCROWN_PROF_NCLASS = 7
 };
@@ -400,8 +404,9 @@ int bcrown_autotune(bcrown_net* net, const bcrown_domain* dom, const bcrown_batc
  * It allocates nothing.  Its scratch (per-neuron tables and row-chunk buffers) is one
  * file-scope device array of BCROWN_STATIC_SCRATCH_BYTES bytes that every GPU loading the
  * library holds until the process exits.  The caller passes inputs and outputs exactly as for
- * bcrown_bound.  The first call on a device looks the array's device address up (once per
- * device, with that device current); make that first call before any stream capture begins.
+ * bcrown_bound and gets the same bits.  The first call on a device looks the array's device
+ * address up (once per device, with that device current); make that first call before any stream
+ * capture begins.
  * Problems whose per-property tables and a single row do not fit in the array are rejected
  * with BCROWN_ERR_ARG and a message naming the limit; larger batches are processed in row
  * chunks that fit.  Every call shares the one array and it keeps the last call's contents

@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(256) k_init_top(RowsCtx c, int dtop, const flo
 //   Lambda_j = A_j D_j + beta_j S_jj ;  c += Lambda_j b_j + A_j lambda_j
 // One warp per row (8 rows per block), or a block per row for wide layers: the row's splits of this
 // layer are compacted into shared memory by ballots, with one bit per neuron; a lane takes four
-// neighbouring neurons where the arrays are aligned.  Bound by memory and its latency.  2,997 rows,
+// neighbouring neurons where the width is a multiple of 4.  Bound by memory and its latency.  2,997 rows,
 // certified, of 8,192 / 4,096 / 512 neurons: 126 / 80 / 34 us a neuron per lane, 101 / 65 / 19 now;
 // 4,608 rows of 256, not certified, 16.6 / 12.
 // CERT: outward chord constants (from the tables), c summed rounded down, error terms rounded up.
