@@ -19,9 +19,9 @@
 // Activations are BF16 in NHWC order (channels innermost, padded to a multiple of 8).  The GEMM
 // operand -- rows = (subdomain row, output position), K = (tap, channel) -- comes by TMA where an M
 // tile is one box of the map, else it is gathered into shared memory in 16-byte pieces of 8 channels
-// by gather warps, one per stage of the ring (at most 4).  TMA streams the weights, one warp issues the MMAs into up to four TMEM
-// accumulators (two for 256-column tiles), and as many groups of 4 epilogue warps read them, each
-// group its own, so that their tiles' epilogues run at once.
+// by gather warps, one per stage of the ring (at most 4).  TMA streams the weights, one warp issues
+// the MMAs into up to four TMEM accumulators (two for 256-column tiles), and as many groups of 4
+// epilogue warps read them, each group its own, so that their tiles' epilogues run at once.
 // The bias sums of each row are written as partial sums (one slot per position block and column
 // group) and added in a fixed order at the end, so the result does not depend on scheduling.
 // A at the unstable neurons is stashed in BF16, laid out like alpha, for the adjoint pass; its
